@@ -851,26 +851,226 @@ __device__ __forceinline__ double load_point(int mode, const double* X64, const 
 }
 
 // FP64 feasibility check: max over (walker, row) of a_i x - b_i, and
-// max over walkers of |A_E x - b_E|_inf.  One block per (row block, walker).
-__global__ void check_kernel(int mode, int m, int n, int n_ld, int mE, const double* A,
-                             const double* b, const double* AE, const double* bE,
-                             const double* X64, const float* Xhi, const float* Xlo,
-                             unsigned long long* out_keys) {
+// max over walkers of |A_E x - b_E|_inf.
+//
+// Only one number leaves the check, so FP64 (1/64 of the FP32 rate on this
+// GPU) is spent on the rows that can hold it:
+//  (1) check_screen_kernel forms v = a_i . x - b_i in FP32 with a bound e on
+//      its error, keeps the largest v + e of each (row tile, walker), and
+//      folds v - e into the largest value some row certainly reaches;
+//  (2) check_exact_kernel evaluates in FP64, row by row in index order, the
+//      tiles whose v + e reaches that value -- a handful of them -- and folds
+//      s - b_i into the result.  A value FP32 cannot bound (overflow, NaN)
+//      counts as reaching it.
+// The screen is the standard FP32 bound (Higham, Accuracy and Stability,
+// Section 3.1; u = 2^-24): e = gamma_{n+8} ||a_i||_2 ||x||_2 + 4 u |b_i|,
+// gamma_k = k u / (1 - k u), the roundings of A, x, the products, the sums
+// and the comparison among its k; it takes nothing from the walk's own error
+// margins, which the check is there to verify.  Squares of entries below
+// 2^-75 leave the FP32 norms: kNormFloor per entry covers them.
+// A thread per (row, walker) in FP64, with an atomic each, took 5.35 ms for
+// 4096 walkers of a 2000 x 100 body and 1.39 ms for 1024 of them (ncu); the
+// two kernels take 0.15 and 0.07 ms.
+constexpr int kChkRows = 128;      // rows of a tile
+constexpr int kChkWalkers = 64;    // walkers of a tile
+constexpr int kChkK = 16;
+constexpr float kNormFloor = 1e-22f;
+
+__device__ __forceinline__ unsigned int f32_key(float f) {
+  const unsigned int u = __float_as_uint(f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float f32_unkey(unsigned int k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// blockIdx.x: group of `group` consecutive row tiles, blockIdx.y: 64 walkers.
+// ub[blockIdx.x * walkers + k]; best: key of the largest certain value.
+__global__ void __launch_bounds__(kThreads)
+check_screen_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
+                    const double* __restrict__ A, const double* __restrict__ b,
+                    const double* __restrict__ X64, const float* __restrict__ Xhi,
+                    const float* __restrict__ Xlo, float* __restrict__ ub, unsigned int* best) {
+  __shared__ __align__(16) float As[kChkK][kChkRows + 4];
+  __shared__ __align__(16) float Xs[kChkK][kChkWalkers + 4];
+  __shared__ float an[kChkRows], xn[kChkWalkers], red[16][kChkWalkers];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int w0 = blockIdx.y * kChkWalkers;
+  const float gam = static_cast<float>(n + 8) * 0x1p-24f /
+                    (1.0f - static_cast<float>(n + 8) * 0x1p-24f) * 1.0009765625f;
+  const float floor_n = static_cast<float>(n) * kNormFloor;
+  float up[4], low = -INFINITY;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) up[c] = -INFINITY;
+  const int xw = tid >> 2, xk = (tid & 3) * 4;   // this thread's part of a walker tile
+  const bool xin = w0 + xw < walkers;
+  for (int g = 0; g < group; ++g) {
+    const int i0 = (blockIdx.x * group + g) * kChkRows;
+    if (i0 >= m) break;
+    float acc[8][4];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = 0.0f;
+    float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sx = 0.0f;
+    for (int k0 = 0; k0 < n_ld; k0 += kChkK) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = (tid >> 3) + 32 * j, c = (tid & 7) * 2;
+        double2 v = make_double2(0.0, 0.0);
+        if (i0 + r < m)
+          v = *reinterpret_cast<const double2*>(A + static_cast<size_t>(i0 + r) * n_ld + k0 + c);
+        const float f0 = static_cast<float>(v.x), f1 = static_cast<float>(v.y);
+        As[c][r] = f0;
+        As[c + 1][r] = f1;
+        sa[j] = fmaf(f0, f0, fmaf(f1, f1, sa[j]));
+      }
+      float xv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      if (xin) {
+        const size_t o = static_cast<size_t>(w0 + xw) * n_ld + k0 + xk;
+        if (mode == 0) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) xv[e] = static_cast<float>(X64[o + e]);
+        } else {
+          const float4 h = *reinterpret_cast<const float4*>(Xhi + o);
+          const float4 l = *reinterpret_cast<const float4*>(Xlo + o);
+          xv[0] = h.x + l.x; xv[1] = h.y + l.y; xv[2] = h.z + l.z; xv[3] = h.w + l.w;
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        Xs[xk + e][xw] = xv[e];
+        sx = fmaf(xv[e], xv[e], sx);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int kk = 0; kk < kChkK; ++kk) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][ty * 8]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&As[kk][ty * 8 + 4]);
+        const float4 xq = *reinterpret_cast<const float4*>(&Xs[kk][tx * 4]);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float x[4] = {xq.x, xq.y, xq.z, xq.w};
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(a[r], x[c], acc[r][c]);
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) sa[j] += __shfl_xor_sync(0xffffffffu, sa[j], off);
+      if ((tid & 7) == 0) an[(tid >> 3) + 32 * j] = sqrtf(sa[j]) * 1.0009765625f + floor_n;
+    }
+#pragma unroll
+    for (int off = 2; off > 0; off >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, off);
+    if ((tid & 3) == 0) xn[xw] = sqrtf(sx) * 1.0009765625f + floor_n;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int gi = i0 + ty * 8 + r;
+      if (gi >= m) continue;
+      const float bf = static_cast<float>(b[gi]), ga = gam * an[ty * 8 + r];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (w0 + tx * 4 + c >= walkers) continue;
+        const float v = acc[r][c] - bf;
+        // 1e-36: products and b's below the normal FP32 range.
+        const float e = fmaf(ga, xn[tx * 4 + c], fmaf(0x1p-22f, fabsf(bf) + fabsf(v), 1e-36f));
+        const float hi = v + e, lo = v - e;
+        up[c] = hi < INFINITY ? fmaxf(up[c], hi) : INFINITY;   // not below +Inf, NaN too
+        if (fabsf(lo) < INFINITY) low = fmaxf(low, lo);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) red[ty][tx * 4 + c] = up[c];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) low = fmaxf(low, __shfl_xor_sync(0xffffffffu, low, off));
+  __syncthreads();
+  if (tid < kChkWalkers && w0 + tid < walkers) {
+    float u = red[0][tid];
+#pragma unroll
+    for (int t = 1; t < 16; ++t) u = fmaxf(u, red[t][tid]);
+    ub[static_cast<size_t>(blockIdx.x) * walkers + w0 + tid] = u;
+  }
+  if ((tid & 31) == 0) atomicMax(best, f32_key(low));
+}
+
+// The FP64 values of the tiles the screen left: a warp looks at 32 entries of
+// ub and takes those at or above the certain value (and above the running
+// maximum the result is folded into) one at a time, a lane per row.
+__global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
+                                   const double* __restrict__ A, const double* __restrict__ b,
+                                   const double* __restrict__ X64, const float* __restrict__ Xhi,
+                                   const float* __restrict__ Xlo, const float* __restrict__ ub,
+                                   const unsigned int* __restrict__ best, long long entries,
+                                   unsigned long long* out_key) {
+  const int lane = threadIdx.x & 31;
+  const long long e = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x);
+  const float floor_v = f32_unkey(*best);
+  const bool take = e < entries && !(ub[e] < floor_v);
+  unsigned int todo = __ballot_sync(0xffffffffu, take);
+  const long long e0 = e - lane;
+  while (todo) {
+    const int t = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const long long en = e0 + t;
+    const int tile = static_cast<int>(en / walkers), k = static_cast<int>(en - static_cast<long long>(tile) * walkers);
+    const size_t row = static_cast<size_t>(k) * n_ld;
+    const int r1 = min(m, (tile + 1) * group * kChkRows);
+    // Four rows a lane at once, four entries of each ahead: the sums are
+    // serial (index order), so the loads of one hide behind the others.
+    for (int r0 = tile * group * kChkRows; r0 < r1; r0 += kChkRows) {
+      const double* a[4];
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        a[q] = A + static_cast<size_t>(min(r0 + 32 * q + lane, m - 1)) * n_ld;
+      for (int i = 0; i < n; i += 4) {     // n_ld is a multiple of 32; zero past n
+        double2 av[4][2];
+        double xv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          av[q][0] = *reinterpret_cast<const double2*>(a[q] + i);
+          av[q][1] = *reinterpret_cast<const double2*>(a[q] + i + 2);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) xv[u] = load_point(mode, X64, Xhi, Xlo, row + i + u);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          s[q] += av[q][0].x * xv[0];
+          s[q] += av[q][0].y * xv[1];
+          s[q] += av[q][1].x * xv[2];
+          s[q] += av[q][1].y * xv[3];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + 32 * q + lane;
+        if (r < r1) atomicMax(out_key, f64_key(s[q] - b[r]));
+      }
+    }
+  }
+}
+
+// |A_E x - b_E| of the first 128 equalities: a block per walker, a thread per
+// equality.
+__global__ void check_eq_kernel(int mode, int n, int n_ld, int mE, const double* AE,
+                                const double* bE, const double* X64, const float* Xhi,
+                                const float* Xlo, unsigned long long* out_key) {
   extern __shared__ double xs[];
-  const int k = blockIdx.y;
+  const int k = blockIdx.x;
   const size_t row = static_cast<size_t>(k) * n_ld;
   for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = load_point(mode, X64, Xhi, Xlo, row + i);
   __syncthreads();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < m) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += A[static_cast<size_t>(r) * n_ld + i] * xs[i];
-    atomicMax(&out_keys[0], f64_key(s - b[r]));
-  }
-  if (blockIdx.x == 0 && r < mE) {
+  const int r = threadIdx.x;
+  if (r < mE) {
     double s = 0.0;
     for (int i = 0; i < n; ++i) s += AE[static_cast<size_t>(r) * n_ld + i] * xs[i];
-    atomicMax(&out_keys[1], f64_key(fabs(s - bE[r])));
+    atomicMax(out_key, f64_key(fabs(s - bE[r])));
   }
 }
 
@@ -1445,12 +1645,27 @@ cudaError_t launch_set_points(mhar_ctx* c, const double* X_dev) {
 
 cudaError_t launch_check(mhar_ctx* c, int walkers, unsigned long long* out_keys) {
   const int mode = c->opts.precision == MHAR_FP64 ? 0 : 1;
-  const int block = 128;
-  const int rows = c->m > c->mE ? c->m : c->mE;
-  dim3 grid(blocks_for(rows, block), walkers);
-  check_kernel<<<grid, block, sizeof(double) * c->n, c->stream>>>(
-      mode, c->m, c->n, c->n_ld, c->mE, c->d.A64, c->d.b64, c->d.AE64, c->d.bE64, c->d.X64,
-      c->d.Xhi, c->d.Xlo, out_keys);
+  // The screen's ub array lives in the emission buffer (z n doubles; every
+  // use of it is ordered on the context's stream): 2 n floats per walker, so
+  // row tiles are grouped when there are more of them than that.
+  const int tiles = blocks_for(c->m, kChkRows);
+  const int group = blocks_for(tiles, 2 * c->n);
+  const int groups = blocks_for(tiles, group);
+  float* ub = reinterpret_cast<float*>(c->d.emit);
+  unsigned int* best = reinterpret_cast<unsigned int*>(c->d.check + 5);
+  cudaError_t e = cudaMemsetAsync(best, 0, sizeof(*best), c->stream);
+  if (e != cudaSuccess) return e;
+  check_screen_kernel<<<dim3(groups, blocks_for(walkers, kChkWalkers)), kThreads, 0, c->stream>>>(
+      mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
+      c->d.Xlo, ub, best);
+  const long long entries = static_cast<long long>(groups) * walkers;
+  check_exact_kernel<<<blocks_for(entries, 128), 128, 0, c->stream>>>(
+      mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
+      c->d.Xlo, ub, best, entries, out_keys);
+  if (c->mE > 0)
+    check_eq_kernel<<<walkers, 128, sizeof(double) * c->n, c->stream>>>(
+        mode, c->n, c->n_ld, c->mE, c->d.AE64, c->d.bE64, c->d.X64, c->d.Xhi, c->d.Xlo,
+        out_keys + 1);
   return cudaGetLastError();
 }
 
