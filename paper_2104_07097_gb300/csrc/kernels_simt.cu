@@ -1691,10 +1691,11 @@ cudaError_t launch_reproject(mhar_ctx* c) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_prepare_tc_operands(mhar_ctx* c) {
+cudaError_t launch_prepare_tc_operands(mhar_ctx* c, bool blocks) {
   prepare_tc_kernel<<<c->m_pad, kThreads, 0, c->stream>>>(
       c->m, c->n, c->n_ld, c->m_pad, c->k_pad, mma_per_step(c), c->d.A64, c->d.b64, c->d.Ah,
       c->d.Al, c->d.row_scale, c->d.bS, c->d.rowk, c->d.sigma);
+  if (!blocks) return cudaGetLastError();
   const int groups = c->m_pad / 32;
   row_blocks_kernel<<<blocks_for(groups, 128), 128, 0, c->stream>>>(
       groups, c->d.bS, c->d.rowk, static_cast<float>(c->dir_norm2), static_cast<float>(c->dir_norminf),

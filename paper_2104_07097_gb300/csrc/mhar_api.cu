@@ -90,7 +90,20 @@ bool mixed(const mhar_ctx* c) {
 bool stored(const mhar_ctx* c) { return c->opts.precision == MHAR_MIXED_F16X3; }
 bool recompute(const mhar_ctx* c) { return c->opts.precision == MHAR_MIXED_RECOMPUTE; }
 
+// Gives up the screened chord's operands (pointers into one allocation).
+void drop_screen(mhar_ctx* c) {
+  mhar::DeviceBuffers& d = c->d;
+  if (!d.scr_mem) return;
+  cudaFree(d.scr_mem);
+  d.scr_mem = nullptr;
+  d.Ah = d.Al = d.Dh = d.Dl = d.Xh = d.Xl = nullptr;
+  d.row_scale = d.bS = d.rows = d.rowk = d.scr_walker = d.scr_nrm = nullptr;
+  d.scr_flags = nullptr;
+  d.scr_res = d.scr_tiles = nullptr;
+}
+
 void free_all(mhar_ctx* c) {
+  drop_screen(c);
   mhar::DeviceBuffers& d = c->d;
   void* ptrs[] = {d.A64, d.b64, d.A32, d.b32, d.kr32, d.AE64, d.Q64, d.Q32, d.Q32lo, d.bE64,
                   d.wE64, d.Lchol, d.Ah, d.Al, d.row_scale, d.bS, d.rows, d.rowk, d.nx_ref, d.theta_acc,
@@ -230,6 +243,7 @@ bool projection_draws(const mhar_ctx* c) {
 // the update kernel unless one warp per walker does both.
 int chord_launches(const mhar_ctx* c) {
   if (recompute(c)) return (!c->use_ts && c->use_sk) ? 2 : 1;
+  if (c->use_screen) return 3;
   return (mixed(c) || mhar::simt_warp_path(c)) ? 1 : 2;
 }
 
@@ -266,6 +280,7 @@ cudaError_t enqueue_chord(mhar_ctx* c, int j) {
     if (c->use_ts) return mhar::launch_recompute_ts(c, j);
     return c->use_sk ? mhar::launch_recompute_sk(c, j) : mhar::launch_recompute_tc(c, j);
   }
+  if (c->use_screen) return mhar::launch_screen(c, j);
   if (mhar::simt_warp_path(c)) return mhar::launch_chord_update_warp(c, j);
   cudaError_t e = mhar::launch_chord_simt(c);
   return e == cudaSuccess ? mhar::launch_update_simt(c, j) : e;
@@ -736,6 +751,7 @@ const char* mhar_kernel_name(const mhar_ctx* c) {
   if (!c) return "none";
   if (recompute(c)) return c->use_ts ? "recompute_ts_kernel" : (c->use_sk ? "recompute_sk_kernel" : "recompute_tc_kernel");
   if (stored(c)) return "walker_tc_kernel";
+  if (c->use_screen) return "screen_kernel";
   return mhar::simt_warp_path(c) ? "chord_warp_kernel" : "chord_simt_kernel";
 }
 
@@ -755,6 +771,35 @@ void mhar_destroy(mhar_ctx* c) {
   if (c->stream && c->stream != static_cast<cudaStream_t>(c->opts.stream))
     cudaStreamDestroy(c->stream);
   delete c;
+}
+
+// FP64 / FP32 modes: the screened chord's operands (kernels_screen.cu).  A body
+// outside its range, or memory that does not hold them, leaves the direct
+// kernels in place.
+static int try_screen(mhar_ctx* c) {
+  if (!mhar::screen_eligible(c)) return MHAR_OK;
+  mhar::DeviceBuffers& d = c->d;
+  const size_t bytes = mhar::screen_arena(c, nullptr);
+  if (cudaMalloc(reinterpret_cast<void**>(&d.scr_mem), bytes) != cudaSuccess) {
+    cudaGetLastError();
+    d.scr_mem = nullptr;
+    return MHAR_OK;
+  }
+  mhar::screen_arena(c, d.scr_mem);
+  MHAR_CUDA(cudaMemsetAsync(d.scr_mem, 0, bytes, c->stream), "screen memset");
+  int outside = 0;
+  MHAR_CUDA(mhar::screen_prepare(c, d.status + 1), "screen operands");
+  MHAR_CUDA(cudaMemcpyAsync(&outside, d.status + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
+            "copy");
+  MHAR_CUDA(cudaMemsetAsync(d.status + 1, 0, sizeof(int), c->stream), "memset");
+  MHAR_CUDA(cudaStreamSynchronize(c->stream), "sync");
+  if (outside) {
+    drop_screen(c);
+    return MHAR_OK;
+  }
+  const int rc = mhar::tc_plan_create(c);
+  c->use_screen = rc == MHAR_OK;
+  return rc;
 }
 
 static int create_impl(mhar_ctx* c, const double* A, const double* b, const double* AE,
@@ -964,6 +1009,8 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
       if (rc) return rc;
     }
     if (stored(c) && ((rc = reset_drift(c)) || (rc = refresh(c)))) return rc;
+  } else if ((rc = try_screen(c))) {
+    return rc;
   }
   MHAR_CUDA(cudaStreamSynchronize(c->stream), "create sync");
   return MHAR_OK;

@@ -65,6 +65,17 @@ struct DeviceBuffers {
   float* theta_acc = nullptr;    // z: sum |theta| ||d_hat||_2 since the refresh
   uint64_t* refresh_step = nullptr;  // iteration counter at the refresh
 
+  // FP64 / FP32 modes, screened chord (kernels_screen.cu): the walkers' bound
+  // factors, the FP32 mode's margin norms, range flags and scale exponents, and
+  // the bounds each epilogue thread kept.
+  // One allocation, scr_mem, holds these and the FP16 operands above.
+  uint8_t* scr_mem = nullptr;
+  float* scr_walker = nullptr;   // 4 z
+  float* scr_nrm = nullptr;      // 4 z (FP32 mode)
+  int* scr_flags = nullptr;      // 2 z
+  unsigned int* scr_res = nullptr;    // 4 x streams x z_ld
+  unsigned int* scr_tiles = nullptr;  // streams x z_ld
+
   // Chord bookkeeping.
   unsigned long long* key_lo = nullptr;  // z: ordered key of lambda_min (atomic max)
   unsigned long long* key_hi = nullptr;  // z: ordered key of lambda_max (atomic min)
@@ -118,6 +129,7 @@ struct mhar_ctx {
   bool use_ts = false;         // recompute mode: TMEM-operand kernel (n <= 128)
   bool use_sk = false;         // recompute mode: stream-K schedule (kernels_sk.cu)
   void* sk = nullptr;          // its segment table
+  bool use_screen = false;     // FP64 / FP32 modes: screened chord (kernels_screen.cu)
   int pc_rank = -1;            // -1: isotropic directions; else rank of U (0..32)
   // Recompute mode: the chord kernel itself moves the walkers, re-splits the
   // points and (with no projection / preconditioner) draws the next
@@ -175,12 +187,22 @@ cudaError_t launch_check(mhar_ctx* ctx, int walkers, unsigned long long* out_key
 // accumulated step sum reset, the refresh's iteration recorded.
 cudaError_t launch_stored_reset(mhar_ctx* ctx);
 cudaError_t launch_set_points(mhar_ctx* ctx, const double* X_dev);
-cudaError_t launch_prepare_tc_operands(mhar_ctx* ctx);
+// blocks: also the 32-row blocks of the chord epilogue (else the caller's own).
+cudaError_t launch_prepare_tc_operands(mhar_ctx* ctx, bool blocks = true);
 cudaError_t launch_refresh_simt(mhar_ctx* ctx);
 cudaError_t launch_reproject(mhar_ctx* ctx);
 // d <- delta .* d + U g on the drawn normals (FP64 / FP32 scratch), writing the
 // FP16 pair (divided by sigma) when `split`.
 cudaError_t launch_precondition(mhar_ctx* ctx, int j, int split);
+
+// ---- FP64 / FP32 modes, screened on the tensor cores (kernels_screen.cu) -------
+bool screen_eligible(const mhar_ctx* ctx);    // by its sizes
+// Places the screen's buffers in one allocation (base; null: only its size).
+size_t screen_arena(mhar_ctx* ctx, uint8_t* base);
+// The operands of A; *outside (device) is set when the body's values lie beyond
+// the screen's range.
+cudaError_t screen_prepare(mhar_ctx* ctx, int* outside);
+cudaError_t launch_screen(mhar_ctx* ctx, int j);   // chord, theta, move (3 launches)
 
 // ---- preconditioner fit (kernels_fit.cu) --------------------------------------
 struct FitScratch {
