@@ -1056,21 +1056,30 @@ __global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers
   }
 }
 
-// |A_E x - b_E| of the first 128 equalities: a block per walker, a thread per
-// equality.
-__global__ void check_eq_kernel(int mode, int n, int n_ld, int mE, const double* AE,
-                                const double* bE, const double* X64, const float* Xhi,
-                                const float* Xlo, unsigned long long* out_key) {
+// Both parts in one launch, every (row, walker) in FP64: a block per (128 rows,
+// walker).  Small checks (kCheckScreen products and below; the equalities of
+// the larger ones, with m = 0): 5 us where the screen's launches take 20.
+constexpr long long kCheckScreen = 1ll << 20;
+
+__global__ void check_kernel(int mode, int m, int n, int n_ld, int mE, const double* A,
+                             const double* b, const double* AE, const double* bE,
+                             const double* X64, const float* Xhi, const float* Xlo,
+                             unsigned long long* out_keys) {
   extern __shared__ double xs[];
-  const int k = blockIdx.x;
+  const int k = blockIdx.y;
   const size_t row = static_cast<size_t>(k) * n_ld;
   for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = load_point(mode, X64, Xhi, Xlo, row + i);
   __syncthreads();
-  const int r = threadIdx.x;
-  if (r < mE) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r < m) {
+    double s = 0.0;
+    for (int i = 0; i < n; ++i) s += A[static_cast<size_t>(r) * n_ld + i] * xs[i];
+    atomicMax(&out_keys[0], f64_key(s - b[r]));
+  }
+  if (blockIdx.x == 0 && r < mE) {
     double s = 0.0;
     for (int i = 0; i < n; ++i) s += AE[static_cast<size_t>(r) * n_ld + i] * xs[i];
-    atomicMax(out_key, f64_key(fabs(s - bE[r])));
+    atomicMax(&out_keys[1], f64_key(fabs(s - bE[r])));
   }
 }
 
@@ -1643,8 +1652,27 @@ cudaError_t launch_set_points(mhar_ctx* c, const double* X_dev) {
   return cudaGetLastError();
 }
 
+bool check_direct(const mhar_ctx* c, int walkers) {
+  return static_cast<long long>(c->m) * c->n * walkers <= kCheckScreen;
+}
+
+int check_launches(const mhar_ctx* c, int walkers) {
+  return check_direct(c, walkers) ? 1 : (c->mE > 0 ? 3 : 2);
+}
+
 cudaError_t launch_check(mhar_ctx* c, int walkers, unsigned long long* out_keys) {
   const int mode = c->opts.precision == MHAR_FP64 ? 0 : 1;
+  const int block = 128;
+  auto direct = [&](int m) {
+    const int rows = m > c->mE ? m : c->mE;
+    check_kernel<<<dim3(blocks_for(rows, block), walkers), block, sizeof(double) * c->n, c->stream>>>(
+        mode, m, c->n, c->n_ld, c->mE, c->d.A64, c->d.b64, c->d.AE64, c->d.bE64, c->d.X64,
+        c->d.Xhi, c->d.Xlo, out_keys);
+  };
+  if (check_direct(c, walkers)) {
+    direct(c->m);
+    return cudaGetLastError();
+  }
   // The screen's ub array lives in the emission buffer (z n doubles; every
   // use of it is ordered on the context's stream): 2 n floats per walker, so
   // row tiles are grouped when there are more of them than that.
@@ -1662,10 +1690,7 @@ cudaError_t launch_check(mhar_ctx* c, int walkers, unsigned long long* out_keys)
   check_exact_kernel<<<blocks_for(entries, 128), 128, 0, c->stream>>>(
       mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
       c->d.Xlo, ub, best, entries, out_keys);
-  if (c->mE > 0)
-    check_eq_kernel<<<walkers, 128, sizeof(double) * c->n, c->stream>>>(
-        mode, c->n, c->n_ld, c->mE, c->d.AE64, c->d.bE64, c->d.X64, c->d.Xhi, c->d.Xlo,
-        out_keys + 1);
+  if (c->mE > 0) direct(0);
   return cudaGetLastError();
 }
 

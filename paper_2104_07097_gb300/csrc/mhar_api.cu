@@ -602,7 +602,7 @@ int audit(mhar_ctx* c) {
   const int w = c->opts.audit_walkers > 0 ? c->opts.audit_walkers : c->z;
   MHAR_CUDA(mhar::launch_check(c, w, reinterpret_cast<unsigned long long*>(c->d.check) + 3),
             "audit kernel");
-  c->launches += c->mE > 0 ? 3 : 2;
+  c->launches += mhar::check_launches(c, w);
   ++c->audits;
   c->since_audit = 0;
   return MHAR_OK;

@@ -183,6 +183,7 @@ cudaError_t launch_emit(mhar_ctx* ctx, double* out_device, int walkers);  // wal
 // FP64 feasibility of walkers 0..walkers-1 into the keys at out_keys[0]
 // (max a_i x - b_i) and out_keys[1] (max |A_E x - b_E|).
 cudaError_t launch_check(mhar_ctx* ctx, int walkers, unsigned long long* out_keys);
+int check_launches(const mhar_ctx* ctx, int walkers);   // kernels of one check
 // Stored-slack mode, after a refresh: ||x / sigma|| of every walker, the
 // accumulated step sum reset, the refresh's iteration recorded.
 cudaError_t launch_stored_reset(mhar_ctx* ctx);
