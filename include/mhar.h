@@ -229,7 +229,8 @@ int mhar_set_audit(mhar_ctx* ctx, int32_t every, int32_t walkers);
  * (mixed mode).  Writes average device milliseconds:
  *   ms[0] direction draw (+ projection when mE > 0)   (Section 4.3); 0 in
  *         MHAR_MIXED_RECOMPUTE mode without equalities or preconditioner,
- *         where the chord kernel draws the next directions itself
+ *         where the chord kernel draws the next directions itself, and for
+ *         small bodies in the FP64 / FP32 modes, whose iterations share a launch
  *   ms[1] the rest of one iteration: the fused tensor-core kernel in the
  *         tensor-core modes, the chord and update kernels otherwise
  *         (Sections 4.4-4.5)

@@ -999,9 +999,12 @@ check_screen_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
   if ((tid & 31) == 0) atomicMax(best, f32_key(low));
 }
 
-// The FP64 values of the tiles the screen left: a warp looks at 32 entries of
-// ub and takes those at or above the certain value (and above the running
-// maximum the result is folded into) one at a time, a lane per row.
+// The FP64 values of the tiles the screen left: a warp looks at kChkEntries
+// entries of ub and takes those at or above the certain value one at a time, a
+// lane per row.  (Few entries a warp: sparse bodies with many slacks near the
+// least leave most of them, and 32 in turn took 35 us.)
+constexpr int kChkEntries = 4;
+
 __global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
                                    const double* __restrict__ A, const double* __restrict__ b,
                                    const double* __restrict__ X64, const float* __restrict__ Xhi,
@@ -1009,11 +1012,11 @@ __global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers
                                    const unsigned int* __restrict__ best, long long entries,
                                    unsigned long long* out_key) {
   const int lane = threadIdx.x & 31;
-  const long long e = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x);
+  const long long e0 =
+      (static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kChkEntries;
   const float floor_v = f32_unkey(*best);
-  const bool take = e < entries && !(ub[e] < floor_v);
+  const bool take = lane < kChkEntries && e0 + lane < entries && !(ub[e0 + lane] < floor_v);
   unsigned int todo = __ballot_sync(0xffffffffu, take);
-  const long long e0 = e - lane;
   while (todo) {
     const int t = __ffs(todo) - 1;
     todo &= todo - 1;
@@ -1058,8 +1061,9 @@ __global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers
 
 // Both parts in one launch, every (row, walker) in FP64: a block per (128 rows,
 // walker).  Small checks (kCheckScreen products and below; the equalities of
-// the larger ones, with m = 0): 5 us where the screen's launches take 20.
-constexpr long long kCheckScreen = 1ll << 20;
+// the larger ones, with m = 0): about 5 us and 7 us per 2^20 products where the
+// screen's launches take 25 us and hardly grow.
+constexpr long long kCheckScreen = 1ll << 22;
 
 __global__ void check_kernel(int mode, int m, int n, int n_ld, int mE, const double* A,
                              const double* b, const double* AE, const double* bE,
@@ -1687,7 +1691,7 @@ cudaError_t launch_check(mhar_ctx* c, int walkers, unsigned long long* out_keys)
       mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
       c->d.Xlo, ub, best);
   const long long entries = static_cast<long long>(groups) * walkers;
-  check_exact_kernel<<<blocks_for(entries, 128), 128, 0, c->stream>>>(
+  check_exact_kernel<<<blocks_for(entries, 4 * kChkEntries), 128, 0, c->stream>>>(
       mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
       c->d.Xlo, ub, best, entries, out_keys);
   if (c->mE > 0) direct(0);

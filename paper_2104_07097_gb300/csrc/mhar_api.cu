@@ -109,7 +109,8 @@ void free_all(mhar_ctx* c) {
                   d.wE64, d.Lchol, d.Ah, d.Al, d.row_scale, d.bS, d.rows, d.rowk, d.nx_ref, d.theta_acc,
                   d.refresh_step, d.X64, d.Xhi, d.Xlo, d.D64, d.D32, d.Dh, d.Dl, d.S, d.corr, d.corrn, d.Xh, d.Xl, d.wscale, d.Dh2, d.Dl2,
                   d.key_lo, d.key_hi, d.lmin, d.lmax, d.theta, d.status, d.counters, d.step,
-                  d.emit, d.check, d.pc_delta64, d.pc_U64, d.pc_delta32, d.pc_U32, d.sigma};
+                  d.emit, d.check, d.pc_delta64, d.pc_U64, d.pc_delta32, d.pc_U32, d.sigma,
+                  d.small_at};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   d = mhar::DeviceBuffers();
@@ -325,6 +326,31 @@ int capture(mhar_ctx* c, int count, cudaGraphExec_t* out) {
   e = cudaGraphInstantiate(out, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
+  return MHAR_OK;
+}
+
+// Small bodies: `count` iterations from iteration c->step, at most kSmallIters a
+// launch so that none runs for long.  out (device, may be null): the samples,
+// as SmallRun has them, with `phase` iterations since the last one done before.
+constexpr int kSmallIters = 1024;
+
+int advance_small(mhar_ctx* c, int64_t count, double* out, int64_t thin, int64_t phase) {
+  for (int64_t at = 0; at < count; at += kSmallIters) {
+    mhar::SmallRun r;
+    r.step = c->step + static_cast<uint64_t>(at);
+    r.iters = static_cast<int>(std::min<int64_t>(kSmallIters, count - at));
+    // A sample falls into this launch, and the indices fit.
+    const int64_t since = out ? (phase + at) % thin : 0;
+    if (out && since + r.iters >= thin) {
+      const int64_t wide = 2 * kSmallIters;   // one sample at most when thin is longer
+      r.thin = static_cast<int>(std::min(thin, wide));
+      r.phase = static_cast<int>(r.thin - (thin - since));
+      r.emit = emit_count(c);
+      r.out = out + static_cast<size_t>((phase + at) / thin) * r.emit * c->n;
+    }
+    MHAR_CUDA(mhar::launch_small(c, r), "iteration kernel");
+    ++c->launches;
+  }
   return MHAR_OK;
 }
 
@@ -751,6 +777,7 @@ const char* mhar_kernel_name(const mhar_ctx* c) {
   if (!c) return "none";
   if (recompute(c)) return c->use_ts ? "recompute_ts_kernel" : (c->use_sk ? "recompute_sk_kernel" : "recompute_tc_kernel");
   if (stored(c)) return "walker_tc_kernel";
+  if (c->use_small) return "small_kernel";
   if (c->use_screen) return "screen_kernel";
   return mhar::simt_warp_path(c) ? "chord_warp_kernel" : "chord_simt_kernel";
 }
@@ -773,28 +800,45 @@ void mhar_destroy(mhar_ctx* c) {
   delete c;
 }
 
-// FP64 / FP32 modes: the screened chord's operands (kernels_screen.cu).  A body
-// outside its range, or memory that does not hold them, leaves the direct
-// kernels in place.
-static int try_screen(mhar_ctx* c) {
-  if (!mhar::screen_eligible(c)) return MHAR_OK;
+// FP64 / FP32 modes: the operands of the screened chord (kernels_screen.cu) or of
+// the small-body kernel (kernels_small.cu).  A body outside their range, or
+// memory that does not hold them, leaves the direct kernels in place.
+static int try_fast_chord(mhar_ctx* c) {
+  const bool small = mhar::small_eligible(c);
+  if (!small && !mhar::screen_eligible(c)) return MHAR_OK;
   mhar::DeviceBuffers& d = c->d;
-  const size_t bytes = mhar::screen_arena(c, nullptr);
-  if (cudaMalloc(reinterpret_cast<void**>(&d.scr_mem), bytes) != cudaSuccess) {
+  const size_t bytes = small ? mhar::small_arena(c, nullptr) : mhar::screen_arena(c, nullptr);
+  uint8_t* mem = nullptr;
+  if (cudaMalloc(reinterpret_cast<void**>(&mem), bytes) != cudaSuccess) {
     cudaGetLastError();
-    d.scr_mem = nullptr;
     return MHAR_OK;
   }
-  mhar::screen_arena(c, d.scr_mem);
-  MHAR_CUDA(cudaMemsetAsync(d.scr_mem, 0, bytes, c->stream), "screen memset");
+  if (small) {
+    mhar::small_arena(c, mem);
+  } else {
+    d.scr_mem = mem;
+    mhar::screen_arena(c, mem);
+  }
+  MHAR_CUDA(cudaMemsetAsync(mem, 0, bytes, c->stream), "operand memset");
   int outside = 0;
-  MHAR_CUDA(mhar::screen_prepare(c, d.status + 1), "screen operands");
+  MHAR_CUDA(small ? mhar::small_prepare(c, d.status + 1) : mhar::screen_prepare(c, d.status + 1),
+            "operand preparation kernels");
   MHAR_CUDA(cudaMemcpyAsync(&outside, d.status + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
             "copy");
   MHAR_CUDA(cudaMemsetAsync(d.status + 1, 0, sizeof(int), c->stream), "memset");
   MHAR_CUDA(cudaStreamSynchronize(c->stream), "sync");
   if (outside) {
-    drop_screen(c);
+    if (small) {
+      cudaFree(d.small_at);
+      d.small_at = nullptr;
+      d.small_an = nullptr;
+    } else {
+      drop_screen(c);
+    }
+    return MHAR_OK;
+  }
+  if (small) {
+    c->use_small = true;
     return MHAR_OK;
   }
   const int rc = mhar::tc_plan_create(c);
@@ -1009,7 +1053,7 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
       if (rc) return rc;
     }
     if (stored(c) && ((rc = reset_drift(c)) || (rc = refresh(c)))) return rc;
-  } else if ((rc = try_screen(c))) {
+  } else if ((rc = try_fast_chord(c))) {
     return rc;
   }
   MHAR_CUDA(cudaStreamSynchronize(c->stream), "create sync");
@@ -1078,12 +1122,30 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
   const int64_t au = c->opts.audit_every;
   while (done < steps) {
     int64_t adv = steps - done;
-    if (thin > 0) adv = std::min<int64_t>(adv, thin - (done % thin));
+    // The small-body kernel writes samples itself: all of a call's when they
+    // stay on the device, else one to the staging buffer at a time.
+    const bool fused = c->use_small && nsamp > 0;
+    const bool whole = fused && c->opts.out_on_device;
+    if (thin > 0 && !whole) adv = std::min<int64_t>(adv, thin - (done % thin));
     if (k > 0) adv = std::min<int64_t>(adv, k - c->since_refresh);
     if (au > 0) adv = std::min<int64_t>(adv, au - c->since_audit);
-    if ((rc = advance(c, adv))) return rc;
+    if (c->use_small) {
+      double* to = !fused ? nullptr : whole
+                       ? out + static_cast<size_t>(done / thin) * emit_count(c) * c->n
+                       : c->d.emit;
+      rc = advance_small(c, adv, to, thin, fused ? done % thin : 0);
+    } else {
+      rc = advance(c, adv);
+    }
+    if (rc) return rc;
     done += adv;
     c->step += static_cast<uint64_t>(adv);
+    // Out of the staging buffer before the audit takes it as its scratch.
+    if (fused && !whole && done % thin == 0)
+      MHAR_CUDA(cudaMemcpyAsync(out + static_cast<size_t>(done / thin - 1) * emit_count(c) * c->n,
+                                c->d.emit, sizeof(double) * emit_count(c) * c->n,
+                                cudaMemcpyDeviceToHost, c->stream),
+                "sample copy");
     if (au > 0) {
       c->since_audit += adv;
       if (c->since_audit >= au && (rc = audit(c))) return rc;
@@ -1092,7 +1154,7 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
       c->since_refresh += adv;
       if (c->since_refresh >= k && (rc = refresh(c, true))) return rc;
     }
-    if (thin > 0 && done % thin == 0 && emitted < nsamp) {
+    if (!fused && thin > 0 && done % thin == 0 && emitted < nsamp) {
       if ((rc = emit_to(c, out + static_cast<size_t>(emitted) * emit_count(c) * c->n,
                         c->opts.out_on_device != 0, emit_count(c))))
         return rc;
@@ -1372,6 +1434,7 @@ int mhar_time_kernels(mhar_ctx* c, int iters, double* ms) {
   if (orc) return orc;
   // (1) `iters` real iterations, replayed back to back from one graph.
   auto full = [&]() -> cudaError_t {
+    if (c->use_small) return advance_small(c, iters, nullptr, 0, 0) ? cudaErrorUnknown : cudaSuccess;
     for (int it = 0; it < iters; ++it) {
       cudaError_t e = enqueue_directions(c, it);
       if (e == cudaSuccess) e = enqueue_chord(c, it);
@@ -1391,9 +1454,9 @@ int mhar_time_kernels(mhar_ctx* c, int iters, double* ms) {
   float t_full = 0.f, t_dir = 0.f, t_ref = 0.f;
   cudaError_t e = time_graph(c, full, &t_full);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel timing");
-  c->launches += static_cast<int64_t>(iters) * kernels_per_iteration(c) + 1;
+  if (!c->use_small) c->launches += static_cast<int64_t>(iters) * kernels_per_iteration(c) + 1;
   c->step += static_cast<uint64_t>(iters);
-  if (!tail_draws(c)) {  // otherwise the draw is part of the chord kernel
+  if (!tail_draws(c) && !c->use_small) {  // otherwise the draw is part of the chord kernel
     e = time_graph(c, dirs, &t_dir);
     if (e != cudaSuccess) return cuda_fail(c, e, "kernel timing");
     c->launches += static_cast<int64_t>(iters) * (kernels_per_iteration(c) - chord_launches(c));

@@ -76,6 +76,10 @@ struct DeviceBuffers {
   unsigned int* scr_res = nullptr;    // 4 x streams x z_ld
   unsigned int* scr_tiles = nullptr;  // streams x z_ld
 
+  // Small bodies in one launch (kernels_small.cu): A by columns, gamma ||a_i||_2.
+  uint8_t* small_at = nullptr;   // one allocation
+  float* small_an = nullptr;     // inside it
+
   // Chord bookkeeping.
   unsigned long long* key_lo = nullptr;  // z: ordered key of lambda_min (atomic max)
   unsigned long long* key_hi = nullptr;  // z: ordered key of lambda_max (atomic min)
@@ -129,6 +133,7 @@ struct mhar_ctx {
   bool use_ts = false;         // recompute mode: TMEM-operand kernel (n <= 128)
   bool use_sk = false;         // recompute mode: stream-K schedule (kernels_sk.cu)
   void* sk = nullptr;          // its segment table
+  bool use_small = false;      // FP64 / FP32 modes: all iterations of a call in one launch
   bool use_screen = false;     // FP64 / FP32 modes: screened chord (kernels_screen.cu)
   int pc_rank = -1;            // -1: isotropic directions; else rank of U (0..32)
   // Recompute mode: the chord kernel itself moves the walkers, re-splits the
@@ -204,6 +209,22 @@ size_t screen_arena(mhar_ctx* ctx, uint8_t* base);
 // the screen's range.
 cudaError_t screen_prepare(mhar_ctx* ctx, int* outside);
 cudaError_t launch_screen(mhar_ctx* ctx, int j);   // chord, theta, move (3 launches)
+
+// ---- FP64 / FP32 modes, small bodies (kernels_small.cu) -------------------------
+bool small_eligible(const mhar_ctx* ctx);     // by its sizes
+size_t small_arena(mhar_ctx* ctx, uint8_t* base);
+cudaError_t small_prepare(mhar_ctx* ctx, int* outside);   // as screen_prepare
+// `iters` iterations from iteration `step` (host counter: the device counter
+// is not used).  out: null, or the device buffer of the samples of walkers
+// 0 .. emit - 1 after the iterations it (0-based) with (phase + it + 1) % thin
+// == 0, sample (phase + it + 1) / thin - 1 at [..][emit][n].
+struct SmallRun {
+  uint64_t step = 0;
+  int iters = 0;
+  double* out = nullptr;
+  int emit = 0, thin = 1, phase = 0;
+};
+cudaError_t launch_small(mhar_ctx* ctx, const SmallRun& r);
 
 // ---- preconditioner fit (kernels_fit.cu) --------------------------------------
 struct FitScratch {

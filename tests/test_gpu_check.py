@@ -22,8 +22,8 @@ def reference(A, b, X):
 # one walker and ragged 64-walker tiles.
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("n,m,z", [(1, 2, 1), (1, 700, 65), (2, 1100, 3), (17, 127, 64),
-                                   (33, 128, 131), (100, 129, 63), (40, 1000, 200), (1, 5000, 300),
-                                   (64, 129, 130)])
+                                   (33, 128, 131), (100, 129, 63), (40, 1000, 200), (1, 5000, 900),
+                                   (64, 129, 520)])
 def test_check_against_numpy(precision, n, m, z):
     rng = np.random.default_rng(n + m + z)
     A = rng.standard_normal((m, n))
@@ -42,7 +42,7 @@ def test_check_against_numpy(precision, n, m, z):
 @pytest.mark.parametrize("kind", ["huge", "tiny", "ties", "cancel"])
 def test_check_screen_limits(kind):
     rng = np.random.default_rng(5)
-    n, m, z = 20, 300, 400
+    n, m, z = 20, 300, 800
     A, b = rng.standard_normal((m, n)), np.ones(m)
     X = 0.1 * rng.standard_normal((z, n))
     if kind == "huge":
