@@ -12,7 +12,7 @@
 //      Philox stream 3 for walker c at step 0), then power_iters times
 //      Q = orth(Y), Y = Sigma Q, and finally Q = orth(Y);
 //      orth is the Q factor with a positive diagonal in R, computed by
-//      classical Gram-Schmidt with one re-orthogonalisation pass;
+//      classical Gram-Schmidt with re-orthogonalisation;
 //   3. Rayleigh-Ritz: T = Q^T Sigma Q, T = V Lambda V^T by cyclic Jacobi
 //      rotations (Golub & Van Loan, Matrix Computations, Section 8.5),
 //      U = Q V Lambda_+^{1/2}, largest eigenvalue first;
@@ -25,6 +25,7 @@
 
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
+#include "tc_common.cuh"
 
 namespace mhar {
 namespace {
@@ -156,16 +157,42 @@ __global__ void omega_kernel(uint64_t seed, int n, int rank, double* Q) {
     if (4 * q + e < n) Q[static_cast<size_t>(4 * q + e) * kMaxPcRank + c] = v[e];
 }
 
-// Y = Sigma Q (n x n times n x 32): a warp per row, a lane per column.
-__global__ void symm_block_kernel(int n, const double* __restrict__ sigma,
-                                  const double* __restrict__ Q, double* __restrict__ Y) {
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= n) return;
-  const double* row = sigma + static_cast<size_t>(i) * n;
-  double acc = 0.0;
-  for (int k = 0; k < n; ++k) acc = fma(row[k], Q[static_cast<size_t>(k) * kMaxPcRank + lane], acc);
-  Y[static_cast<size_t>(i) * kMaxPcRank + lane] = acc;
+// Y = Sigma Q (n x n times n x 32): a lane per column; a block's eight warps
+// split the sum over k for kSymmRows rows and their partial sums are added in
+// warp order.  Bound by the FP64 rate (2 FMAs a clock and SM: 13 us for n = 500
+// on the whole chip); a warp per row, 63 blocks for n = 500, left it to the
+// latency of 500 dependent steps: 79 us, now 22.
+constexpr int kSymmRows = 4;
+constexpr int kSymmWarps = 8;
+
+__global__ void __launch_bounds__(kSymmWarps * 32)
+symm_block_kernel(int n, const double* __restrict__ sigma, const double* __restrict__ Q,
+                  double* __restrict__ Y) {
+  __shared__ double part[kSymmWarps][kSymmRows][kMaxPcRank];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * kSymmRows;
+  const int per = (n + kSymmWarps - 1) / kSymmWarps;
+  const int k0 = warp * per, k1 = min(n, k0 + per);
+  double acc[kSymmRows] = {};
+  const double* row[kSymmRows];
+#pragma unroll
+  for (int r = 0; r < kSymmRows; ++r)
+    row[r] = sigma + static_cast<size_t>(min(i0 + r, n - 1)) * n;
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k) {
+    const double q = Q[static_cast<size_t>(k) * kMaxPcRank + lane];
+#pragma unroll
+    for (int r = 0; r < kSymmRows; ++r) acc[r] = fma(row[r][k], q, acc[r]);
+  }
+#pragma unroll
+  for (int r = 0; r < kSymmRows; ++r) part[warp][r][lane] = acc[r];
+  __syncthreads();
+  if (warp < kSymmRows && i0 + warp < n) {
+    double s = part[0][warp][lane];
+#pragma unroll
+    for (int w = 1; w < kSymmWarps; ++w) s += part[w][warp][lane];
+    Y[static_cast<size_t>(i0 + warp) * kMaxPcRank + lane] = s;
+  }
 }
 
 __device__ double block_sum(double v, double* red) {
@@ -187,7 +214,8 @@ __device__ double block_sum(double v, double* red) {
 }
 
 // Q = orth(Y) for the first `rank` columns (zero beyond): classical
-// Gram-Schmidt, each column projected out twice, then normalised.  One block.
+// Gram-Schmidt, each column projected out twice, then normalised.  One block:
+// the general form, for n past what the cluster keeps in shared memory.
 __global__ void __launch_bounds__(kFitThreads)
 orth_kernel(int n, int rank, const double* __restrict__ Y, double* __restrict__ Q) {
   __shared__ double dots[kMaxPcRank];
@@ -229,130 +257,316 @@ orth_kernel(int n, int rank, const double* __restrict__ Y, double* __restrict__ 
   }
 }
 
-// Rayleigh-Ritz on span(Q) with SQ = Sigma Q, the diagonal floor, and the
-// outputs.  One block of 1024 threads; Jacobi on warp 0.
-__global__ void __launch_bounds__(kFitThreads)
-ritz_kernel(int n, int n_ld, int rank, const double* __restrict__ Q, const double* __restrict__ SQ,
-            const double* __restrict__ sigma_mat, double* delta64, double* U64, float* delta32,
-            float* U32, float* coord_scale, int* flag) {
-  __shared__ double T[kMaxPcRank][kMaxPcRank + 1];
-  __shared__ double V[kMaxPcRank][kMaxPcRank + 1];
-  __shared__ double lam[kMaxPcRank];
-  __shared__ int perm[kMaxPcRank];
-  __shared__ double red[33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // T = Q^T (Sigma Q), symmetrised.
-  {
-    const int a = warp, bcol = lane;
-    double acc = 0.0;
-    if (a < rank && bcol < rank)
-      for (int i = 0; i < n; ++i)
-        acc = fma(Q[static_cast<size_t>(i) * kMaxPcRank + a], SQ[static_cast<size_t>(i) * kMaxPcRank + bcol], acc);
-    T[a][bcol] = acc;
-    V[a][bcol] = a == bcol ? 1.0 : 0.0;
+__device__ __forceinline__ uint32_t cluster_addr(const void* local, uint32_t cta) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(remote)
+               : "r"(tc::smem_u32(local)), "r"(cta));
+  return remote;
+}
+__device__ __forceinline__ void st_cluster_f64(double* local, uint32_t cta, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(local, cta)), "d"(v)
+               : "memory");
+}
+__device__ __forceinline__ void st_cluster_u32(int* local, uint32_t cta, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(local, cta)), "r"(v)
+               : "memory");
+}
+
+// Q = orth(Y) by a cluster of kOrthCtas CTAs, each with a share of the rows in
+// shared memory (column-major, unnormalised until the end).  Column c is
+// projected out of the earlier ones; one exchange over distributed shared
+// memory brings every CTA the products with them and |v|^2, so |v - proj|^2
+// follows without another.  A second (third) projection only while one took
+// away more than half of |v|^2 -- "twice is enough" (Parlett, The Symmetric
+// Eigenvalue Problem, Section 6.9): with less taken the rounding left along
+// the earlier columns is of the order of the unit roundoff already.
+// Bound by the latency of the chain (products, exchange, update) and by the FP64
+// rate of the SMs, which one CTA alone used on one SM: n = 500, rank 32 took 1064
+// us in orth_kernel, 98 here.
+constexpr int kOrthCtas = 8;
+constexpr int kOrthThreads = 9 * 32;      // eight warps of products, one that sums
+constexpr int kOrthPasses = 3;
+constexpr int kOrthMaxLd = 872;           // 32 columns of 872 rows: 223232 bytes
+
+__host__ __device__ constexpr int orth_ld(int n) {   // 8 mod 16: spreads the banks
+  return ((n + kOrthCtas - 1) / kOrthCtas + 7) / 16 * 16 + 8;
+}
+
+__global__ void __cluster_dims__(kOrthCtas, 1, 1) __launch_bounds__(kOrthThreads)
+orth_cluster_kernel(int n, int rank, const double* __restrict__ Y, double* __restrict__ Q) {
+  extern __shared__ double col[];                      // [32][ld]
+  __shared__ double recv[2][kOrthCtas][kMaxPcRank];    // products of each CTA's rows
+  __shared__ double coef[kMaxPcRank];                  // products / |q_p|^2
+  __shared__ double inv2[kMaxPcRank];                  // 1 / |q_p|^2
+  __shared__ int again;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cta = static_cast<int>(blockIdx.x);
+  const int ld = orth_ld(n), per = (n + kOrthCtas - 1) / kOrthCtas;
+  const int r0 = cta * per, rows = max(0, min(per, n - r0));
+  for (int e = tid; e < rows * kMaxPcRank; e += kOrthThreads)
+    col[(e & 31) * ld + (e >> 5)] = Y[static_cast<size_t>(r0) * kMaxPcRank + e];
+  // No CTA writes into another before that one runs.
+  tc::cluster_sync_all();
+
+  int turn = 0;
+  for (int c = 0; c < rank; ++c) {
+    double* v = col + c * ld;
+    for (int pass = 0; pass < kOrthPasses; ++pass) {
+      // Written for pass t + 2 only when every CTA has read it in pass t.
+      auto& got = recv[turn];
+      turn ^= 1;
+      // Products of columns 0 .. c with v: 8 lanes a column, which then send
+      // the sum to one CTA each.
+      const int p = tid >> 3, g = tid & 7;
+      if ((tid & ~31) >> 3 <= c && warp < 8) {
+        double acc = 0.0;
+        if (p <= c)
+          for (int i = g; i < rows; i += 8) acc = fma(col[p * ld + i], v[i], acc);
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        st_cluster_f64(&got[cta][p], static_cast<uint32_t>(g), acc);
+      }
+      tc::cluster_sync_all();
+      double nrm2 = 0.0, vv = 0.0;
+      if (warp == 8) {
+        double s[kOrthCtas];
+#pragma unroll
+        for (int r = 0; r < kOrthCtas; ++r) s[r] = lane <= c ? got[r][lane] : 0.0;
+        // The same order in every CTA: every CTA decides alike.
+        const double dot = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+        const double cf = lane < c ? dot * inv2[lane] : 0.0;
+        coef[lane] = cf;
+        nrm2 = lane < c ? -dot * cf : dot;     // dot = 0 past c
+        vv = dot;
+      }
+      __syncthreads();
+      if (warp < 8) {
+        // v -= sum_p coef_p q_p: four lanes a row.
+        const int h = tid & 3;
+        for (int ib = 0; ib < rows; ib += 64) {
+          const int i = ib + (tid >> 2);
+          double acc = 0.0;
+          if (i < rows)
+            for (int q = h; q < c; q += 4) acc = fma(coef[q], col[q * ld + i], acc);
+          acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+          acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+          if (h == 0 && i < rows) v[i] -= acc;
+        }
+      } else {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, off);
+        vv = __shfl_sync(0xffffffffu, vv, c);
+        if (lane == 0) {
+          again = !(nrm2 >= 0.5 * vv);
+          inv2[c] = nrm2 > 0.0 ? 1.0 / nrm2 : 0.0;
+        }
+      }
+      __syncthreads();
+      if (!again) break;
+    }
   }
-  __syncthreads();
-  {
-    const int a = warp, bcol = lane;
-    const double s = 0.5 * (T[a][bcol] + T[bcol][a]);
-    __syncthreads();
-    T[a][bcol] = s;
+  for (int e = tid; e < rows * kMaxPcRank; e += kOrthThreads) {
+    const int c = e & 31;
+    Q[static_cast<size_t>(r0) * kMaxPcRank + e] =
+        c < rank ? col[c * ld + (e >> 5)] * sqrt(inv2[c]) : 0.0;
   }
+}
+
+// T = Q^T (Sigma Q): a block per row of T, a lane per column, the sum over the
+// coordinates split over the warps and added in their order.
+__global__ void __launch_bounds__(256)
+ritz_matrix_kernel(int n, int rank, const double* __restrict__ Q, const double* __restrict__ SQ,
+                   double* __restrict__ T) {
+  __shared__ double part[8][kMaxPcRank];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = blockIdx.x;
+  double acc = 0.0;
+  if (a < rank && lane < rank)
+#pragma unroll 4
+    for (int i = warp; i < n; i += 8)
+      acc = fma(Q[static_cast<size_t>(i) * kMaxPcRank + a],
+                SQ[static_cast<size_t>(i) * kMaxPcRank + lane], acc);
+  part[warp][lane] = acc;
   __syncthreads();
-  if (warp == 0 && rank > 1) {
-    for (int sweep = 0; sweep < 60; ++sweep) {
+  if (warp == 0) {
+    double s = part[0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w][lane];
+    T[a * kMaxPcRank + lane] = s;
+  }
+}
+
+// T = V Lambda V^T by Jacobi rotations in cyclic row order, all rotations of
+// one antidiagonal p + q at once: (p, q) shares an index only with rotations
+// of smaller p + q before it in that order and of larger p + q after it, so
+// the result is the row-cyclic one with 2 rank - 3 steps a sweep instead of
+// rank (rank - 1) / 2.  Two CTAs: the first rotates T (a warp per pair), the
+// second V, one step behind, so V's half of the FP64 work is off the chain.
+// The angle comes from FP32 (a relative error of 1e-7 in tan leaves that share
+// of the entry to the next sweep); cos and sin are normalised in FP64, so the
+// rotations are orthogonal to the FP64 roundoff.
+// Bound by the chain of steps and one SM's FP64 rate; rank 32 with one warp and
+// one rotation at a time took most of 8018 us, 697 here.
+constexpr int kJacobiThreads = 512;
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kJacobiThreads)
+jacobi_kernel(int rank, const double* __restrict__ Tin, double* __restrict__ lam,
+              double* __restrict__ Vout) {
+  __shared__ double M[kMaxPcRank][kMaxPcRank + 1];     // T, or V
+  __shared__ double2 rot[2][kMaxPcRank / 2];           // (cos, sin) of a step's pairs
+  __shared__ double red[2][kJacobiThreads / 32];
+  __shared__ int go;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool t_side = blockIdx.x == 0;
+  // Scaled by a power of two to a trace near 1 (the angles are formed in FP32).
+  double tr = 0.0;
+  for (int a = 0; a < rank; ++a) tr += fabs(Tin[a * kMaxPcRank + a]);
+  int e = 0;
+  if (tr > 0.0 && isfinite(tr)) frexp(tr, &e);
+  e = max(-1000, min(1000, e));
+  const double down = ldexp(1.0, -e), up = ldexp(1.0, e);
+  for (int idx = tid; idx < kMaxPcRank * kMaxPcRank; idx += kJacobiThreads) {
+    const int a = idx >> 5, b = idx & 31;
+    M[a][b] = t_side ? 0.5 * (Tin[a * kMaxPcRank + b] + Tin[b * kMaxPcRank + a]) * down
+                     : (a == b ? 1.0 : 0.0);
+  }
+  tc::cluster_sync_all();
+  for (int sweep = 0; sweep < 60; ++sweep) {
+    if (t_side) {
       double off = 0.0, tot = 0.0;
-      for (int a = 0; a < rank; ++a) {
-        const double v = lane < rank ? T[a][lane] : 0.0;
-        tot += v * v;
-        if (lane != a) off += v * v;
+      for (int a = warp; a < kMaxPcRank; a += kJacobiThreads / 32) {
+        const double v = M[a][lane], v2 = v * v;
+        tot += v2;
+        if (lane != a) off += v2;
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         off += __shfl_xor_sync(0xffffffffu, off, o);
         tot += __shfl_xor_sync(0xffffffffu, tot, o);
       }
-      if (!(off > 1e-30 * tot)) break;
-      for (int p = 0; p < rank - 1; ++p) {
-        for (int q = p + 1; q < rank; ++q) {
-          const double apq = T[p][q];
-          if (apq == 0.0) continue;
-          const double tau = (T[q][q] - T[p][p]) / (2.0 * apq);
-          const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          const double cs = 1.0 / sqrt(1.0 + t * t);
-          const double sn = t * cs;
-          __syncwarp();
-          // T <- T J (columns p, q), V <- V J.
-          if (lane < rank) {
-            const double tp = T[lane][p], tq = T[lane][q];
-            T[lane][p] = cs * tp - sn * tq;
-            T[lane][q] = sn * tp + cs * tq;
-            const double vp = V[lane][p], vq = V[lane][q];
-            V[lane][p] = cs * vp - sn * vq;
-            V[lane][q] = sn * vp + cs * vq;
+      if (lane == 0) { red[0][warp] = off; red[1][warp] = tot; }
+      __syncthreads();
+      if (tid == 0) {
+        off = tot = 0.0;
+        for (int w = 0; w < kJacobiThreads / 32; ++w) { off += red[0][w]; tot += red[1][w]; }
+        go = off > 1e-30 * tot;
+        st_cluster_u32(&go, 1u, static_cast<uint32_t>(go));
+      }
+      __syncwarp();
+    }
+    tc::cluster_sync_all();
+    if (!go) break;
+    for (int t = 1; t <= 2 * rank - 3; ++t) {
+      const int p0 = max(0, t - rank + 1), pairs = (t - 1) / 2 - p0 + 1;
+      const int p = p0 + warp, q = t - p;
+      double2* const cs = rot[t & 1];
+      if (t_side) {
+        if (warp == 0 && lane < pairs) {
+          const int pp = p0 + lane, qq = t - pp;
+          const float apq = static_cast<float>(M[pp][qq]);
+          double2 r = make_double2(1.0, 0.0);
+          if (apq != 0.0f) {
+            const float tau = static_cast<float>(M[qq][qq] - M[pp][pp]) / (2.0f * apq);
+            const double tn = static_cast<double>((tau >= 0.0f ? 1.0f : -1.0f) /
+                                                  (fabsf(tau) + sqrtf(1.0f + tau * tau)));
+            // 1 / sqrt(1 + tn^2), 1 <= 1 + tn^2 <= 2: one step of third order from
+            // the FP32 value (error below 1e-20 of it before rounding).
+            const double w = fma(tn, tn, 1.0);
+            const double y = static_cast<double>(rsqrtf(static_cast<float>(w)));
+            const double d = fma(-w * y, y, 1.0);
+            r.x = fma(y * d, fma(0.375, d, 0.5), y);
+            r.y = tn * r.x;
           }
-          __syncwarp();
-          // T <- J^T T (rows p, q).
-          if (lane < rank) {
-            const double tp = T[p][lane], tq = T[q][lane];
-            T[p][lane] = cs * tp - sn * tq;
-            T[q][lane] = sn * tp + cs * tq;
-          }
-          __syncwarp();
+          cs[lane] = r;
+          st_cluster_f64(&cs[lane].x, 1u, r.x);
+          st_cluster_f64(&cs[lane].y, 1u, r.y);
+        }
+        __syncthreads();
+        tc::cluster_arrive();
+        if (warp < pairs) {      // T <- T J
+          const double c = cs[warp].x, s = cs[warp].y;
+          const double a = M[lane][p], b = M[lane][q];
+          M[lane][p] = c * a - s * b;
+          M[lane][q] = s * a + c * b;
+        }
+        __syncthreads();
+        if (warp < pairs) {      // T <- J^T T
+          const double c = cs[warp].x, s = cs[warp].y;
+          const double a = M[p][lane], b = M[q][lane];
+          M[p][lane] = c * a - s * b;
+          M[q][lane] = s * a + c * b;
+        }
+        __syncthreads();
+        tc::cluster_wait();      // the step before is done with the other buffer
+      } else {
+        tc::cluster_arrive();
+        tc::cluster_wait();
+        if (warp < pairs) {      // V <- V J
+          const double c = cs[warp].x, s = cs[warp].y;
+          const double a = M[lane][p], b = M[lane][q];
+          M[lane][p] = c * a - s * b;
+          M[lane][q] = s * a + c * b;
         }
       }
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // Eigenvalues largest first (selection sort over at most 32 values).
-    bool used[kMaxPcRank];
-    for (int a = 0; a < kMaxPcRank; ++a) used[a] = false;
-    for (int a = 0; a < rank; ++a) {
-      int best = -1;
-      for (int q = 0; q < rank; ++q)
-        if (!used[q] && (best < 0 || T[q][q] > T[best][best])) best = q;
-      used[best] = true;
-      perm[a] = best;
-      lam[a] = fmax(T[best][best], 0.0);
-    }
+  if (t_side) {
+    if (tid < kMaxPcRank) lam[tid] = tid < rank ? M[tid][tid] * up : 0.0;
+  } else {
+    for (int idx = tid; idx < kMaxPcRank * kMaxPcRank; idx += kJacobiThreads)
+      Vout[idx] = M[idx >> 5][idx & 31];
   }
-  __syncthreads();
+}
+
+// U = Q V Lambda_+^{1/2} (largest eigenvalue first), the diagonal floor and the
+// outputs: a warp per coordinate.  (Rank 0: the diagonal alone.)
+__global__ void __launch_bounds__(256)
+ritz_finish_kernel(int n, int n_ld, int rank, const double* __restrict__ Q,
+                   const double* __restrict__ lam_in, const double* __restrict__ V_in,
+                   const double* __restrict__ sigma_mat, double* delta64, double* U64,
+                   float* delta32, float* U32, int* flag) {
+  __shared__ double V[kMaxPcRank][kMaxPcRank + 1];
+  __shared__ double lam[kMaxPcRank];
+  __shared__ int perm[kMaxPcRank];
+  __shared__ double red[33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (rank > 0)
+    for (int idx = threadIdx.x; idx < kMaxPcRank * kMaxPcRank; idx += blockDim.x)
+      V[idx >> 5][idx & 31] = V_in[idx];
+  if (warp == 0 && lane < rank) {
+    const double mine = lam_in[lane];
+    int at = 0;
+    for (int q = 0; q < rank; ++q) at += lam_in[q] > mine || (lam_in[q] == mine && q < lane);
+    perm[at] = lane;
+    lam[at] = fmax(mine, 0.0);
+  }
   // Trace of Sigma for the absolute floor.
   double part = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) part += sigma_mat[static_cast<size_t>(i) * n + i];
   const double tr = block_sum(part, red);
-  // Rows of U, delta and the coordinate scale: a warp per coordinate.
-  for (int i = warp; i < n_ld; i += blockDim.x >> 5) {
-    double u = 0.0;
-    if (i < n && lane < rank) {
-      const int col = perm[lane];
-      for (int bcol = 0; bcol < rank; ++bcol)
-        u = fma(Q[static_cast<size_t>(i) * kMaxPcRank + bcol], V[bcol][col], u);
-      u *= sqrt(lam[lane]);
-    }
-    double u2 = u * u;
+  const int i = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (i >= n_ld) return;
+  double u = 0.0;
+  if (i < n && lane < rank) {
+    const int c = perm[lane];
+    for (int b = 0; b < rank; ++b) u = fma(Q[static_cast<size_t>(i) * kMaxPcRank + b], V[b][c], u);
+    u *= sqrt(lam[lane]);
+  }
+  double u2 = u * u;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) u2 += __shfl_xor_sync(0xffffffffu, u2, o);
-    double d2 = 0.0, sc = 1.0;
-    if (i < n) {
-      const double sii = sigma_mat[static_cast<size_t>(i) * n + i];
-      d2 = fmax(sii - u2, fmax(kEpsRel * sii, kEpsAbs * tr / n));
-      const double var = d2 + u2;
-      if (!isfinite(var) || !isfinite(u)) atomicOr(flag, 1);
-      if (var > 0.0 && isfinite(var)) {
-        int e = 0;
-        frexp(sqrt(var), &e);
-        sc = ldexp(1.0, e);
-      }
-    }
-    U64[static_cast<size_t>(i) * kMaxPcRank + lane] = u;
-    U32[static_cast<size_t>(i) * kMaxPcRank + lane] = static_cast<float>(u);
-    if (lane == 0) {
-      delta64[i] = sqrt(d2);
-      delta32[i] = static_cast<float>(sqrt(d2));
-      if (coord_scale) coord_scale[i] = static_cast<float>(sc);
-    }
+  for (int o = 16; o > 0; o >>= 1) u2 += __shfl_xor_sync(0xffffffffu, u2, o);
+  double d2 = 0.0;
+  if (i < n) {
+    const double sii = sigma_mat[static_cast<size_t>(i) * n + i];
+    d2 = fmax(sii - u2, fmax(kEpsRel * sii, kEpsAbs * tr / n));
+    if (!isfinite(d2 + u2) || !isfinite(u)) atomicOr(flag, 1);
+  }
+  U64[static_cast<size_t>(i) * kMaxPcRank + lane] = u;
+  U32[static_cast<size_t>(i) * kMaxPcRank + lane] = static_cast<float>(u);
+  if (lane == 0) {
+    delta64[i] = sqrt(d2);
+    delta32[i] = static_cast<float>(sqrt(d2));
   }
 }
 
@@ -385,25 +599,35 @@ cudaError_t launch_fit_factor(mhar_ctx* c, FitScratch* f, long long samples, int
       n, static_cast<double>(samples), f->s1, f->s2, f->sigma, f->flag);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int rows_per_block = 8;
   if (rank > 0) {
     omega_kernel<<<blocks_for(static_cast<long long>(kMaxPcRank) * ((n + 3) / 4), 256), 256, 0,
                    c->stream>>>(c->opts.seed, n, rank, f->Q);
-    symm_block_kernel<<<blocks_for(n, rows_per_block), rows_per_block * 32, 0, c->stream>>>(
-        n, f->sigma, f->Q, f->Y);
-    for (int it = 0; it < power_iters; ++it) {
-      orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->Y, f->Q);
-      symm_block_kernel<<<blocks_for(n, rows_per_block), rows_per_block * 32, 0, c->stream>>>(
-          n, f->sigma, f->Q, f->Y);
+    const size_t smem = sizeof(double) * kMaxPcRank * orth_ld(n);
+    const bool cluster = orth_ld(n) <= kOrthMaxLd;
+    if (cluster) {
+      // The largest any call needs: the attribute belongs to the function.
+      e = cudaFuncSetAttribute(orth_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(sizeof(double) * kMaxPcRank * kOrthMaxLd));
+      if (e != cudaSuccess) return e;
     }
-    orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->Y, f->Q);
-    symm_block_kernel<<<blocks_for(n, rows_per_block), rows_per_block * 32, 0, c->stream>>>(
+    for (int it = 0; it <= power_iters; ++it) {
+      symm_block_kernel<<<blocks_for(n, kSymmRows), kSymmWarps * 32, 0, c->stream>>>(
+          n, f->sigma, f->Q, f->Y);
+      if (cluster)
+        orth_cluster_kernel<<<kOrthCtas, kOrthThreads, smem, c->stream>>>(n, rank, f->Y, f->Q);
+      else
+        orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->Y, f->Q);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    symm_block_kernel<<<blocks_for(n, kSymmRows), kSymmWarps * 32, 0, c->stream>>>(
         n, f->sigma, f->Q, f->Y);
+    ritz_matrix_kernel<<<kMaxPcRank, 256, 0, c->stream>>>(n, rank, f->Q, f->Y, f->T);
+    jacobi_kernel<<<2, kJacobiThreads, 0, c->stream>>>(rank, f->T, f->lam, f->V);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  ritz_kernel<<<1, kFitThreads, 0, c->stream>>>(n, c->n_ld, rank, f->Q, f->Y, f->sigma,
-                                                c->d.pc_delta64, c->d.pc_U64, c->d.pc_delta32,
-                                                c->d.pc_U32, nullptr, f->flag);
+  ritz_finish_kernel<<<blocks_for(c->n_ld, 8), 256, 0, c->stream>>>(
+      n, c->n_ld, rank, f->Q, f->lam, f->V, f->sigma, c->d.pc_delta64, c->d.pc_U64,
+      c->d.pc_delta32, c->d.pc_U32, f->flag);
   return cudaGetLastError();
 }
 

@@ -660,21 +660,30 @@ bool factor_args_ok(mhar_ctx* c, int32_t rank, int32_t power_iters) {
 
 void fit_release(mhar_ctx* c, mhar::FitScratch* f) {
   cudaStreamSynchronize(c->stream);
-  void* ptrs[] = {f->shift, f->s1, f->s2, f->sigma, f->Y, f->Q, f->flag};
-  for (void* p : ptrs)
-    if (p) cudaFree(p);
+  if (f->arena) cudaFree(f->arena);
   *f = mhar::FitScratch();
 }
 
 int fit_alloc(mhar_ctx* c, mhar::FitScratch* f) {
-  const size_t n = static_cast<size_t>(c->n), nn = n * n;
+  // One allocation: seven took longer than the kernels of a small fit.
+  const size_t n = static_cast<size_t>(c->n), R = mhar::kMaxPcRank;
+  double** parts[] = {&f->shift, &f->s1, &f->s2, &f->sigma, &f->Y, &f->Q, &f->T, &f->V, &f->lam};
+  const size_t counts[] = {n, n, n * n, n * n, n * R, n * R, R * R, R * R, R};
+  size_t total = 32;                       // the flag
+  for (size_t k : counts) total += (k + 31) / 32 * 32;
+  double* base = nullptr;
   int rc;
-  if ((rc = dmalloc(c, &f->shift, n)) || (rc = dmalloc(c, &f->s1, n)) || (rc = dmalloc(c, &f->s2, nn)) ||
-      (rc = dmalloc(c, &f->sigma, nn)) || (rc = dmalloc(c, &f->Y, n * mhar::kMaxPcRank)) ||
-      (rc = dmalloc(c, &f->Q, n * mhar::kMaxPcRank)) || (rc = dmalloc(c, &f->flag, 1)) ||
-      (rc = alloc_preconditioner(c))) {
+  if ((rc = dmalloc(c, &base, total)) || (rc = alloc_preconditioner(c))) {
+    f->arena = base;
     fit_release(c, f);
     return rc;
+  }
+  f->arena = base;
+  f->flag = reinterpret_cast<int*>(base);
+  base += 32;
+  for (size_t i = 0; i < sizeof(counts) / sizeof(counts[0]); ++i) {
+    *parts[i] = base;
+    base += (counts[i] + 31) / 32 * 32;
   }
   return MHAR_OK;
 }
@@ -708,7 +717,7 @@ int fit_factor_device(mhar_ctx* c, mhar::FitScratch* f, long long samples, int r
                       int power_iters) {
   cudaError_t e = mhar::launch_fit_factor(c, f, samples, rank, power_iters);
   if (e != cudaSuccess) return cuda_fail(c, e, "preconditioner fit kernels");
-  c->launches += rank > 0 ? 5 + 2 * power_iters : 2;
+  c->launches += rank > 0 ? 8 + 2 * power_iters : 2;
   int flag = 0;
   e = cudaMemcpyAsync(&flag, f->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -228,12 +228,16 @@ cudaError_t launch_small(mhar_ctx* ctx, const SmallRun& r);
 
 // ---- preconditioner fit (kernels_fit.cu) --------------------------------------
 struct FitScratch {
+  void* arena = nullptr;     // holds all of the below
   double* shift = nullptr;   // n: centre subtracted before the products
   double* s1 = nullptr;      // n: sum of (x - shift)
   double* s2 = nullptr;      // n x n: sum of (x - shift)(x - shift)^T (upper tiles)
   double* sigma = nullptr;   // n x n covariance
   double* Y = nullptr;       // n x 32
   double* Q = nullptr;       // n x 32
+  double* T = nullptr;       // 32 x 32: Q^T Sigma Q
+  double* V = nullptr;       // 32 x 32: its eigenvectors
+  double* lam = nullptr;     // 32: its eigenvalues
   int* flag = nullptr;       // [0] set when a fit kernel met a non-finite value
 };
 cudaError_t launch_fit_shift(mhar_ctx* ctx, FitScratch* f);   // shift = walker 0's point
