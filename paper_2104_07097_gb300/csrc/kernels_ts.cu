@@ -54,7 +54,12 @@ constexpr int kSlotBytes = kTile * kTcKChunk * 2;    // 128 x 64 FP16 = 16 KB
 constexpr int kSlots = 8;                            // two tiles of A (hi, lo) ahead
 constexpr int kPairs = kSlots / 2;                   // hi + lo of one K chunk per barrier
 constexpr int kEpiWarps = 16;
-constexpr int kThreadsTs = (2 + kEpiWarps) * 32;
+constexpr int kEpiThreads = kEpiWarps * 32;
+// Warps 18 and 19 draw the next directions beside the tiles.  Twenty warps are
+// five on each sub-partition, as eighteen are on two: 96 registers either way.
+constexpr int kDrawWarp = 2 + kEpiWarps;
+constexpr int kDrawThreads = 64;
+constexpr int kThreadsTs = kDrawWarp * 32 + kDrawThreads;
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kOpCol = 256;                     // first TMEM column of the walker operands
 
@@ -69,42 +74,60 @@ struct TsParams {
   int* status;
   unsigned long long* counters;
   int* err;
-  const uint64_t* step_ptr;
-  uint64_t seed;
-  int j;
+  const uint64_t* step_ptr; // the iteration is *step_ptr + j, or (null) step0
+  uint64_t* step_out;       // null, or where the next iteration's number goes
+  uint64_t seed, step0;
+  int j, iters;             // iterations of this launch
+  double* out;              // samples, SmallRun's layout, or null
+  int emit, thin, phase;
   uint32_t walker0;
-  int z, z_ld, kdim, k_chunks, k_pad, tiles_per_cta, m_tiles;
+  int resident;             // the walkers' points stay in shared memory (TsState)
+  int epi_items;            // draw items that the epilogue warps take
+  int n, z, z_ld, kdim, k_chunks, k_pad, tiles_per_cta, m_tiles;
   WalkerTail wt;            // walker-side work (walker_tail.cuh)
 };
+
+// Floats between two walkers' low-rank normals: 16-byte rows, and the rows that a
+// quarter warp reads at once lie on different banks.
+constexpr int kGStride = kMaxPcRank + 4;
 
 struct alignas(16) TsTail {
   uint64_t a_full[kSlots];
   uint64_t a_empty[kSlots];
   uint64_t p_full, p_empty;    // P accumulator: MMAs done / copied out
   uint64_t g_full, g_empty;    // G accumulator
+  uint64_t c_full;             // partial chords of this CTA's walkers
   uint32_t tmem_base;
   int timed_out;
-  float part_lo[4][kWalkers];
-  float part_hi[4][kWalkers];
-  float recv_lo[kMaxCluster][kWalkers];
-  float recv_hi[kMaxCluster][kWalkers];
-  float theta_s[kWalkers];
+  // (lambda_min, lambda_max) of a walker of this CTA from each epilogue warp
+  // group of each CTA: [4 rank + group] [walker], rows of `share` walkers.
+  float2 recv[4 * (kWalkers + kMaxCluster)];
+  float theta_s[kWalkers];            // of the strip's walkers; this CTA's share is set
   double theta_u[kWalkers];           // the chord's uniform u (Philox stream 1), drawn early
-  unsigned int red[kWalkers];
+  unsigned int red[kWalkers];         // this CTA's walkers: largest |x / sigma| (bits)
   float nrm[3][kWalkers];             // each walker's ||d_hat||_2, ||x_hat||_2, max |d_hat|
-  float gs[kWalkers * kMaxPcRank];    // low-rank normals of a preconditioned draw
+  alignas(16) float gs[kWalkers * kGStride];   // low-rank normals of a preconditioned draw
 };
 
-// The walker-side items staged at kernel start: one slot per epilogue thread.
-constexpr size_t kStageBytes = static_cast<size_t>(kEpiWarps) * 32 * kTailStageBytes;
+// The walker-side items.  Either (TsParams::resident) the points of the CTA's
+// walkers for the whole launch: part p of item i, 16 bytes, at (512 p + i) 16, the
+// parts X hi (2), X lo (2), D hi and D lo of pair 0, then of pair 1; or one slot
+// per epilogue thread for its first item, staged in each iteration.
+constexpr int kStateParts = 8;
+constexpr size_t kStageBytes = static_cast<size_t>(kEpiThreads) * 16 * kStateParts;
+static_assert(kStageBytes >= static_cast<size_t>(kEpiThreads) * kTailStageBytes, "stage slots");
 constexpr size_t kSmemTs =
     1024 + static_cast<size_t>(kSlots) * kSlotBytes + sizeof(TsTail) + kStageBytes;
 static_assert(kSmemTs <= 232448, "recompute_ts_kernel exceeds the shared memory of a CTA");
 
-__device__ __forceinline__ void st_dsmem(float* local, uint32_t rank, float v) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+// A pair of floats into CTA `rank`'s copy of *local; counts on its barrier *bar.
+__device__ __forceinline__ void push2(float2* local, uint64_t* bar, uint32_t rank, float x, float y) {
+  uint32_t dst, rbar;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(smem_u32(local)), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar) : "r"(smem_u32(bar)), "r"(rank));
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+                   dst), "f"(x), "f"(y), "r"(rbar)
+               : "memory");
 }
 
 __device__ __forceinline__ void arrive(uint64_t* bar) {
@@ -145,6 +168,207 @@ __device__ __forceinline__ void ts_g_chunk(TsTail* tail, uint8_t* base, int p0, 
   mma_commit(&tail->a_empty[ps]);
 }
 
+// ---- walker-side work ---------------------------------------------------------
+// The arithmetic is that of walker_tail.cuh.  Items are (8-coordinate chunk,
+// walker), the walker fastest.
+
+// Iteration `step`'s directions of items first, first + stride, ... < items, into
+// pair `to`; with a preconditioner the low-rank normals are in gs.
+__device__ __forceinline__ void ts_draw(const WalkerTail& t, int to, uint64_t seed, uint64_t step,
+                                        uint32_t walker0, int strip, int z, int w_begin,
+                                        int w_count, int first, int items, int stride,
+                                        const float* gs, uint4* state) {
+  using namespace tail_detail;
+  for (int it = first; it < items; it += stride) {
+    const int c = it / w_count, wo = it - c * w_count;
+    const int k = strip * kWalkers + w_begin + wo;
+    if (k >= z) continue;
+    const int i0 = 8 * c;
+    float v[8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (i0 + 4 * h < t.n) {
+        const U4 w = philox_block(seed, step, walker0 + static_cast<uint32_t>(k),
+                                  static_cast<uint32_t>(2 * c + h), kStreamDirection);
+        box_muller_f32(w.x, w.y, v[4 * h], v[4 * h + 1]);
+        box_muller_f32(w.z, w.w, v[4 * h + 2], v[4 * h + 3]);
+      } else {
+        v[4 * h] = v[4 * h + 1] = v[4 * h + 2] = v[4 * h + 3] = 0.0f;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (i0 + e >= t.n) v[e] = 0.0f;
+    float sg[8];
+    ld8(t.sigma + i0, sg);
+    if (t.pc_rank >= 0) {
+      // Rows of U four columns at a time, eight sums side by side (scalar
+      // loads, one sum after the other, took 14500 cycles an item).
+      float dl[8];
+      ld8(t.pc_delta + i0, dl);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] *= dl[e];
+      const float* g = gs + wo * kGStride;
+#pragma unroll 2
+      for (int c4 = 0; c4 < kMaxPcRank; c4 += 4) {
+        const float4 g4 = *reinterpret_cast<const float4*>(g + c4);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          if (i0 + e >= t.n) continue;
+          const float4 u = __ldg(reinterpret_cast<const float4*>(
+              t.pc_U + static_cast<size_t>(i0 + e) * kMaxPcRank + c4));
+          v[e] = fmaf(u.w, g4.w, fmaf(u.z, g4.z, fmaf(u.y, g4.y, fmaf(u.x, g4.x, v[e]))));
+        }
+      }
+    }
+    // The FP16 pair holds d_i / sigma_i (sigma a power of two: exact).
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] *= pow2_recip(sg[e]);
+    const size_t o = op_off(k, i0, t.k_pad, t.z_ld, 1);
+    uint4 h, l;
+    if (split8(v, h, l)) atomicOr(t.status, MHAR_ST_NONFINITE);
+    *reinterpret_cast<uint4*>(t.Dh[to] + o) = h;
+    *reinterpret_cast<uint4*>(t.Dl[to] + o) = l;
+    if (state != nullptr) {
+      state[(4 + 2 * to) * kEpiThreads + it] = h;
+      state[(5 + 2 * to) * kEpiThreads + it] = l;
+    }
+  }
+}
+
+// The low-rank normals of the CTA's walkers (Philox stream 2), by `threads` threads.
+__device__ __forceinline__ void ts_lowrank(const WalkerTail& t, uint64_t seed, uint64_t step,
+                                           uint32_t walker0, int strip, int z, int w_begin,
+                                           int w_count, int tid, int threads, float* gs) {
+  const int quads = (t.pc_rank + 3) >> 2;
+  for (int idx = tid; idx < w_count * (kMaxPcRank / 4); idx += threads) {
+    const int w = idx / (kMaxPcRank / 4), q = idx - w * (kMaxPcRank / 4);
+    const int k = strip * kWalkers + w_begin + w;
+    float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (q < quads && k < z) {
+      const U4 r = philox_block(seed, step, walker0 + static_cast<uint32_t>(k),
+                                static_cast<uint32_t>(q), kStreamLowRank);
+      box_muller_f32(r.x, r.y, v[0], v[1]);
+      box_muller_f32(r.z, r.w, v[2], v[3]);
+    }
+    float4 o;
+    o.x = 4 * q < t.pc_rank ? v[0] : 0.0f;
+    o.y = 4 * q + 1 < t.pc_rank ? v[1] : 0.0f;
+    o.z = 4 * q + 2 < t.pc_rank ? v[2] : 0.0f;
+    o.w = 4 * q + 3 < t.pc_rank ? v[3] : 0.0f;
+    *reinterpret_cast<float4*>(gs + w * kGStride + 4 * q) = o;
+  }
+}
+
+// Resident points: thread `tid`'s item into shared memory at the start, and
+// its direction of pair `cur`.
+__device__ __forceinline__ void ts_load_state(const WalkerTail& t, int cur, int strip, int z,
+                                              int w_begin, int w_count, int tid, uint4* state) {
+  const int c = tid / w_count, wo = tid - c * w_count, i0 = 8 * c;
+  const int k = strip * kWalkers + w_begin + wo;
+  if (i0 >= t.n || k >= z) return;
+  const size_t xr = static_cast<size_t>(k) * t.n_ld + i0;
+  const size_t o = op_off(k, i0, t.k_pad, t.z_ld, 1);
+  const uint4* hi = reinterpret_cast<const uint4*>(t.Xhi + xr);
+  const uint4* lo = reinterpret_cast<const uint4*>(t.Xlo + xr);
+  state[tid] = hi[0];
+  state[kEpiThreads + tid] = hi[1];
+  state[2 * kEpiThreads + tid] = lo[0];
+  state[3 * kEpiThreads + tid] = lo[1];
+  state[(4 + 2 * cur) * kEpiThreads + tid] = *reinterpret_cast<const uint4*>(t.Dh[cur] + o);
+  state[(5 + 2 * cur) * kEpiThreads + tid] = *reinterpret_cast<const uint4*>(t.Dl[cur] + o);
+}
+
+// The move and the split of resident points; `red` is zero at the start.
+// out: where the walker's sample goes (null: none).  save: the points go back
+// to global memory.
+__device__ __forceinline__ void ts_move_resident(const WalkerTail& t, int cur, int strip, int z,
+                                                 int w_begin, int w_count, int tid,
+                                                 const float* theta, unsigned int* red,
+                                                 uint4* state, double* out, int emit, bool save) {
+  using namespace tail_detail;
+  const int c = tid / w_count, wo = tid - c * w_count, i0 = 8 * c;
+  const int k = strip * kWalkers + w_begin + wo;
+  const bool mine = i0 < t.n && k < z;
+  float v[8] = {};
+  float hi[8] = {}, lo[8] = {};
+  if (mine) {
+    float sg[8];
+    if (!t.unit_sigma) ld8(t.sigma + i0, sg);
+    const float th = theta[w_begin + wo];
+    ld8(reinterpret_cast<const float*>(state + tid), hi, kEpiThreads);
+    ld8(reinterpret_cast<const float*>(state + 2 * kEpiThreads + tid), lo, kEpiThreads);
+    if (th != 0.0f) {
+      float dh[8], dl[8];
+      ld8h(reinterpret_cast<const __half*>(state + (4 + 2 * cur) * kEpiThreads + tid), dh);
+      ld8h(reinterpret_cast<const __half*>(state + (5 + 2 * cur) * kEpiThreads + tid), dl);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float d = t.unit_sigma ? dh[e] + dl[e] : (dh[e] + dl[e]) * sg[e];
+        df_axpy(hi[e], lo[e], th, i0 + e < t.n ? d : 0.0f);
+      }
+      st8(reinterpret_cast<float*>(state + tid), hi, kEpiThreads);
+      st8(reinterpret_cast<float*>(state + 2 * kEpiThreads + tid), lo, kEpiThreads);
+    }
+    float mx = 0.0f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {   // x = 0 and sigma = 1 past n
+      const float is = t.unit_sigma ? 1.0f : pow2_recip(sg[e]);
+      mx = fmaxf(mx, t.unit_sigma ? fabsf(hi[e]) : fabsf(hi[e]) * is);
+      v[e] = is;
+    }
+    atomicMax(red + wo, __float_as_uint(mx));  // non-negative floats order as their bits
+  }
+  named_bar<kEpiThreads>();
+  if (!mine) return;
+  const unsigned int mb = red[wo];
+  float inv, ws;
+  const int ex = static_cast<int>(mb >> 23) - 126;     // frexp's exponent of a normal value
+  if (mb >= 0x00800000u && ex >= -126 && ex <= 126) {
+    inv = __int_as_float((127 - ex) << 23);
+    ws = __int_as_float((127 + ex) << 23);
+  } else {
+    int e2 = 0;
+    if (mb > 0u) frexpf(__uint_as_float(mb), &e2);
+    inv = ldexpf(1.0f, -e2);
+    ws = ldexpf(1.0f, e2);
+  }
+  if (c == 0) t.wscale[k] = ws;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = t.unit_sigma ? (hi[e] + lo[e]) * inv : (hi[e] + lo[e]) * inv * v[e];
+  const size_t o = op_off(k, i0, t.k_pad, t.z_ld, 1);
+  if (split_store8(v, t.Xh + o, t.Xl + o)) atomicOr(t.status, MHAR_ST_NONFINITE);
+  if (out != nullptr && k < emit) {
+    double* row = out + static_cast<size_t>(k) * t.n + i0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (i0 + e < t.n) row[e] = static_cast<double>(hi[e]) + static_cast<double>(lo[e]);
+  }
+  if (save) {
+    const size_t xr = static_cast<size_t>(k) * t.n_ld + i0;
+    st8(t.Xhi + xr, hi);
+    st8(t.Xlo + xr, lo);
+  }
+}
+
+// Points too many for shared memory, and iterations with equalities:
+// walker_tail on the points in global memory.
+__device__ __forceinline__ void ts_move(const WalkerTail& wt, int cur, int strip, int z, int w_begin,
+                                        int w_count, int tid, TsTail* tail, uint8_t* stage) {
+  // Initialised: in the loop over the iterations an item that a thread does not
+  // have would be kept from one to the next (444 bytes of spills, with the
+  // like of it in the operands' second chunk).
+  TailItem item = {};   // this thread's first tail item
+  walker_tail_unstage<kEpiThreads>(wt, strip, z, w_begin, w_count, tid,
+                                   stage + tid * kTailStageBytes, item);
+  // The stage is free after the tail's first barrier: route the moved rows
+  // through it when they fit.
+  const bool rows_fit =
+      static_cast<size_t>(2 * w_count) * tail_row_stride(wt.n_ld) * sizeof(float) <= kStageBytes;
+  walker_tail<kEpiThreads>(wt, cur, strip, z, w_begin, w_count, tail->theta_s, tail->red, tid, item,
+                           rows_fit ? reinterpret_cast<float*>(stage) : nullptr);
+}
+
 // KCH: 64-column K chunks of A's rows (1 or 2: n <= 128); LAST: K steps (16
 // FP16 each) in the last chunk, 1..4, the other chunk having 4.  A
 // compile-time K structure makes each pass one straight run of MMAs (the
@@ -152,7 +376,7 @@ __device__ __forceinline__ void ts_g_chunk(TsTail* tail, uint8_t* base, int p0, 
 template <int KCH, int LAST>
 __global__ void __launch_bounds__(kThreadsTs, 1)
 recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
-                    const TsParams p) {
+                    const __grid_constant__ TsParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -160,8 +384,6 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
   uint8_t* stage = reinterpret_cast<uint8_t*>(tail + 1);   // 16-byte aligned
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  TailItem tail_item;  // the epilogue threads' first tail item
-  tail_item.valid = 0;
   const int csz_i = static_cast<int>(gridDim.x);
   const int share = (kWalkers + csz_i - 1) / csz_i;   // walkers of this CTA's walker-side work
   const int w_begin = static_cast<int>(blockIdx.x) * share;
@@ -183,6 +405,7 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
     mbar_init(&tail->p_empty, kEpiWarps);
     mbar_init(&tail->g_full, 1);
     mbar_init(&tail->g_empty, kEpiWarps);
+    mbar_init(&tail->c_full, 1);
     tail->timed_out = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -193,7 +416,8 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  __syncwarp();
+  cluster_sync_all();   // every CTA's barriers are ready
   tc_fence_after();
   const uint32_t tmem = tail->tmem_base;
   volatile int* timed_out = &tail->timed_out;
@@ -201,254 +425,288 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
   // the set-up above overlaps its end; nothing it wrote is read before this.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const uint64_t step = *p.step_ptr + static_cast<uint64_t>(p.j);
-  const int cur = static_cast<int>(step & 1ull);  // this iteration's direction pair
+  const uint64_t step0 = p.step_ptr != nullptr ? *p.step_ptr + static_cast<uint64_t>(p.j) : p.step0;
+  uint4* state = p.resident ? reinterpret_cast<uint4*>(stage) : nullptr;
+  const int tid = static_cast<int>(threadIdx.x) - 64;   // of the epilogue, then the draw threads
+  if (state != nullptr && warp >= 2 && warp < kDrawWarp)
+    ts_load_state(p.wt, static_cast<int>(step0 & 1ull), strip, p.z, w_begin, w_count, tid, state);
+  int pu = 0;                // producer: pair uses issued
+  int p0 = 0;                // MMA thread: first pair use of the tile
+  int g = 0;                 // tiles of the iterations before
+#pragma unroll 1
+  for (int it = 0; it < p.iters; ++it, g += ntiles) {
+    const uint64_t step = step0 + static_cast<uint64_t>(it);
+    const int cur = static_cast<int>(step & 1ull);  // this iteration's direction pair
 
-  // ---- walker operands into tensor memory: warp (quarter q, operand op) ------
-  // writes its 32 walkers' row of operand op, 2 FP16 per 32-bit column.
-  if (warp >= 2) {
-    const int e = warp - 2;
-    const int q = warp & 3;
-    const int op = e >> 2;
-    const int k = strip * kWalkers + q * 32 + lane;
-    const __half* src = op == 0 ? p.wt.Dh[cur] : op == 1 ? p.wt.Dl[cur] : op == 2 ? p.Xh : p.Xl;
-    // Operands are interleaved by 8-element chunks: chunk c of walker k is the
-    // 16 bytes at (c z_ld + k) 16, so each load below is one contiguous
-    // 512-byte line for the warp.
-    const uint4* ops = reinterpret_cast<const uint4*>(src);
-    const uint32_t col0 = kOpCol + static_cast<uint32_t>(op * 64);
-    const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
-    uint32_t r0[32], r1[32];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint4 v = __ldg(ops + static_cast<size_t>(i) * p.z_ld + k);
-      r0[4 * i] = v.x; r0[4 * i + 1] = v.y; r0[4 * i + 2] = v.z; r0[4 * i + 3] = v.w;
-    }
-    if (p.k_pad > 64) {
+    // ---- walker operands into tensor memory: warp (quarter q, operand op) ------
+    // writes its 32 walkers' row of operand op, 2 FP16 per 32-bit column.
+    if (warp >= 2 && warp < kDrawWarp) {
+      const int e = warp - 2;
+      const int q = warp & 3;
+      const int op = e >> 2;
+      const int k = strip * kWalkers + q * 32 + lane;
+      const __half* src = op == 0 ? p.wt.Dh[cur] : op == 1 ? p.wt.Dl[cur] : op == 2 ? p.Xh : p.Xl;
+      // Operands are interleaved by 8-element chunks: chunk c of walker k is the
+      // 16 bytes at (c z_ld + k) 16, so each load below is one contiguous
+      // 512-byte line for the warp.
+      const uint4* ops = reinterpret_cast<const uint4*>(src);
+      const uint32_t col0 = kOpCol + static_cast<uint32_t>(op * 64);
+      const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
+      uint32_t r0[32], r1[32];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const uint4 v = __ldg(ops + static_cast<size_t>(8 + i) * p.z_ld + k);
-        r1[4 * i] = v.x; r1[4 * i + 1] = v.y; r1[4 * i + 2] = v.z; r1[4 * i + 3] = v.w;
+        const uint4 v = __ldcg(ops + static_cast<size_t>(i) * p.z_ld + k);
+        r0[4 * i] = v.x; r0[4 * i + 1] = v.y; r0[4 * i + 2] = v.z; r0[4 * i + 3] = v.w;
       }
-    }
-    tmem_st32(tmem + lane_off + col0, r0);
-    if (p.k_pad > 64) tmem_st32(tmem + lane_off + col0 + 32u, r1);
-    tmem_st_wait();
-    tc_fence_before();
-    // Operands ready: release the MMA warp (the producer never waits on this).
-    asm volatile("bar.arrive 2, %0;" ::"n"((kEpiWarps + 1) * 32) : "memory");
-    if (op == 0 || op == 2) {
-      // The 2-norm bound of the walker's direction (op 0) or scaled point
-      // (op 2) from its FP16 hi row, for the chord's error margins.
-      // Sums of squares in chunk order: the same bits as operand_norms in the
-      // shared-memory-operand kernels.
-      float ss = 0.0f, mx = 0.0f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint4 u = make_uint4(r0[4 * i], r0[4 * i + 1], r0[4 * i + 2], r0[4 * i + 3]);
-        ss += sumsq8(u);
-        mx = fmaxf(mx, absmax8(u));
-      }
-      if (p.k_pad > 64) {
+      if constexpr (KCH == 2) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const uint4 u = make_uint4(r1[4 * i], r1[4 * i + 1], r1[4 * i + 2], r1[4 * i + 3]);
+          const uint4 v = __ldcg(ops + static_cast<size_t>(8 + i) * p.z_ld + k);
+          r1[4 * i] = v.x; r1[4 * i + 1] = v.y; r1[4 * i + 2] = v.z; r1[4 * i + 3] = v.w;
+        }
+      }
+      tmem_st32(tmem + lane_off + col0, r0);
+      if constexpr (KCH == 2) tmem_st32(tmem + lane_off + col0 + 32u, r1);
+      tmem_st_wait();
+      tc_fence_before();
+      // Operands ready: release the MMA warp (the producer never waits on this).
+      asm volatile("bar.arrive 2, %0;" ::"n"((kEpiWarps + 1) * 32) : "memory");
+      if (op == 0 || op == 2) {
+        // The 2-norm bound of the walker's direction (op 0) or scaled point
+        // (op 2) from its FP16 hi row, for the chord's error margins.
+        // Sums of squares in chunk order: the same bits as operand_norms in the
+        // shared-memory-operand kernels.
+        float ss = 0.0f, mx = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 u = make_uint4(r0[4 * i], r0[4 * i + 1], r0[4 * i + 2], r0[4 * i + 3]);
           ss += sumsq8(u);
           mx = fmaxf(mx, absmax8(u));
         }
-      }
-      tail->nrm[op >> 1][q * 32 + lane] = norm_bound(ss);
-      if (op == 0) tail->nrm[2][q * 32 + lane] = mx * 1.00390625f;
-    }
-  }
-
-  if (warp == 0) {
-    // ---- TMA producer: A rows, 64-row tiles, hi and lo in separate slots ------
-    if (lane == 0) {
-      int pu = 0;
-      for (int nt = 0; nt < ntiles; ++nt) {
-        const int yr = row_base + nt * kTile;
+        if constexpr (KCH == 2) {
 #pragma unroll
-        for (int kc = 0; kc < KCH; ++kc, ++pu) {
-          const int s = pu % kPairs;
+          for (int i = 0; i < 8; ++i) {
+            const uint4 u = make_uint4(r1[4 * i], r1[4 * i + 1], r1[4 * i + 2], r1[4 * i + 3]);
+            ss += sumsq8(u);
+            mx = fmaxf(mx, absmax8(u));
+          }
+        }
+        tail->nrm[op >> 1][q * 32 + lane] = norm_bound(ss);
+        if (op == 0) tail->nrm[2][q * 32 + lane] = mx * 1.00390625f;
+      }
+    }
+
+    if (warp == 0) {
+      // ---- TMA producer: A rows, 64-row tiles, hi and lo in separate slots ------
+      if (lane == 0) {
+        // This iteration's tiles and the first of the next one's, which then
+        // arrive while the walkers move.
+        const int per = ntiles * KCH;
+        const int end = min(p.iters * per, (it + 1) * per + kPairs);
+        for (; pu < end; ++pu) {
+          const int s = pu % kPairs, nt = (pu / KCH) % ntiles, kc = pu % KCH;
+          const int yr = row_base + nt * kTile;
           if (pu >= kPairs) mbar_wait(&tail->a_empty[s], ((pu / kPairs) - 1) & 1, timed_out, p.err);
           mbar_expect_tx(&tail->a_full[s], 2 * kSlotBytes);
           tma_load_2d(base + (2 * s) * kSlotBytes, &tm_ah, &tail->a_full[s], kc * kTcKChunk, yr);
           tma_load_2d(base + (2 * s + 1) * kSlotBytes, &tm_al, &tail->a_full[s], kc * kTcKChunk, yr);
         }
       }
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---- MMA issuer ------------------------------------------------------------
+      asm volatile("bar.sync 2, %0;" ::"n"((kEpiWarps + 1) * 32) : "memory");
+      tc_fence_after();
+      if (lane == 0) {
+        constexpr uint32_t idesc = make_idesc(kWalkers, kTile);
+        const uint32_t op_dh = tmem + kOpCol, op_dl = op_dh + 64u, op_xh = op_dh + 128u,
+                       op_xl = op_dh + 192u;
+        const uint32_t g_tmem = tmem;
+        const uint32_t p_tmem = tmem + 128u;
+        for (int nt = 0; nt < ntiles; ++nt, p0 += KCH) {
+          // P pass: X hi, X lo times A hi; X hi times A lo.  The accumulator is
+          // free once the epilogue has copied the previous tile's P out.
+          if (g + nt >= 1) mbar_wait(&tail->p_empty, (g + nt - 1) & 1, timed_out, p.err);
+          tc_fence_after();
+          if constexpr (KCH == 2)
+            ts_p_chunk<4>(tail, base, p0, 0, p_tmem, op_xh, op_xl, idesc, timed_out, p.err);
+          ts_p_chunk<LAST>(tail, base, p0, KCH - 1, p_tmem, op_xh, op_xl, idesc, timed_out, p.err);
+          mma_commit(&tail->p_full);
+          // G pass: D hi, D lo times A hi; D hi times A lo.  Each slot is
+          // released after its last use here.
+          if (g + nt >= 1) mbar_wait(&tail->g_empty, (g + nt - 1) & 1, timed_out, p.err);
+          tc_fence_after();
+          if constexpr (KCH == 2) ts_g_chunk<4>(tail, base, p0, 0, g_tmem, op_dh, op_dl, idesc);
+          ts_g_chunk<LAST>(tail, base, p0, KCH - 1, g_tmem, op_dh, op_dl, idesc);
+          mma_commit(&tail->g_full);
+        }
+      }
+      __syncwarp();
+    } else if (warp >= kDrawWarp) {
+      // ---- iteration s+1's directions into the other pair ------------------------
+      if (p.wt.draw) {
+        const int dt = tid - kEpiThreads;
+        const int items = ((p.wt.n + 7) >> 3) * w_count;
+        if (p.wt.pc_rank >= 0) {
+          ts_lowrank(p.wt, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count, dt,
+                     kDrawThreads, tail->gs);
+          if (p.epi_items > 0)
+            asm volatile("bar.sync 3, %0;" ::"n"(kEpiThreads + kDrawThreads) : "memory");
+          else
+            asm volatile("bar.sync 3, %0;" ::"n"(kDrawThreads) : "memory");
+        }
+        ts_draw(p.wt, cur ^ 1, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count,
+                p.epi_items + dt, items, kDrawThreads, tail->gs, state);
+      }
+    } else {
+      // ---- epilogue: s = b - p, ratios, per-walker partial chord ------------------
+      // First, while the first row tiles are on their way: iteration s+1's
+      // directions into the other pair (walker_tail.cuh, step 0).
+      const int e = warp - 2;
+      const int q = warp & 3;
+      const int cg = e >> 2;              // 32-column group of each 128-column tile
+      const int row0 = row_base + cg * 32;
+      if (lane < 4 && ntiles > 0) prefetch_l1(row_block(p.rows, row0) + 32 * lane);
+      if (tid == 0)
+        mbar_expect_tx(&tail->c_full, static_cast<uint32_t>(4 * csz_i * w_count * sizeof(float2)));
+      // This thread's walker-side item, copied to shared memory in the background.
+      if (state == nullptr)
+        walker_tail_stage<kEpiThreads>(p.wt, cur, strip, p.z, w_begin, w_count, tid,
+                                       stage + tid * kTailStageBytes);
+      if (tid < w_count) {
+        // The chord's uniform does not depend on the chord: draw it now.
+        const int kk = strip * kWalkers + w_begin + tid;
+        const U4 w = philox_block(p.seed, step, p.walker0 + static_cast<uint32_t>(kk), 0u,
+                                  kStreamChord);
+        tail->theta_u[tid] = open_unit_f64(w.x);
+        tail->red[tid] = 0u;
+      }
+      if (p.epi_items > 0) {
+        if (p.wt.pc_rank >= 0)
+          asm volatile("bar.sync 3, %0;" ::"n"(kEpiThreads + kDrawThreads) : "memory");
+        ts_draw(p.wt, cur ^ 1, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count, tid,
+                p.epi_items, kEpiThreads, tail->gs, state);
+      }
+      const int wl = q * 32 + lane;
+      const int k = strip * kWalkers + wl;
+      const float ws = __ldcg(p.wscale + k);
+      // The operand norms of this thread's walker (written by the warps that
+      // loaded the operands into tensor memory, before the draw above).
+      named_bar<kEpiWarps * 32>();
+      WalkerNorms wn;
+      wn.nd2 = tail->nrm[0][wl];
+      wn.nxw2 = ws * tail->nrm[1][wl];
+      wn.ws = ws;
+      wn.ndinf = tail->nrm[2][wl];
+      if (k < p.z) add_correction(p.wt, k, wn);
+      ChordAcc acc;
+      acc.init();
+      const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
+      const uint32_t gcol = tmem + lane_off + static_cast<uint32_t>(cg * 32);
+#pragma unroll 1
+      for (int nt = 0; nt < ntiles; ++nt) {
+        // P first (its pass ends first), then G; each accumulator is released
+        // as soon as it is in registers.
+        if (lane < 4 && nt + 1 < ntiles) prefetch_l1(row_block(p.rows, row0 + (nt + 1) * kTile) + 32 * lane);
+        float sv[32], gv[32];
+        mbar_wait(&tail->p_full, (g + nt) & 1, timed_out, p.err);
+        tc_fence_after();
+        tmem_ld32(gcol + 128u, sv);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive(&tail->p_empty);
+        // The slacks while the G pass finishes.
+        float fx, fd;
+        wn.pick(p.rows, row0 + nt * kTile, fx, fd);
+        slack32(sv, p.rows, row0 + nt * kTile, ws, fx);
+        mbar_wait(&tail->g_full, (g + nt) & 1, timed_out, p.err);
+        tc_fence_after();
+        tmem_ld32(gcol, gv);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive(&tail->g_empty);
+        scan32(sv, gv, p.rows, row0 + nt * kTile, fd, acc);
+      }
+      // The partial chord to the CTA that holds the walker: the data and its
+      // arrival in one message (a cluster barrier took 1500 cycles here).
+      {
+        const int owner = wl / share;
+        push2(&tail->recv[(4 * static_cast<int>(rank) + cg) * share + wl - owner * share],
+              &tail->c_full, static_cast<uint32_t>(owner), acc.lo_all(), acc.hi_all());
+      }
+      if (tid < w_count) {
+        mbar_wait(&tail->c_full, it & 1, timed_out, p.err);
+        const int kk = strip * kWalkers + w_begin + tid;
+        float L = -INFINITY, H = INFINITY;
+        for (int r = 0; r < 4 * csz_i; ++r) {
+          const float2 v = tail->recv[r * share + tid];
+          L = fmaxf(L, v.x);
+          H = fminf(H, v.y);
+        }
+        float t = 0.0f;
+        if (kk < p.z) {
+          int flag = 0;
+          if (isinf(L) || isinf(H)) {
+            flag = MHAR_ST_UNBOUNDED;
+          } else if (L > H) {
+            flag = MHAR_ST_STALL;
+          } else {
+            const double u = tail->theta_u[tid];
+            t = static_cast<float>(static_cast<double>(L) +
+                                   u * (static_cast<double>(H) - static_cast<double>(L)));
+          }
+          if (it + 1 == p.iters) {
+            p.lmin[kk] = L;
+            p.lmax[kk] = H;
+            p.theta[kk] = t;
+          }
+          if (flag) {
+            atomicOr(p.status, flag);
+            atomicAdd(&p.counters[flag == MHAR_ST_STALL ? 0 : 1], 1ull);
+          }
+        }
+        tail->theta_s[w_begin + tid] = t;
+      }
+      named_bar<kEpiThreads>();
+      // Algorithm 2's thinning: a sample after this iteration?
+      const int done = p.phase + it + 1;
+      double* out = p.out != nullptr && done % p.thin == 0
+                        ? p.out + static_cast<size_t>(done / p.thin - 1) * p.emit * p.n
+                        : nullptr;
+      if (state != nullptr) {
+        ts_move_resident(p.wt, cur, strip, p.z, w_begin, w_count, tid, tail->theta_s, tail->red,
+                         state, out, p.emit, it + 1 == p.iters);
+      } else {
+        ts_move(p.wt, cur, strip, p.z, w_begin, w_count, tid, tail, stage);
+        if (out != nullptr) {   // this CTA's walkers, a warp per row
+          named_bar<kEpiThreads>();
+          for (int w = warp - 2; w < w_count; w += kEpiWarps) {
+            const int kk = strip * kWalkers + w_begin + w;
+            if (kk >= p.emit) break;
+            const float* hi = p.wt.Xhi + static_cast<size_t>(kk) * p.wt.n_ld;
+            const float* lo = p.wt.Xlo + static_cast<size_t>(kk) * p.wt.n_ld;
+            for (int i = lane; i < p.n; i += 32)
+              out[static_cast<size_t>(kk) * p.n + i] =
+                  static_cast<double>(hi[i]) + static_cast<double>(lo[i]);
+          }
+        }
+      }
     }
+    // The cluster's points and directions, and this CTA's shared memory, are
+    // ready for the next iteration (at the end: no message is still under way).
+    tc_fence_before();
     __syncwarp();
-  } else if (warp == 1) {
-    // ---- MMA issuer ------------------------------------------------------------
-    asm volatile("bar.sync 2, %0;" ::"n"((kEpiWarps + 1) * 32) : "memory");
+    cluster_sync_all();
     tc_fence_after();
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc(kWalkers, kTile);
-      const uint32_t op_dh = tmem + kOpCol, op_dl = op_dh + 64u, op_xh = op_dh + 128u,
-                     op_xl = op_dh + 192u;
-      const uint32_t g_tmem = tmem;
-      const uint32_t p_tmem = tmem + 128u;
-      int p0 = 0;    // first pair use of the tile
-      for (int nt = 0; nt < ntiles; ++nt, p0 += KCH) {
-        // P pass: X hi, X lo times A hi; X hi times A lo.  The accumulator is
-        // free once the epilogue has copied the previous tile's P out.
-        if (nt >= 1) mbar_wait(&tail->p_empty, (nt - 1) & 1, timed_out, p.err);
-        tc_fence_after();
-        if constexpr (KCH == 2)
-          ts_p_chunk<4>(tail, base, p0, 0, p_tmem, op_xh, op_xl, idesc, timed_out, p.err);
-        ts_p_chunk<LAST>(tail, base, p0, KCH - 1, p_tmem, op_xh, op_xl, idesc, timed_out, p.err);
-        mma_commit(&tail->p_full);
-        // G pass: D hi, D lo times A hi; D hi times A lo.  Each slot is
-        // released after its last use here.
-        if (nt >= 1) mbar_wait(&tail->g_empty, (nt - 1) & 1, timed_out, p.err);
-        tc_fence_after();
-        if constexpr (KCH == 2) ts_g_chunk<4>(tail, base, p0, 0, g_tmem, op_dh, op_dl, idesc);
-        ts_g_chunk<LAST>(tail, base, p0, KCH - 1, g_tmem, op_dh, op_dl, idesc);
-        mma_commit(&tail->g_full);
-      }
-    }
-    __syncwarp();
-  } else {
-    // ---- epilogue: s = b - p, ratios, per-walker partial chord ------------------
-    // First, while the first row tiles are on their way: iteration s+1's
-    // directions into the other pair (walker_tail.cuh, step 0).
-    const int e = warp - 2;
-    const int q = warp & 3;
-    const int cg = e >> 2;              // 32-column group of each 128-column tile
-    const int row0 = row_base + cg * 32;
-    if (lane < 4 && ntiles > 0) prefetch_l1(row_block(p.rows, row0) + 32 * lane);
-    // This thread's walker-side item, copied to shared memory in the background.
-    walker_tail_stage<kEpiWarps * 32>(p.wt, cur, strip, p.z, w_begin, w_count,
-                                      static_cast<int>(threadIdx.x) - 64,
-                                      stage + (threadIdx.x - 64) * kTailStageBytes);
-    if (cg == 0) {
-      // The chord's uniform does not depend on the chord: draw it now.
-      const int kk = strip * kWalkers + q * 32 + lane;
-      const U4 w = philox_block(p.seed, step, p.walker0 + static_cast<uint32_t>(kk), 0u,
-                                kStreamChord);
-      tail->theta_u[q * 32 + lane] = open_unit_f64(w.x);
-    }
-    if (p.wt.draw)
-      walker_draw_next<kEpiWarps * 32>(p.wt, cur, p.seed, step + 1ull, p.walker0, strip, p.z,
-                                       w_begin, w_count, static_cast<int>(threadIdx.x) - 64,
-                                       tail->gs);
-    const int wl = q * 32 + lane;
-    const int k = strip * kWalkers + wl;
-    const float ws = p.wscale[k];
-    // The operand norms of this thread's walker (written by the warps that
-    // loaded the operands into tensor memory, before the draw above).
-    named_bar<kEpiWarps * 32>();
-    WalkerNorms wn;
-    wn.nd2 = tail->nrm[0][wl];
-    wn.nxw2 = ws * tail->nrm[1][wl];
-    wn.ws = ws;
-    wn.ndinf = tail->nrm[2][wl];
-    if (k < p.z) add_correction(p.wt, k, wn);
-    ChordAcc acc;
-    acc.init();
-    const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
-    const uint32_t gcol = tmem + lane_off + static_cast<uint32_t>(cg * 32);
-    for (int nt = 0; nt < ntiles; ++nt) {
-      // P first (its pass ends first), then G; each accumulator is released
-      // as soon as it is in registers.
-      if (lane < 4 && nt + 1 < ntiles) prefetch_l1(row_block(p.rows, row0 + (nt + 1) * kTile) + 32 * lane);
-      float sv[32], gv[32];
-      mbar_wait(&tail->p_full, nt & 1, timed_out, p.err);
-      tc_fence_after();
-      tmem_ld32(gcol + 128u, sv);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) arrive(&tail->p_empty);
-      // The slacks while the G pass finishes.
-      float fx, fd;
-      wn.pick(p.rows, row0 + nt * kTile, fx, fd);
-      slack32(sv, p.rows, row0 + nt * kTile, ws, fx);
-      mbar_wait(&tail->g_full, nt & 1, timed_out, p.err);
-      tc_fence_after();
-      tmem_ld32(gcol, gv);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) arrive(&tail->g_empty);
-      scan32(sv, gv, p.rows, row0 + nt * kTile, fd, acc);
-    }
-    const float lo = acc.lo_all(), hi = acc.hi_all();
-    tail->part_lo[cg][wl] = lo;
-    tail->part_hi[cg][wl] = hi;
-    named_bar<kEpiWarps * 32>();
-    if (cg == 0) {
-      const float L = fmaxf(fmaxf(lo, tail->part_lo[1][wl]), fmaxf(tail->part_lo[2][wl], tail->part_lo[3][wl]));
-      const float H = fminf(fminf(hi, tail->part_hi[1][wl]), fminf(tail->part_hi[2][wl], tail->part_hi[3][wl]));
-      // Every CTA of the cluster gets every partial: each then knows the
-      // strip's chords and theta without a second barrier.
-      for (uint32_t r = 0; r < gridDim.x; ++r) {
-        st_dsmem(&tail->recv_lo[rank][wl], r, L);
-        st_dsmem(&tail->recv_hi[rank][wl], r, H);
-      }
-    }
   }
 
-  // Every push is visible after this barrier; no remote access follows it.
-  // Between its arrive and its wait the epilogue reads its first tail item
-  // back from shared memory (staged at kernel start; it does not depend on
-  // theta).
-  tc_fence_before();
-  cluster_arrive();
-  if (warp >= 2)
-    walker_tail_unstage<kEpiWarps * 32>(p.wt, strip, p.z, w_begin, w_count,
-                                        static_cast<int>(threadIdx.x) - 64,
-                                        stage + (threadIdx.x - 64) * kTailStageBytes, tail_item);
-  cluster_wait();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
                  : "memory");
   }
-
-  if (warp >= 2 && ((warp - 2) >> 2) == 0) {
-    const int q = warp & 3;
-    const int wl = q * 32 + lane;
-    const int k = strip * kWalkers + wl;
-    float L = -INFINITY, H = INFINITY;
-    for (uint32_t r = 0; r < gridDim.x; ++r) {
-      L = fmaxf(L, tail->recv_lo[r][wl]);
-      H = fminf(H, tail->recv_hi[r][wl]);
-    }
-    if (k >= p.z) tail->theta_s[wl] = 0.0f;
-    if (k < p.z) {
-      float t = 0.0f;
-      int flag = 0;
-      if (isinf(L) || isinf(H)) {
-        flag = MHAR_ST_UNBOUNDED;
-      } else if (L > H) {
-        flag = MHAR_ST_STALL;
-      } else {
-        const double u = tail->theta_u[wl];
-        t = static_cast<float>(static_cast<double>(L) +
-                               u * (static_cast<double>(H) - static_cast<double>(L)));
-      }
-      tail->theta_s[wl] = t;
-      if (rank == 0) {
-        p.lmin[k] = L;
-        p.lmax[k] = H;
-        p.theta[k] = t;
-        if (flag) {
-          atomicOr(p.status, flag);
-          atomicAdd(&p.counters[flag == MHAR_ST_STALL ? 0 : 1], 1ull);
-        }
-      }
-    }
-  }
-  if (warp >= 2) {
-    named_bar<kEpiWarps * 32>();
-    // The stage is free again (its items are in registers): route the moved
-    // rows through it when they fit.
-    const bool rows_fit = static_cast<size_t>(2 * w_count) * tail_row_stride(p.wt.n_ld) *
-                              sizeof(float) <= kStageBytes;
-    walker_tail<kEpiWarps * 32>(p.wt, cur, strip, p.z, w_begin, w_count, tail->theta_s,
-                                tail->red, static_cast<int>(threadIdx.x) - 64, tail_item,
-                                rows_fit ? reinterpret_cast<float*>(stage) : nullptr);
-  }
+  if (p.step_out != nullptr && threadIdx.x == 0 && rank == 0 && strip == 0)
+    *p.step_out = step0 + static_cast<uint64_t>(p.iters);
 }
 
 struct TsShape {
@@ -502,7 +760,9 @@ int ts_prepare(mhar_ctx* c) {
   return MHAR_OK;
 }
 
-cudaError_t launch_recompute_ts(mhar_ctx* c, int j) {
+namespace {
+
+cudaError_t launch_ts(mhar_ctx* c, int j, const SmallRun* r) {
   const TcPlan* plan = static_cast<const TcPlan*>(c->tc);
   const TsShape s = ts_shape(c, plan);
   TsParams p;
@@ -516,7 +776,15 @@ cudaError_t launch_recompute_ts(mhar_ctx* c, int j) {
   p.status = c->d.status;
   p.counters = c->d.counters;
   p.err = c->d.status + 1;
-  p.step_ptr = c->d.step;
+  p.step_ptr = r ? nullptr : c->d.step;
+  p.step_out = r ? c->d.step : nullptr;
+  p.step0 = r ? r->step : 0;
+  p.iters = r ? r->iters : 1;
+  p.out = r ? r->out : nullptr;
+  p.emit = r ? r->emit : 0;
+  p.thin = r ? r->thin : 1;
+  p.phase = r ? r->phase : 0;
+  p.n = c->n;
   p.seed = c->opts.seed;
   p.j = j;
   p.walker0 = c->opts.walker0;
@@ -528,6 +796,20 @@ cudaError_t launch_recompute_ts(mhar_ctx* c, int j) {
   p.tiles_per_cta = s.tiles_per_cta;
   p.m_tiles = s.m_tiles;
   p.wt = make_walker_tail(c, 1, true);
+  const int share = (kWalkers + s.C - 1) / s.C, items = (c->n + 7) / 8 * share;
+  p.resident = r && items <= kEpiThreads ? 1 : 0;
+  // What the draw warps get done beside the tiles: about 100 cycles an MMA (six
+  // per K step) and 8000 of the rest of an iteration, against 1250 cycles a
+  // round of 64 items, 1000 more with U g and 600 a round of low-rank normals.
+  // The epilogue warps draw what is left, before their first tile (4800 cycles
+  // for 416 items).
+  int cycles = s.tiles_per_cta * (p.kdim / kTcK) * 600 + 8000, round = 1250;
+  if (c->pc_rank >= 0) {
+    cycles -= (share * (kMaxPcRank / 4) + kDrawThreads - 1) / kDrawThreads * 600;
+    round += 1000;
+  }
+  const int rounds = cycles > 0 ? cycles / round : 0;
+  p.epi_items = p.wt.draw && rounds * kDrawThreads < items ? items - rounds * kDrawThreads : 0;
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.C, plan->strips, 1);
@@ -548,5 +830,11 @@ cudaError_t launch_recompute_ts(mhar_ctx* c, int j) {
   const TsKernel k = kTsKernels[4 * (p.k_chunks - 1) + last_chunk_steps(p.kdim, p.k_chunks) - 1];
   return cudaLaunchKernelEx(&cfg, k, plan->ah64, plan->al64, p);
 }
+
+}  // namespace
+
+cudaError_t launch_recompute_ts(mhar_ctx* c, int j) { return launch_ts(c, j, nullptr); }
+
+cudaError_t launch_recompute_ts_run(mhar_ctx* c, const SmallRun& r) { return launch_ts(c, 0, &r); }
 
 }  // namespace mhar

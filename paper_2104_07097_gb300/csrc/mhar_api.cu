@@ -329,26 +329,32 @@ int capture(mhar_ctx* c, int count, cudaGraphExec_t* out) {
   return MHAR_OK;
 }
 
-// Small bodies: `count` iterations from iteration c->step, at most kSmallIters a
-// launch so that none runs for long.  out (device, may be null): the samples,
-// as SmallRun has them, with `phase` iterations since the last one done before.
-constexpr int kSmallIters = 1024;
+// Whether one launch runs many iterations: small bodies, and the
+// tensor-memory-operand kernel when nothing comes between its iterations.
+bool loops(const mhar_ctx* c) { return c->use_small || (c->use_ts && tail_draws(c)); }
 
-int advance_small(mhar_ctx* c, int64_t count, double* out, int64_t thin, int64_t phase) {
-  for (int64_t at = 0; at < count; at += kSmallIters) {
+// `count` iterations from iteration c->step, at most kLoopIters a launch so that
+// none runs for long.  out (device, may be null): the samples, as SmallRun has
+// them, with `phase` iterations since the last one done before.
+int advance_loop(mhar_ctx* c, int64_t count, double* out, int64_t thin, int64_t phase) {
+  const int most = c->use_small ? 1024 : 256;
+  int rc = ensure_operands(c);
+  if (rc) return rc;
+  for (int64_t at = 0; at < count; at += most) {
     mhar::SmallRun r;
     r.step = c->step + static_cast<uint64_t>(at);
-    r.iters = static_cast<int>(std::min<int64_t>(kSmallIters, count - at));
+    r.iters = static_cast<int>(std::min<int64_t>(most, count - at));
     // A sample falls into this launch, and the indices fit.
     const int64_t since = out ? (phase + at) % thin : 0;
     if (out && since + r.iters >= thin) {
-      const int64_t wide = 2 * kSmallIters;   // one sample at most when thin is longer
+      const int64_t wide = 2 * most;   // one sample at most when thin is longer
       r.thin = static_cast<int>(std::min(thin, wide));
       r.phase = static_cast<int>(r.thin - (thin - since));
       r.emit = emit_count(c);
       r.out = out + static_cast<size_t>((phase + at) / thin) * r.emit * c->n;
     }
-    MHAR_CUDA(mhar::launch_small(c, r), "iteration kernel");
+    MHAR_CUDA(c->use_small ? mhar::launch_small(c, r) : mhar::launch_recompute_ts_run(c, r),
+              "iteration kernel");
     ++c->launches;
   }
   return MHAR_OK;
@@ -1131,18 +1137,18 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
   const int64_t au = c->opts.audit_every;
   while (done < steps) {
     int64_t adv = steps - done;
-    // The small-body kernel writes samples itself: all of a call's when they
-    // stay on the device, else one to the staging buffer at a time.
-    const bool fused = c->use_small && nsamp > 0;
+    // A kernel that runs many iterations writes samples itself: all of a call's
+    // when they stay on the device, else one to the staging buffer at a time.
+    const bool fused = loops(c) && nsamp > 0;
     const bool whole = fused && c->opts.out_on_device;
     if (thin > 0 && !whole) adv = std::min<int64_t>(adv, thin - (done % thin));
     if (k > 0) adv = std::min<int64_t>(adv, k - c->since_refresh);
     if (au > 0) adv = std::min<int64_t>(adv, au - c->since_audit);
-    if (c->use_small) {
+    if (loops(c)) {
       double* to = !fused ? nullptr : whole
                        ? out + static_cast<size_t>(done / thin) * emit_count(c) * c->n
                        : c->d.emit;
-      rc = advance_small(c, adv, to, thin, fused ? done % thin : 0);
+      rc = advance_loop(c, adv, to, thin, fused ? done % thin : 0);
     } else {
       rc = advance(c, adv);
     }
@@ -1443,7 +1449,7 @@ int mhar_time_kernels(mhar_ctx* c, int iters, double* ms) {
   if (orc) return orc;
   // (1) `iters` real iterations, replayed back to back from one graph.
   auto full = [&]() -> cudaError_t {
-    if (c->use_small) return advance_small(c, iters, nullptr, 0, 0) ? cudaErrorUnknown : cudaSuccess;
+    if (loops(c)) return advance_loop(c, iters, nullptr, 0, 0) ? cudaErrorUnknown : cudaSuccess;
     for (int it = 0; it < iters; ++it) {
       cudaError_t e = enqueue_directions(c, it);
       if (e == cudaSuccess) e = enqueue_chord(c, it);
@@ -1463,7 +1469,7 @@ int mhar_time_kernels(mhar_ctx* c, int iters, double* ms) {
   float t_full = 0.f, t_dir = 0.f, t_ref = 0.f;
   cudaError_t e = time_graph(c, full, &t_full);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel timing");
-  if (!c->use_small) c->launches += static_cast<int64_t>(iters) * kernels_per_iteration(c) + 1;
+  if (!loops(c)) c->launches += static_cast<int64_t>(iters) * kernels_per_iteration(c) + 1;
   c->step += static_cast<uint64_t>(iters);
   if (!tail_draws(c) && !c->use_small) {  // otherwise the draw is part of the chord kernel
     e = time_graph(c, dirs, &t_dir);

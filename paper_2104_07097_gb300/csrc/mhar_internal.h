@@ -299,5 +299,7 @@ cudaError_t launch_recompute_sk(mhar_ctx* ctx, int j);
 bool ts_eligible(const mhar_ctx* ctx);              // n <= 128
 int ts_prepare(mhar_ctx* ctx);
 cudaError_t launch_recompute_ts(mhar_ctx* ctx, int j);
+// r.iters iterations in one launch (the draw is part of the chord kernel).
+cudaError_t launch_recompute_ts_run(mhar_ctx* ctx, const SmallRun& r);
 
 }  // namespace mhar

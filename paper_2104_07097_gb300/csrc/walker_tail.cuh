@@ -46,8 +46,8 @@ struct WalkerTail {
   const float* corrn;    // z or null: ||Q^T corr / sigma||_2 of each walker's direction
   int mE, n, n_ld, k_pad, z_ld, inter, draw;
   int unit_sigma;        // 1: every sigma_i is 1, skip them
-  // Preconditioned draw d = delta .* h + U g (pc_rank >= 0; only kernels that
-  // pass shared scratch for g to walker_draw_next draw it themselves).
+  // Preconditioned draw d = delta .* h + U g (pc_rank >= 0; only the
+  // tensor-memory-operand kernel draws it itself).
   const float* pc_delta; // n_ld
   const float* pc_U;     // n_ld x 32, zero beyond the rank
   int pc_rank;
@@ -88,14 +88,15 @@ inline WalkerTail make_walker_tail(const mhar_ctx* c, int inter, bool pc_draw = 
 
 namespace tail_detail {
 
-__device__ __forceinline__ void ld8(const float* p, float* v) {
+// `next`: the second four follow at that many float4s past the first.
+__device__ __forceinline__ void ld8(const float* p, float* v, int next = 1) {
   const float4 a = *reinterpret_cast<const float4*>(p);
-  const float4 b = *reinterpret_cast<const float4*>(p + 4);
+  const float4 b = *reinterpret_cast<const float4*>(p + 4 * next);
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
-__device__ __forceinline__ void st8(float* p, const float* v) {
+__device__ __forceinline__ void st8(float* p, const float* v, int next = 1) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-  *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+  *reinterpret_cast<float4*>(p + 4 * next) = make_float4(v[4], v[5], v[6], v[7]);
 }
 __device__ __forceinline__ void ld8h(const __half* p, float* v) {
   const uint4 u = *reinterpret_cast<const uint4*>(p);
@@ -106,9 +107,9 @@ __device__ __forceinline__ void ld8h(const __half* p, float* v) {
     v[2 * e + 1] = __half2float(__ushort_as_half(static_cast<unsigned short>(w[e] >> 16)));
   }
 }
-// Splits 8 values into FP16 hi / lo halves and stores both 16-byte chunks;
-// true if a value is non-finite or beyond the FP16 range.
-__device__ __forceinline__ bool split_store8(const float* v, __half* hi_dst, __half* lo_dst) {
+// Splits 8 values into FP16 hi / lo halves; true if a value is non-finite or
+// beyond the FP16 range.
+__device__ __forceinline__ bool split8(const float* v, uint4& hi, uint4& lo) {
   uint32_t h[4], l[4];
   bool bad = false;
 #pragma unroll
@@ -122,8 +123,16 @@ __device__ __forceinline__ bool split_store8(const float* v, __half* hi_dst, __h
     h[e] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
     l[e] = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
   }
-  *reinterpret_cast<uint4*>(hi_dst) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(lo_dst) = make_uint4(l[0], l[1], l[2], l[3]);
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+  return bad;
+}
+// The same, stored as both 16-byte chunks.
+__device__ __forceinline__ bool split_store8(const float* v, __half* hi_dst, __half* lo_dst) {
+  uint4 h, l;
+  const bool bad = split8(v, h, l);
+  *reinterpret_cast<uint4*>(hi_dst) = h;
+  *reinterpret_cast<uint4*>(lo_dst) = l;
   return bad;
 }
 
@@ -269,39 +278,17 @@ __device__ __forceinline__ void walker_tail_unstage(const WalkerTail& t, int str
   r.valid = 1;
 }
 
-// (0): run by kThreads threads (tid = 0..kThreads-1, sharing named barrier 1
-// when preconditioned); `next_step` = s + 1.  With a preconditioner the
-// direction is d = delta .* h + U g, g the walker's rank-r normals (Philox
-// stream 2), kept in `gs` (w_count x 32 floats of shared memory); the
-// arithmetic is that of precondition_kernel (FP32, terms in column order,
-// then d / sigma split into the FP16 pair).
+// (0): run by kThreads threads (tid = 0..kThreads-1); `next_step` = s + 1.  (The
+// tensor-memory-operand kernel has its own, with the preconditioner.)
 template <int kThreads>
 __device__ void walker_draw_next(const WalkerTail& t, int cur, uint64_t seed, uint64_t next_step,
                                  uint32_t walker0, int strip, int z, int w_begin, int w_count,
-                                 int tid, float* gs = nullptr) {
+                                 int tid) {
   using namespace tail_detail;
   const int chunks = (t.n + 7) >> 3;
   const int items = w_count * chunks;
   __half* Dh = t.Dh[cur ^ 1];
   __half* Dl = t.Dl[cur ^ 1];
-  const bool pre = t.pc_rank >= 0 && gs != nullptr;
-  if (pre) {
-    const int quads = (t.pc_rank + 3) >> 2;
-    for (int idx = tid; idx < w_count * (kMaxPcRank / 4); idx += kThreads) {
-      const int w = idx / (kMaxPcRank / 4), q = idx - w * (kMaxPcRank / 4);
-      const int k = strip * tc::kWalkers + w_begin + w;
-      float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      if (q < quads && k < z) {
-        const U4 r = philox_block(seed, next_step, walker0 + static_cast<uint32_t>(k),
-                                  static_cast<uint32_t>(q), kStreamLowRank);
-        box_muller_f32(r.x, r.y, v[0], v[1]);
-        box_muller_f32(r.z, r.w, v[2], v[3]);
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) gs[w * kMaxPcRank + 4 * q + e] = 4 * q + e < t.pc_rank ? v[e] : 0.0f;
-    }
-    tc::named_bar<kThreads>();
-  }
   for (int it = tid; it < items; it += kThreads) {
     const int c = it / w_count, wo = it - c * w_count;
     const int k = strip * tc::kWalkers + w_begin + wo;
@@ -323,23 +310,10 @@ __device__ void walker_draw_next(const WalkerTail& t, int cur, uint64_t seed, ui
 #pragma unroll
     for (int e = 0; e < 8; ++e)
       if (i0 + e >= t.n) v[e] = 0.0f;
-    if (!pre && !t.unit_sigma) {
+    if (!t.unit_sigma) {
       // The FP16 pair holds d_i / sigma_i (sigma a power of two: exact).
 #pragma unroll
       for (int e = 0; e < 8; ++e) v[e] *= pow2_recip(t.sigma[i0 + e]);
-    }
-    if (pre) {
-      const float* g = gs + wo * kMaxPcRank;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int i = i0 + e;
-        if (i >= t.n) continue;
-        const float* u = t.pc_U + static_cast<size_t>(i) * kMaxPcRank;
-        float acc = t.pc_delta[i] * v[e];
-#pragma unroll 8
-        for (int c2 = 0; c2 < kMaxPcRank; ++c2) acc = fmaf(u[c2], g[c2], acc);
-        v[e] = acc * pow2_recip(t.sigma[i]);
-      }
     }
     if (split_store8(v, Dh + o, Dl + o)) atomicOr(t.status, MHAR_ST_NONFINITE);
   }
@@ -377,7 +351,7 @@ __device__ void walker_tail(const WalkerTail& t, int cur, int strip, int z, int 
     const size_t xr = static_cast<size_t>(k) * t.n_ld + i0;
     const float th = theta_s[w_begin + wo];
     const bool cached = it == tid && first.valid;
-    float hi[8], lo[8], d[8];
+    float hi[8], lo[8], d[8] = {};
     if (cached) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) { hi[e] = first.hi[e]; lo[e] = first.lo[e]; d[e] = first.d[e]; }
