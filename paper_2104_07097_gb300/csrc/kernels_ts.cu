@@ -37,7 +37,9 @@
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstdio>
+#include <type_traits>
 
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
@@ -82,7 +84,7 @@ struct TsParams {
   int emit, thin, phase;
   uint32_t walker0;
   int resident;             // the walkers' points stay in shared memory (TsState)
-  int epi_items;            // draw items that the epilogue warps take
+  int draw_chunks;          // 8-coordinate chunks that the draw warps take; the epilogue warps the rest
   int n, z, z_ld, kdim, k_chunks, k_pad, tiles_per_cta, m_tiles;
   WalkerTail wt;            // walker-side work (walker_tail.cuh)
 };
@@ -106,6 +108,8 @@ struct alignas(16) TsTail {
   double theta_u[kWalkers];           // the chord's uniform u (Philox stream 1), drawn early
   unsigned int red[kWalkers];         // this CTA's walkers: largest |x / sigma| (bits)
   float nrm[3][kWalkers];             // each walker's ||d_hat||_2, ||x_hat||_2, max |d_hat|
+  alignas(16) float sigma[kWalkers];  // coordinate scales, and delta of a preconditioner
+  alignas(16) float delta[kWalkers];
   alignas(16) float gs[kWalkers * kGStride];   // low-rank normals of a preconditioned draw
 };
 
@@ -172,66 +176,70 @@ __device__ __forceinline__ void ts_g_chunk(TsTail* tail, uint8_t* base, int p0, 
 // The arithmetic is that of walker_tail.cuh.  Items are (8-coordinate chunk,
 // walker), the walker fastest.
 
-// Iteration `step`'s directions of items first, first + stride, ... < items, into
-// pair `to`; with a preconditioner the low-rank normals are in gs.
+// Iteration `step`'s directions into pair `to`: the items (group of 4 Q
+// coordinates, walker), the walker fastest, first, first + stride, ... < last; with
+// a preconditioner the low-rank normals are in gs.
+template <int Q>
 __device__ __forceinline__ void ts_draw(const WalkerTail& t, int to, uint64_t seed, uint64_t step,
                                         uint32_t walker0, int strip, int z, int w_begin,
-                                        int w_count, int first, int items, int stride,
-                                        const float* gs, uint4* state) {
+                                        int w_count, int first, int last, int stride,
+                                        const TsTail* tail, uint4* state) {
   using namespace tail_detail;
-  for (int it = first; it < items; it += stride) {
+  using Vec = std::conditional_t<Q == 2, uint4, uint2>;
+#pragma unroll 1
+  for (int it = first; it < last; it += stride) {
     const int c = it / w_count, wo = it - c * w_count;
     const int k = strip * kWalkers + w_begin + wo;
     if (k >= z) continue;
-    const int i0 = 8 * c;
-    float v[8];
+    const int i0 = 4 * Q * c;
+    float v[4 * Q] = {};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < Q; ++h)
       if (i0 + 4 * h < t.n) {
         const U4 w = philox_block(seed, step, walker0 + static_cast<uint32_t>(k),
-                                  static_cast<uint32_t>(2 * c + h), kStreamDirection);
+                                  static_cast<uint32_t>(Q * c + h), kStreamDirection);
         box_muller_f32(w.x, w.y, v[4 * h], v[4 * h + 1]);
         box_muller_f32(w.z, w.w, v[4 * h + 2], v[4 * h + 3]);
-      } else {
-        v[4 * h] = v[4 * h + 1] = v[4 * h + 2] = v[4 * h + 3] = 0.0f;
       }
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (i0 + e >= t.n) v[e] = 0.0f;
-    float sg[8];
-    ld8(t.sigma + i0, sg);
     if (t.pc_rank >= 0) {
-      // Rows of U four columns at a time, eight sums side by side (scalar
-      // loads, one sum after the other, took 14500 cycles an item).
-      float dl[8];
-      ld8(t.pc_delta + i0, dl);
+      // Rows of U four columns at a time, the sums side by side (scalar loads,
+      // one sum after the other, took 14500 cycles for eight).
+      const float* g = tail->gs + wo * kGStride;
+      const float4* u4 = reinterpret_cast<const float4*>(t.pc_U + static_cast<size_t>(i0) * kMaxPcRank);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] *= dl[e];
-      const float* g = gs + wo * kGStride;
+      for (int e = 0; e < 4 * Q; ++e) v[e] *= tail->delta[i0 + e];
 #pragma unroll 2
-      for (int c4 = 0; c4 < kMaxPcRank; c4 += 4) {
-        const float4 g4 = *reinterpret_cast<const float4*>(g + c4);
+      for (int c4 = 0; c4 < kMaxPcRank / 4; ++c4) {
+        const float4 g4 = *reinterpret_cast<const float4*>(g + 4 * c4);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          if (i0 + e >= t.n) continue;
-          const float4 u = __ldg(reinterpret_cast<const float4*>(
-              t.pc_U + static_cast<size_t>(i0 + e) * kMaxPcRank + c4));
+        for (int e = 0; e < 4 * Q; ++e) {      // rows of U up to n_ld, zero past n
+          const float4 u = __ldg(u4 + e * (kMaxPcRank / 4) + c4);
           v[e] = fmaf(u.w, g4.w, fmaf(u.z, g4.z, fmaf(u.y, g4.y, fmaf(u.x, g4.x, v[e]))));
         }
       }
     }
     // The FP16 pair holds d_i / sigma_i (sigma a power of two: exact).
+    alignas(16) __half2 h[2 * Q];
+    alignas(16) __half2 l[2 * Q];
+    bool bad = false;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] *= pow2_recip(sg[e]);
+    for (int e = 0; e < 4 * Q; e += 2) {
+      const float a = i0 + e < t.n ? v[e] * pow2_recip(tail->sigma[i0 + e]) : 0.0f;
+      const float b = i0 + e + 1 < t.n ? v[e + 1] * pow2_recip(tail->sigma[i0 + e + 1]) : 0.0f;
+      h[e / 2] = __floats2half2_rn(a, b);
+      l[e / 2] = __floats2half2_rn(a - __low2float(h[e / 2]), b - __high2float(h[e / 2]));
+      bad |= !(fabsf(a) <= kHalfMax) || !(fabsf(b) <= kHalfMax);
+    }
+    if (bad) atomicOr(t.status, MHAR_ST_NONFINITE);
+    const Vec hv = *reinterpret_cast<const Vec*>(h), lv = *reinterpret_cast<const Vec*>(l);
     const size_t o = op_off(k, i0, t.k_pad, t.z_ld, 1);
-    uint4 h, l;
-    if (split8(v, h, l)) atomicOr(t.status, MHAR_ST_NONFINITE);
-    *reinterpret_cast<uint4*>(t.Dh[to] + o) = h;
-    *reinterpret_cast<uint4*>(t.Dl[to] + o) = l;
+    *reinterpret_cast<Vec*>(t.Dh[to] + o) = hv;
+    *reinterpret_cast<Vec*>(t.Dl[to] + o) = lv;
     if (state != nullptr) {
-      state[(4 + 2 * to) * kEpiThreads + it] = h;
-      state[(5 + 2 * to) * kEpiThreads + it] = l;
+      Vec* part = reinterpret_cast<Vec*>(state + (4 + 2 * to) * kEpiThreads + (i0 >> 3) * w_count + wo);
+      const int half = Q == 2 ? 0 : c & 1;
+      part[half] = hv;
+      part[(2 / Q) * kEpiThreads + half] = lv;
     }
   }
 }
@@ -283,19 +291,20 @@ __device__ __forceinline__ void ts_load_state(const WalkerTail& t, int cur, int 
 // out: where the walker's sample goes (null: none).  save: the points go back
 // to global memory.
 __device__ __forceinline__ void ts_move_resident(const WalkerTail& t, int cur, int strip, int z,
-                                                 int w_begin, int w_count, int tid,
-                                                 const float* theta, unsigned int* red,
-                                                 uint4* state, double* out, int emit, bool save) {
+                                                 int w_begin, int c, int wo, int tid,
+                                                 TsTail* tail, uint4* state, double* out, int emit,
+                                                 bool save) {
   using namespace tail_detail;
-  const int c = tid / w_count, wo = tid - c * w_count, i0 = 8 * c;
+  const int i0 = 8 * c;
+  unsigned int* red = tail->red;
   const int k = strip * kWalkers + w_begin + wo;
   const bool mine = i0 < t.n && k < z;
   float v[8] = {};
   float hi[8] = {}, lo[8] = {};
   if (mine) {
     float sg[8];
-    if (!t.unit_sigma) ld8(t.sigma + i0, sg);
-    const float th = theta[w_begin + wo];
+    ld8(tail->sigma + i0, sg);
+    const float th = tail->theta_s[w_begin + wo];
     ld8(reinterpret_cast<const float*>(state + tid), hi, kEpiThreads);
     ld8(reinterpret_cast<const float*>(state + 2 * kEpiThreads + tid), lo, kEpiThreads);
     if (th != 0.0f) {
@@ -304,8 +313,7 @@ __device__ __forceinline__ void ts_move_resident(const WalkerTail& t, int cur, i
       ld8h(reinterpret_cast<const __half*>(state + (5 + 2 * cur) * kEpiThreads + tid), dl);
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        const float d = t.unit_sigma ? dh[e] + dl[e] : (dh[e] + dl[e]) * sg[e];
-        df_axpy(hi[e], lo[e], th, i0 + e < t.n ? d : 0.0f);
+        df_axpy(hi[e], lo[e], th, i0 + e < t.n ? (dh[e] + dl[e]) * sg[e] : 0.0f);
       }
       st8(reinterpret_cast<float*>(state + tid), hi, kEpiThreads);
       st8(reinterpret_cast<float*>(state + 2 * kEpiThreads + tid), lo, kEpiThreads);
@@ -313,9 +321,8 @@ __device__ __forceinline__ void ts_move_resident(const WalkerTail& t, int cur, i
     float mx = 0.0f;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {   // x = 0 and sigma = 1 past n
-      const float is = t.unit_sigma ? 1.0f : pow2_recip(sg[e]);
-      mx = fmaxf(mx, t.unit_sigma ? fabsf(hi[e]) : fabsf(hi[e]) * is);
-      v[e] = is;
+      v[e] = pow2_recip(sg[e]);
+      mx = fmaxf(mx, fabsf(hi[e]) * v[e]);
     }
     atomicMax(red + wo, __float_as_uint(mx));  // non-negative floats order as their bits
   }
@@ -335,7 +342,7 @@ __device__ __forceinline__ void ts_move_resident(const WalkerTail& t, int cur, i
   }
   if (c == 0) t.wscale[k] = ws;
 #pragma unroll
-  for (int e = 0; e < 8; ++e) v[e] = t.unit_sigma ? (hi[e] + lo[e]) * inv : (hi[e] + lo[e]) * inv * v[e];
+  for (int e = 0; e < 8; ++e) v[e] = (hi[e] + lo[e]) * inv * v[e];
   const size_t o = op_off(k, i0, t.k_pad, t.z_ld, 1);
   if (split_store8(v, t.Xh + o, t.Xl + o)) atomicOr(t.status, MHAR_ST_NONFINITE);
   if (out != nullptr && k < emit) {
@@ -426,8 +433,18 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint64_t step0 = p.step_ptr != nullptr ? *p.step_ptr + static_cast<uint64_t>(p.j) : p.step0;
-  uint4* state = p.resident ? reinterpret_cast<uint4*>(stage) : nullptr;
   const int tid = static_cast<int>(threadIdx.x) - 64;   // of the epilogue, then the draw threads
+  const int my_c = tid / w_count, my_w = tid - my_c * w_count;   // a resident thread's item
+  const int theta_threads = (w_count + 31) & ~31;
+  const int quads = p.wt.draw ? ((p.wt.n + 7) >> 3) * 2 * w_count : 0;
+  const int epi_draws = kEpiThreads - theta_threads;             // threads that draw after the tiles
+  uint4* state = p.resident ? reinterpret_cast<uint4*>(stage) : nullptr;
+  if (tid >= 0 && tid < kWalkers) {
+    const bool in = tid < p.wt.n_ld;
+    tail->sigma[tid] = in ? p.wt.sigma[tid] : 1.0f;
+    tail->delta[tid] = in && p.wt.pc_rank >= 0 ? p.wt.pc_delta[tid] : 0.0f;
+  }
+  __syncthreads();
   if (state != nullptr && warp >= 2 && warp < kDrawWarp)
     ts_load_state(p.wt, static_cast<int>(step0 & 1ull), strip, p.z, w_begin, w_count, tid, state);
   int pu = 0;                // producer: pair uses issued
@@ -544,20 +561,16 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
       __syncwarp();
     } else if (warp >= kDrawWarp) {
       // ---- iteration s+1's directions into the other pair ------------------------
-      if (p.wt.draw) {
-        const int dt = tid - kEpiThreads;
-        const int items = ((p.wt.n + 7) >> 3) * w_count;
-        if (p.wt.pc_rank >= 0) {
-          ts_lowrank(p.wt, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count, dt,
-                     kDrawThreads, tail->gs);
-          if (p.epi_items > 0)
-            asm volatile("bar.sync 3, %0;" ::"n"(kEpiThreads + kDrawThreads) : "memory");
-          else
-            asm volatile("bar.sync 3, %0;" ::"n"(kDrawThreads) : "memory");
-        }
-        ts_draw(p.wt, cur ^ 1, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count,
-                p.epi_items + dt, items, kDrawThreads, tail->gs, state);
+      const int dt = tid - kEpiThreads;
+      if (quads > 0 && p.wt.pc_rank >= 0) {
+        ts_lowrank(p.wt, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count, dt,
+                   kDrawThreads, tail->gs);
+        asm volatile("bar.sync 4, %0;" ::"n"(kDrawThreads) : "memory");
+        if (2 * p.draw_chunks * w_count < quads)
+          asm volatile("bar.arrive 3, %0;" ::"r"(epi_draws + kDrawThreads) : "memory");
       }
+      ts_draw<2>(p.wt, cur ^ 1, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count, dt,
+                 min(p.draw_chunks * w_count, quads / 2), kDrawThreads, tail, state);
     } else {
       // ---- epilogue: s = b - p, ratios, per-walker partial chord ------------------
       // First, while the first row tiles are on their way: iteration s+1's
@@ -580,12 +593,6 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
                                   kStreamChord);
         tail->theta_u[tid] = open_unit_f64(w.x);
         tail->red[tid] = 0u;
-      }
-      if (p.epi_items > 0) {
-        if (p.wt.pc_rank >= 0)
-          asm volatile("bar.sync 3, %0;" ::"n"(kEpiThreads + kDrawThreads) : "memory");
-        ts_draw(p.wt, cur ^ 1, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count, tid,
-                p.epi_items, kEpiThreads, tail->gs, state);
       }
       const int wl = q * 32 + lane;
       const int k = strip * kWalkers + wl;
@@ -666,6 +673,13 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
           }
         }
         tail->theta_s[w_begin + tid] = t;
+      } else if (tid >= theta_threads && 2 * p.draw_chunks * w_count < quads) {
+        // The other warps draw their quads of iteration s+1's directions while
+        // the chords are on their way.
+        if (p.wt.pc_rank >= 0)
+          asm volatile("bar.sync 3, %0;" ::"r"(epi_draws + kDrawThreads) : "memory");
+        ts_draw<1>(p.wt, cur ^ 1, p.seed, step + 1ull, p.walker0, strip, p.z, w_begin, w_count,
+                   2 * p.draw_chunks * w_count + tid - theta_threads, quads, epi_draws, tail, state);
       }
       named_bar<kEpiThreads>();
       // Algorithm 2's thinning: a sample after this iteration?
@@ -674,8 +688,8 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
                         ? p.out + static_cast<size_t>(done / p.thin - 1) * p.emit * p.n
                         : nullptr;
       if (state != nullptr) {
-        ts_move_resident(p.wt, cur, strip, p.z, w_begin, w_count, tid, tail->theta_s, tail->red,
-                         state, out, p.emit, it + 1 == p.iters);
+        ts_move_resident(p.wt, cur, strip, p.z, w_begin, my_c, my_w, tid, tail, state, out, p.emit,
+                         it + 1 == p.iters);
       } else {
         ts_move(p.wt, cur, strip, p.z, w_begin, w_count, tid, tail, stage);
         if (out != nullptr) {   // this CTA's walkers, a warp per row
@@ -798,18 +812,15 @@ cudaError_t launch_ts(mhar_ctx* c, int j, const SmallRun* r) {
   p.wt = make_walker_tail(c, 1, true);
   const int share = (kWalkers + s.C - 1) / s.C, items = (c->n + 7) / 8 * share;
   p.resident = r && items <= kEpiThreads ? 1 : 0;
-  // What the draw warps get done beside the tiles: about 100 cycles an MMA (six
-  // per K step) and 8000 of the rest of an iteration, against 1250 cycles a
-  // round of 64 items, 1000 more with U g and 600 a round of low-rank normals.
-  // The epilogue warps draw what is left, before their first tile (4800 cycles
-  // for 416 items).
-  int cycles = s.tiles_per_cta * (p.kdim / kTcK) * 600 + 8000, round = 1250;
-  if (c->pc_rank >= 0) {
-    cycles -= (share * (kMaxPcRank / 4) + kDrawThreads - 1) / kDrawThreads * 600;
-    round += 1000;
-  }
-  const int rounds = cycles > 0 ? cycles / round : 0;
-  p.epi_items = p.wt.draw && rounds * kDrawThreads < items ? items - rounds * kDrawThreads : 0;
+  // The draw warps take what they get done beside the tiles: about 100 cycles an
+  // MMA (six per K step) and 9000 of the rest of an iteration, against 3400 cycles
+  // a round of 64 items (1700 a round of low-rank normals) and 2600 more with
+  // U g.  The epilogue warps draw the others, a quad at a time, between their last
+  // tile and theta, a gap of about 2000 cycles.
+  const bool pc = c->pc_rank >= 0;
+  int cycles = s.tiles_per_cta * (p.kdim / kTcK) * 600 + 9000;
+  if (pc) cycles -= (share * (kMaxPcRank / 4) + kDrawThreads - 1) / kDrawThreads * 1700;
+  p.draw_chunks = std::min(items, std::max(0, cycles / (pc ? 6000 : 3400)) * kDrawThreads) / share;
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.C, plan->strips, 1);
