@@ -398,30 +398,22 @@ projection_ff_kernel(int draw, uint64_t seed, const uint64_t* step_ptr, int j, u
 }
 
 // ---- preconditioned directions ---------------------------------------------
-// d = delta .* h + U g for a block of 32 walkers x 128 coordinates: the block
-// draws the 32 walkers' low-rank normals g (Philox stream 2, Box-Muller as in
+// FP64 mode: d = delta .* h + U g for a block of 32 walkers x 128 coordinates: the
+// block draws the 32 walkers' low-rank normals g (Philox stream 2, Box-Muller as in
 // Section 4.3) into shared memory; each thread keeps its coordinate's row of U
 // in registers and walks the 32 walkers (coalesced along coordinates).
-// In place on the FP64 / FP32 normals, or (split) into the FP16 operand pair
-// as d_i / sigma_i.  The projection (when m_E > 0) follows on the result.
+// In place on the normals.  The projection (when m_E > 0) follows on the result.
 constexpr int kPcWalkers = 32;
 constexpr int kPcThreads = 128;
 
-template <typename T>
 __global__ void __launch_bounds__(kPcThreads)
 precondition_kernel(uint64_t seed, const uint64_t* step_ptr, int j, uint32_t walker0, int z,
-                    int n, int n_ld, int rank, const T* __restrict__ delta,
-                    const T* __restrict__ U, T* D, int split, int k_pad, int z_ld, int inter,
-                    const float* sigma, __half* Dh, __half* Dl, __half* Dh1, __half* Dl1,
-                    int* status) {
-  __shared__ T g[kPcWalkers][kMaxPcRank + 1];
-  if (Dh1 != nullptr && ((*step_ptr + static_cast<uint64_t>(j)) & 1ull)) {
-    Dh = Dh1;  // recompute mode: iteration s's pair is s % 2
-    Dl = Dl1;
-  }
+                    int n, int n_ld, int rank, const double* __restrict__ delta,
+                    const double* __restrict__ U, double* D) {
+  __shared__ double g[kPcWalkers][kMaxPcRank + 1];
   const int k0 = blockIdx.y * kPcWalkers;
   for (int t = threadIdx.x; t < kPcWalkers * (kMaxPcRank + 1); t += kPcThreads)
-    g[t / (kMaxPcRank + 1)][t % (kMaxPcRank + 1)] = T(0);
+    g[t / (kMaxPcRank + 1)][t % (kMaxPcRank + 1)] = 0.0;
   __syncthreads();
   const uint64_t step = *step_ptr + static_cast<uint64_t>(j);
   const int quads = (rank + 3) >> 2;
@@ -430,14 +422,9 @@ precondition_kernel(uint64_t seed, const uint64_t* step_ptr, int j, uint32_t wal
     if (k0 + w >= z) continue;
     const U4 r = philox_block(seed, step, walker0 + static_cast<uint32_t>(k0 + w),
                               static_cast<uint32_t>(q), kStreamLowRank);
-    T v[4];
-    if constexpr (sizeof(T) == 8) {
-      box_muller_f64(open_unit_f64(r.x), open_unit_f64(r.y), v[0], v[1]);
-      box_muller_f64(open_unit_f64(r.z), open_unit_f64(r.w), v[2], v[3]);
-    } else {
-      box_muller_f32(r.x, r.y, v[0], v[1]);
-      box_muller_f32(r.z, r.w, v[2], v[3]);
-    }
+    double v[4];
+    box_muller_f64(open_unit_f64(r.x), open_unit_f64(r.y), v[0], v[1]);
+    box_muller_f64(open_unit_f64(r.z), open_unit_f64(r.w), v[2], v[3]);
 #pragma unroll
     for (int e = 0; e < 4; ++e)
       if (4 * q + e < rank) g[w][4 * q + e] = v[e];
@@ -445,26 +432,129 @@ precondition_kernel(uint64_t seed, const uint64_t* step_ptr, int j, uint32_t wal
   __syncthreads();
   const int i = blockIdx.x * kPcThreads + threadIdx.x;
   if (i >= n) return;
-  T u[kMaxPcRank];
+  double u[kMaxPcRank];
 #pragma unroll
   for (int c = 0; c < kMaxPcRank; ++c) u[c] = U[static_cast<size_t>(i) * kMaxPcRank + c];
-  const T di = delta[i];
-  const float inv_sigma = split ? 1.0f / sigma[i] : 1.0f;  // power of two: exact
+  const double di = delta[i];
   const int wend = min(kPcWalkers, z - k0);
   for (int w = 0; w < wend; ++w) {
     const int k = k0 + w;
-    T acc = di * D[static_cast<size_t>(k) * n_ld + i];
+    double acc = di * D[static_cast<size_t>(k) * n_ld + i];
 #pragma unroll
     for (int c = 0; c < kMaxPcRank; ++c) acc = fma(u[c], g[w][c], acc);
-    if (split) {
-      const float v = static_cast<float>(acc) * inv_sigma;
-      const __half h = __float2half_rn(v);
-      const size_t o = op_off(k, i, k_pad, z_ld, inter);
-      Dh[o] = h;
-      Dl[o] = __float2half_rn(v - __half2float(h));
-      if (!(fabsf(v) <= kHalfMax)) atomicOr(status, MHAR_ST_NONFINITE);
-    } else {
-      D[static_cast<size_t>(k) * n_ld + i] = acc;
+    D[static_cast<size_t>(k) * n_ld + i] = acc;
+  }
+}
+
+// FP32 and tensor-core modes: the draw and d = delta .* h + U g in one kernel, into
+// the FP16 pair as d_i / sigma_i (split), or into D32.  A block takes 64 walkers and
+// a range of 64-coordinate tiles: the walkers' g once in shared memory, U
+// transposed a tile at a time; a thread draws one quad of coordinates for each of
+// four walkers and keeps the sixteen sums, so a step of four columns reads eight
+// 16-byte words for 64 FMAs.  Bound by instruction issue (the Philox words and
+// Box-Muller transforms, then the FMAs).  Two kernels, the normals through memory and a
+// load for each FMA, took 21 + 76 us on illcond500x10000 (z = 16384, rank 32);
+// this one 43 (three blocks an SM: 79 registers).
+constexpr int kDpWalkers = 64;
+constexpr int kDpTile = 64;
+constexpr int kDpThreads = 256;      // 16 quads x 16 groups of four walkers
+
+__global__ void __launch_bounds__(kDpThreads, 3)
+draw_precondition_kernel(uint64_t seed, const uint64_t* step_ptr, int j, uint32_t walker0, int z,
+                         int n, int n_ld, int rank, int tiles_per_block,
+                         const float* __restrict__ delta, const float* __restrict__ U, float* D32,
+                         int split, int k_pad, int z_ld, int inter, const float* __restrict__ sigma,
+                         __half* Dh, __half* Dl, __half* Dh1, __half* Dl1, int* status) {
+  __shared__ __align__(16) float g[kDpWalkers][kMaxPcRank];
+  __shared__ __align__(16) float ut[kMaxPcRank][kDpTile + 4];   // U^T of the tile
+  const uint64_t step = *step_ptr + static_cast<uint64_t>(j);
+  if (Dh1 != nullptr && (step & 1ull)) {
+    Dh = Dh1;  // recompute mode: iteration s's pair is s % 2
+    Dl = Dl1;
+  }
+  const int tid = threadIdx.x, k0 = blockIdx.y * kDpWalkers;
+  for (int t = tid; t < kDpWalkers * (kMaxPcRank / 4); t += kDpThreads) {
+    const int w = t / (kMaxPcRank / 4), q = t % (kMaxPcRank / 4);
+    float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (4 * q < rank && k0 + w < z) {
+      const U4 r = philox_block(seed, step, walker0 + static_cast<uint32_t>(k0 + w),
+                                static_cast<uint32_t>(q), kStreamLowRank);
+      box_muller_f32(r.x, r.y, v[0], v[1]);
+      box_muller_f32(r.z, r.w, v[2], v[3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) g[w][4 * q + e] = 4 * q + e < rank ? v[e] : 0.0f;
+  }
+  const int q = tid & 15, wg = 4 * (tid >> 4);
+  const int t_end = min((n + kDpTile - 1) / kDpTile, static_cast<int>(blockIdx.x + 1) * tiles_per_block);
+  for (int t = blockIdx.x * tiles_per_block; t < t_end; ++t) {
+    const int i0 = t * kDpTile;
+    __syncthreads();      // g is ready; the tile before is done with
+    for (int e = tid; e < kDpTile * kMaxPcRank; e += kDpThreads) {
+      const int i = i0 + (e >> 5);
+      ut[e & 31][e >> 5] = i < n ? U[static_cast<size_t>(i) * kMaxPcRank + (e & 31)] : 0.0f;
+    }
+    __syncthreads();
+    const int i = i0 + 4 * q;
+    if (i >= n) continue;
+    float acc[4][4], dl[4], is[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      dl[e] = i + e < n ? delta[i + e] : 0.0f;
+      is[e] = split && i + e < n ? pow2_recip(sigma[i + e]) : 1.0f;
+    }
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const U4 r = philox_block(seed, step, walker0 + static_cast<uint32_t>(k0 + wg + w),
+                                static_cast<uint32_t>(i >> 2), kStreamDirection);
+      box_muller_f32(r.x, r.y, acc[w][0], acc[w][1]);
+      box_muller_f32(r.z, r.w, acc[w][2], acc[w][3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[w][e] *= dl[e];
+    }
+#pragma unroll 2
+    for (int c = 0; c < kMaxPcRank; c += 4) {
+      float4 gv[4];
+#pragma unroll
+      for (int w = 0; w < 4; ++w) gv[w] = *reinterpret_cast<const float4*>(&g[wg + w][c]);
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const float4 u = *reinterpret_cast<const float4*>(&ut[c + cc][4 * q]);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const float gc = cc == 0 ? gv[w].x : cc == 1 ? gv[w].y : cc == 2 ? gv[w].z : gv[w].w;
+          acc[w][0] = fmaf(u.x, gc, acc[w][0]);
+          acc[w][1] = fmaf(u.y, gc, acc[w][1]);
+          acc[w][2] = fmaf(u.z, gc, acc[w][2]);
+          acc[w][3] = fmaf(u.w, gc, acc[w][3]);
+        }
+      }
+    }
+    // n_ld and k_pad are multiples of four: the quad's padding is 0 and stays so.
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int k = k0 + wg + w;
+      if (k >= z) continue;
+      if (split) {
+        __half2 h[2], l[2];
+        bool bad = false;
+#pragma unroll
+        for (int e = 0; e < 4; e += 2) {
+          const float a = i + e < n ? acc[w][e] * is[e] : 0.0f;
+          const float b = i + e + 1 < n ? acc[w][e + 1] * is[e + 1] : 0.0f;
+          h[e / 2] = __floats2half2_rn(a, b);
+          l[e / 2] = __floats2half2_rn(a - __low2float(h[e / 2]), b - __high2float(h[e / 2]));
+          bad |= !(fabsf(a) <= kHalfMax) || !(fabsf(b) <= kHalfMax);
+        }
+        if (bad) atomicOr(status, MHAR_ST_NONFINITE);
+        const size_t o = op_off(k, i, k_pad, z_ld, inter);
+        *reinterpret_cast<uint2*>(Dh + o) = *reinterpret_cast<const uint2*>(h);
+        *reinterpret_cast<uint2*>(Dl + o) = *reinterpret_cast<const uint2*>(l);
+      } else {
+        *reinterpret_cast<float4*>(D32 + static_cast<size_t>(k) * n_ld + i) =
+            make_float4(acc[w][0], i + 1 < n ? acc[w][1] : 0.0f, i + 2 < n ? acc[w][2] : 0.0f,
+                        i + 3 < n ? acc[w][3] : 0.0f);
+      }
     }
   }
 }
@@ -1548,20 +1638,28 @@ cudaError_t launch_projection(mhar_ctx* c, int j, int draw) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_precondition(mhar_ctx* c, int j, int split) {
+cudaError_t launch_precondition(mhar_ctx* c, int j) {
   dim3 grid(blocks_for(c->n, kPcThreads), blocks_for(c->z, kPcWalkers));
+  precondition_kernel<<<grid, kPcThreads, 0, c->stream>>>(
+      c->opts.seed, c->d.step, j, c->opts.walker0, c->z, c->n, c->n_ld, c->pc_rank,
+      c->d.pc_delta64, c->d.pc_U64, c->d.D64);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_draw_precondition(mhar_ctx* c, int j, int split) {
   const int z_ld = (c->z + 127) / 128 * 128;
-  if (c->opts.precision == MHAR_FP64) {
-    precondition_kernel<double><<<grid, kPcThreads, 0, c->stream>>>(
-        c->opts.seed, c->d.step, j, c->opts.walker0, c->z, c->n, c->n_ld, c->pc_rank,
-        c->d.pc_delta64, c->d.pc_U64, c->d.D64, 0, c->k_pad, z_ld, 0, nullptr, nullptr, nullptr,
-        nullptr, nullptr, c->d.status);
-  } else {
-    precondition_kernel<float><<<grid, kPcThreads, 0, c->stream>>>(
-        c->opts.seed, c->d.step, j, c->opts.walker0, c->z, c->n, c->n_ld, c->pc_rank,
-        c->d.pc_delta32, c->d.pc_U32, c->d.D32, split, c->k_pad, z_ld, c->use_ts ? 1 : 0,
-        c->d.sigma, c->d.Dh, c->d.Dl, c->d.Dh2, c->d.Dl2, c->d.status);
-  }
+  int sms = 148;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  // A block's g is drawn again by each block beside it along the coordinates (as
+  // much work as half a tile), so only as many as give an SM four blocks.
+  const int tiles = blocks_for(c->n, kDpTile), rows = blocks_for(c->z, kDpWalkers);
+  int across = blocks_for(4 * sms, rows);
+  across = across > tiles ? tiles : across;
+  const int per = blocks_for(tiles, across);
+  draw_precondition_kernel<<<dim3(blocks_for(tiles, per), rows), kDpThreads, 0, c->stream>>>(
+      c->opts.seed, c->d.step, j, c->opts.walker0, c->z, c->n, c->n_ld, c->pc_rank, per,
+      c->d.pc_delta32, c->d.pc_U32, c->d.D32, split, c->k_pad, z_ld, c->use_ts ? 1 : 0, c->d.sigma,
+      c->d.Dh, c->d.Dl, c->d.Dh2, c->d.Dl2, c->d.status);
   return cudaGetLastError();
 }
 

@@ -251,7 +251,7 @@ int chord_launches(const mhar_ctx* c) {
 int kernels_per_iteration(const mhar_ctx* c) {
   const int chord = chord_launches(c);
   if (tail_draws(c)) return chord;
-  return (projection_draws(c) ? 0 : 1) + (c->mE > 0 ? 1 : 0) + (c->pc_rank >= 0 ? 1 : 0) + chord;
+  return (projection_draws(c) ? 0 : 1) + (c->mE > 0 ? 1 : 0) + (c->pc_rank >= 0 && c->opts.precision == MHAR_FP64 ? 1 : 0) + chord;
 }
 
 int emit_count(const mhar_ctx* c) {
@@ -264,12 +264,14 @@ cudaError_t enqueue_directions(mhar_ctx* c, int j) {
   if (tail_draws(c)) return cudaSuccess;  // drawn by the previous chord kernel
   const bool fused = projection_draws(c);
   cudaError_t e = cudaSuccess;
-  if (!fused)
+  if (c->pc_rank >= 0 && c->opts.precision != MHAR_FP64) {
+    // Preconditioned draw d = delta .* h + U g; the tensor-core modes split it
+    // into the FP16 pair here unless the projection still has to run.
+    e = mhar::launch_draw_precondition(c, j, (mixed(c) && c->mE == 0) ? 1 : 0);
+  } else if (!fused) {
     e = recompute(c) ? mhar::launch_prep_walkers(c, j, 4) : mhar::launch_directions(c, j);
-  // Preconditioned draw d = delta .* h + U g; the tensor-core modes split it
-  // into the FP16 pair here unless the projection still has to run.
-  if (e == cudaSuccess && c->pc_rank >= 0)
-    e = mhar::launch_precondition(c, j, (mixed(c) && c->mE == 0) ? 1 : 0);
+    if (e == cudaSuccess && c->pc_rank >= 0) e = mhar::launch_precondition(c, j);
+  }
   if (e == cudaSuccess && c->mE > 0) e = mhar::launch_projection(c, j, fused ? 1 : 0);
   return e;
 }
@@ -294,10 +296,11 @@ cudaError_t enqueue_chord(mhar_ctx* c, int j) {
 // directions when the chord kernel draws them.
 int ensure_operands(mhar_ctx* c) {
   if (!recompute(c) || c->operands_fresh) return MHAR_OK;
-  MHAR_CUDA(mhar::launch_prep_walkers(c, 0, tail_draws(c) ? 6 : 2), "operand preparation");
+  const bool draw = tail_draws(c) && c->pc_rank < 0;
+  MHAR_CUDA(mhar::launch_prep_walkers(c, 0, draw ? 6 : 2), "operand preparation");
   ++c->launches;
-  if (tail_draws(c) && c->pc_rank >= 0) {  // preconditioned first directions
-    MHAR_CUDA(mhar::launch_precondition(c, 0, 1), "operand preparation");
+  if (tail_draws(c) && !draw) {  // preconditioned first directions
+    MHAR_CUDA(mhar::launch_draw_precondition(c, 0, 1), "operand preparation");
     ++c->launches;
   }
   c->operands_fresh = true;

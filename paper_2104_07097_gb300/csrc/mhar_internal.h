@@ -197,9 +197,11 @@ cudaError_t launch_set_points(mhar_ctx* ctx, const double* X_dev);
 cudaError_t launch_prepare_tc_operands(mhar_ctx* ctx, bool blocks = true);
 cudaError_t launch_refresh_simt(mhar_ctx* ctx);
 cudaError_t launch_reproject(mhar_ctx* ctx);
-// d <- delta .* d + U g on the drawn normals (FP64 / FP32 scratch), writing the
+// Preconditioned directions: d <- delta .* d + U g on the drawn normals (FP64)
+cudaError_t launch_precondition(mhar_ctx* ctx, int j);
+// and, in the other modes, draw and preconditioner in one: into D32, or into the
 // FP16 pair (divided by sigma) when `split`.
-cudaError_t launch_precondition(mhar_ctx* ctx, int j, int split);
+cudaError_t launch_draw_precondition(mhar_ctx* ctx, int j, int split);
 
 // ---- FP64 / FP32 modes, screened on the tensor cores (kernels_screen.cu) -------
 bool screen_eligible(const mhar_ctx* ctx);    // by its sizes
