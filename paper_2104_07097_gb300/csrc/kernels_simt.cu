@@ -13,6 +13,7 @@
 //   on the chord and moves x += theta d.
 // These kernels serve MHAR_FP64 (T = double) and MHAR_FP32 (T = float; points
 // kept as FP32 pairs).  The tensor-core mode is in kernels_tc.cu.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <cuda_fp16.h>
@@ -919,6 +920,34 @@ __global__ void emit_kernel(int mode, int z, int n, int n_ld, const double* X64,
   out[idx] = mode == 0 ? X64[src] : static_cast<double>(Xhi[src]) + static_cast<double>(Xlo[src]);
 }
 
+// A batch: the samples of up to kBatchEmit problems (grid.y) in one launch, and
+// every problem's status words cleared or gathered (a launch, and a copy, of its
+// own for each of 48 problems took 350 us of a call).
+__global__ void batch_emit_kernel(const BatchProblem* __restrict__ probs, const BatchOuts outs) {
+  const BatchProblem p = probs[blockIdx.y];
+  double* out = outs.out[blockIdx.y];
+  if (out == nullptr) return;
+  const long long count = static_cast<long long>(p.walkers) * p.n;
+  for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < count;
+       idx += static_cast<long long>(gridDim.x) * blockDim.x) {
+    const int k = static_cast<int>(idx / p.n), i = static_cast<int>(idx - static_cast<long long>(k) * p.n);
+    const size_t src = static_cast<size_t>(k) * p.n_ld + i;
+    out[idx] = static_cast<double>(p.Xhi[src]) + static_cast<double>(p.Xlo[src]);
+  }
+}
+
+__global__ void batch_status_kernel(const BatchProblem* __restrict__ probs, int count, int2* gather) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= count) return;
+  int* st = probs[q].status;
+  if (gather != nullptr) {
+    gather[q] = make_int2(st[0], st[1]);
+  } else {
+    st[0] = 0;
+    st[1] = 0;
+  }
+}
+
 __global__ void set_points_kernel(int mode, int z, int n, int n_ld, const double* Xin, double* X64,
                                   float* Xhi, float* Xlo) {
   const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1740,6 +1769,19 @@ cudaError_t launch_emit(mhar_ctx* c, double* out_device, int walkers) {
   const long long count = static_cast<long long>(walkers) * c->n;
   emit_kernel<<<blocks_for(count, kThreads), kThreads, 0, c->stream>>>(
       mode, walkers, c->n, c->n_ld, c->d.X64, c->d.Xhi, c->d.Xlo, out_device);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_emit(const BatchProblem* probs, int count, long long most,
+                              const BatchOuts& outs, cudaStream_t stream) {
+  const int bx = std::min(64, blocks_for(most, 4 * kThreads));
+  batch_emit_kernel<<<dim3(bx, count), kThreads, 0, stream>>>(probs, outs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_status(const BatchProblem* probs, int count, int2* gather,
+                                cudaStream_t stream) {
+  batch_status_kernel<<<blocks_for(count, kThreads), kThreads, 0, stream>>>(probs, count, gather);
   return cudaGetLastError();
 }
 

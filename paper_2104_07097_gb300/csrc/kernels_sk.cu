@@ -352,12 +352,16 @@ recompute_sk_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
 }
 
 // ---- batched persistent launch --------------------------------------------------
-// Many polytopes in one persistent launch: one CTA per SM pulls whole
-// (problem, walker strip) units from a device queue (an atomic counter over
-// the unit table, largest units first) until the table is exhausted, with
-// the same pipelines as above carried across units.  The producer fetches
-// the next unit as soon as it has issued the current one's loads and hands
-// its index to the MMA issuer and the epilogue through a small ring in
+// Many polytopes in one persistent launch: one CTA per SM pulls units -- a range
+// of the row tiles of a (problem, walker strip) -- from a device queue (an atomic
+// counter over the unit table, largest units first) until the table is
+// exhausted, with the same pipelines as above carried across units.  A strip
+// long beside an SM's share of the batch's work is cut into several units,
+// whose partial chords meet in global memory as in the kernel above: whole
+// strips as units left the launch to its largest bodies (48 bodies of 20 to 400
+// dimensions, 512 walkers each, 16 iterations: 8.63 ms, now 3.88).
+// The producer fetches the next unit as soon as it has issued the current one's
+// loads and hands its index to the MMA issuer and the epilogue through a small ring in
 // shared memory, so one unit's walker-side work (on the epilogue warps)
 // overlaps the next unit's loads and first MMAs, and no CTA is launched or
 // torn down between units.  A unit names its problem, whose tensor maps and
@@ -386,6 +390,11 @@ struct alignas(128) BskProblem {
 struct BskUnit {
   int prob;      // problem
   int strip;     // walker strip within the problem
+  int t0, t1;    // row tiles [t0, t1)
+  int slot;      // index of this unit among the strip's units
+  int nseg;      // units of the strip
+  int part;      // of the first unit: its index among the partial chords
+  int arrival;   // the strip's counter
 };
 
 struct BskParams {
@@ -393,6 +402,8 @@ struct BskParams {
   const BskUnit* units;     // largest first
   int n_units;
   int* queue;               // two counters, used by alternate iterations
+  float* partials;          // [part + slot][2][128]: lambda_min, lambda_max of a unit's rows
+  int* arrivals;            // units of a strip done this iteration (reset by the last)
 };
 
 constexpr int kRing = 4;    // unit indices in flight between the producer and the consumers
@@ -480,7 +491,7 @@ recompute_batch_sk_kernel(const __grid_constant__ BskParams bp, int j) {
         };
         if (resident)
           for (int kc = 0; kc < kch; ++kc) load_w(kc);
-        for (int nt = 0; nt < P.m_tiles; ++nt) {
+        for (int nt = un.t0; nt < un.t1; ++nt) {
           for (int kc = 0; kc < kch; ++kc, ++a_it) {
             if (!resident) load_w(kc);
             // A's hi and lo chunk in one pair of half-slots behind one barrier.
@@ -509,11 +520,12 @@ recompute_batch_sk_kernel(const __grid_constant__ BskParams bp, int j) {
         const int u = ok ? ring->unit[rs] : -1;
         mbar_arrive_sk(&ring->empty[rs]);
         if (u < 0) break;
-        const BskProblem& P = bp.probs[bp.units[u].prob];
+        const BskUnit un = bp.units[u];
+        const BskProblem& P = bp.probs[un.prob];
         const int kch = P.k_chunks, kdim = P.kdim;
         const bool resident = kch <= kWSlots;
         const int wbase = w_it;
-        for (int nt = 0; nt < P.m_tiles; ++nt, ++gt) {
+        for (int nt = un.t0; nt < un.t1; ++nt, ++gt) {
           const int b = gt & 1;
           if (gt >= 2) mbar_wait(&tail->t_empty[b], ((gt >> 1) - 1) & 1, timed_out, P.err);
           tc_fence_after();
@@ -521,7 +533,7 @@ recompute_batch_sk_kernel(const __grid_constant__ BskParams bp, int j) {
           for (int kc = 0; kc < kch; ++kc) {
             const int use = resident ? wbase + kc : w_it;
             const int ws = use % kWSlots;
-            if (!resident || nt == 0)
+            if (!resident || nt == un.t0)
               mbar_wait(&tail->w_full[ws], (use / kWSlots) & 1, timed_out, P.err);
             const uint32_t w0 = smem_u32(wslot + ws * kWBytes) + op0;
             const uint64_t o_h = sw128_desc(w0), o_l = sw128_desc(w0 + kOperandBytes);
@@ -570,10 +582,14 @@ recompute_batch_sk_kernel(const __grid_constant__ BskParams bp, int j) {
       const int cur = static_cast<int>(step & 1ull);
       const int strip = un.strip;
       const int row0 = cg * 32;
-      if (lane < 4) prefetch_l1(row_block(P.rows, row0) + 32 * lane);
-      if (P.wt.draw)
+      if (lane < 4) prefetch_l1(row_block(P.rows, row0 + un.t0 * kRowsTile) + 32 * lane);
+      // Iteration s+1's directions for this unit's share of the strip's walkers.
+      if (P.wt.draw) {
+        const int share = (kWalkers + un.nseg - 1) / un.nseg;
+        const int wb = un.slot * share;
         walker_draw_next<kEpiWarps * 32>(P.wt, cur, P.seed, step + 1ull, P.walker0, strip, P.z,
-                                         0, kWalkers, tid);
+                                         wb, max(0, min(share, kWalkers - wb)), tid);
+      }
       const int k = strip * kWalkers + wl;
       const float ws = P.wscale[k];
       WalkerNorms wn =
@@ -581,9 +597,9 @@ recompute_batch_sk_kernel(const __grid_constant__ BskParams bp, int j) {
       if (k < P.z) add_correction(P.wt, k, wn);
       ChordAcc acc;
       acc.init();
-      for (int nt = 0; nt < P.m_tiles; ++nt, ++gt) {
+      for (int nt = un.t0; nt < un.t1; ++nt, ++gt) {
         const int b = gt & 1;
-        if (lane < 4 && nt + 1 < P.m_tiles) prefetch_l1(row_block(P.rows, row0 + (nt + 1) * kRowsTile) + 32 * lane);
+        if (lane < 4 && nt + 1 < un.t1) prefetch_l1(row_block(P.rows, row0 + (nt + 1) * kRowsTile) + 32 * lane);
         mbar_wait(&tail->t_full[b], (gt >> 1) & 1, timed_out, P.err, true);
         tc_fence_after();
         const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
@@ -603,9 +619,39 @@ recompute_batch_sk_kernel(const __grid_constant__ BskParams bp, int j) {
       tail->part_lo[cg][wl] = lo;
       tail->part_hi[cg][wl] = hi;
       named_bar<kEpiWarps * 32>();
+      float L = -INFINITY, H = INFINITY;
       if (cg == 0) {
-        const float L = fmaxf(fmaxf(lo, tail->part_lo[1][wl]), fmaxf(tail->part_lo[2][wl], tail->part_lo[3][wl]));
-        const float H = fminf(fminf(hi, tail->part_hi[1][wl]), fminf(tail->part_hi[2][wl], tail->part_hi[3][wl]));
+        L = fmaxf(fmaxf(lo, tail->part_lo[1][wl]), fmaxf(tail->part_lo[2][wl], tail->part_lo[3][wl]));
+        H = fminf(fminf(hi, tail->part_hi[1][wl]), fminf(tail->part_hi[2][wl], tail->part_hi[3][wl]));
+      }
+      if (un.nseg > 1) {
+        // Publish this unit's partial chords and count the strip's units; the
+        // last one to arrive goes on to theta.
+        float* part = bp.partials + static_cast<size_t>(un.part) * 2 * kWalkers;
+        if (cg == 0) {
+          part[un.slot * 2 * kWalkers + wl] = L;
+          part[(un.slot * 2 + 1) * kWalkers + wl] = H;
+          __threadfence();
+        }
+        named_bar<kEpiWarps * 32>();
+        if (tid == 0) {
+          const int last = atomicAdd(&bp.arrivals[un.arrival], 1) == un.nseg - 1;
+          if (last) bp.arrivals[un.arrival] = 0;  // every unit of the strip has counted
+          tail->last = last;
+        }
+        named_bar<kEpiWarps * 32>();
+        if (!tail->last) continue;
+        __threadfence();
+        if (cg == 0) {
+          L = -INFINITY;
+          H = INFINITY;
+          for (int g = 0; g < un.nseg; ++g) {
+            L = fmaxf(L, __ldcg(part + 2 * g * kWalkers + wl));
+            H = fminf(H, __ldcg(part + (2 * g + 1) * kWalkers + wl));
+          }
+        }
+      }
+      if (cg == 0) {
         float t = 0.0f;
         if (k < P.z) {
           int flag = 0;
@@ -1123,6 +1169,8 @@ struct BatchSkPlan {
   BskProblem* probs = nullptr;
   BskUnit* units = nullptr;
   int* queue = nullptr;
+  float* partials = nullptr;
+  int* arrivals = nullptr;
   int n_units = 0;
   int grid = 0;
 };
@@ -1130,7 +1178,7 @@ struct BatchSkPlan {
 void batch_sk_destroy(void* plan_v) {
   BatchSkPlan* plan = static_cast<BatchSkPlan*>(plan_v);
   if (!plan) return;
-  void* ptrs[] = {plan->probs, plan->units, plan->queue};
+  void* ptrs[] = {plan->probs, plan->units, plan->queue, plan->partials, plan->arrivals};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete plan;
@@ -1142,7 +1190,11 @@ int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx[0]->device);
   std::vector<BskProblem> probs(count);
   std::vector<BskUnit> units;
-  std::vector<long long> size(count);
+  // Cost of a row tile and of a unit's set-up, in clocks: six MMAs of 85 clocks
+  // a K step, but no less than the epilogue's 2700 a tile.
+  std::vector<long long> tile_cost(count);
+  constexpr long long kUnitCost = 8000;
+  long long total = 0;
   for (int q = 0; q < count; ++q) {
     const mhar_ctx* c = ctx[q];
     const TcPlan* tp = static_cast<const TcPlan*>(c->tc);
@@ -1168,12 +1220,41 @@ int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, 
     P.k_pad = c->k_pad;
     P.m_tiles = tc_plan_m_tiles(c);
     P.wt = make_walker_tail(c, 0);
-    size[q] = static_cast<long long>(P.m_tiles) * P.k_chunks;
-    for (int st = 0; st < tc_plan_strips(c); ++st) units.push_back({q, st});
+    tile_cost[q] = std::max<long long>(2700, 6 * 85 * (c->kdim / kTcK));
+    total += tc_plan_strips(c) * P.m_tiles * tile_cost[q];
+  }
+  // The longest unit: of a few lengths the one with the least time estimated, the
+  // SMs' even share of the work with every unit's set-up plus half a longest unit
+  // (largest first), at least one longest unit.
+  auto units_of = [&](int q, long long most) {
+    const long long tiles = probs[q].m_tiles;
+    return static_cast<int>(std::min<long long>(
+        {(tiles * tile_cost[q] + most - 1) / most, tiles, static_cast<long long>(kWalkers)}));
+  };
+  long long most = 0, best = 0;
+  for (long long len = 2700; len <= 16 * std::max(total, 2700ll); len = len * 3 / 2) {
+    long long sum = total, longest = 0;
+    for (int q = 0; q < count; ++q) {
+      const int g = units_of(q, len);
+      sum += static_cast<long long>(tc_plan_strips(ctx[q])) * g * kUnitCost;
+      longest = std::max(longest, (probs[q].m_tiles + g - 1) / g * tile_cost[q] + kUnitCost);
+    }
+    const long long est = std::max(longest, sum / sms + longest / 2);
+    if (most == 0 || est < best) { best = est; most = len; }
+  }
+  int parts = 0, arrivals = 0;
+  for (int q = 0; q < count; ++q) {
+    const int m_tiles = probs[q].m_tiles;
+    const int nseg = units_of(q, most);
+    for (int st = 0; st < tc_plan_strips(ctx[q]); ++st, parts += nseg, ++arrivals)
+      for (int g = 0; g < nseg; ++g)
+        units.push_back({q, st, static_cast<int>(static_cast<long long>(g) * m_tiles / nseg),
+                         static_cast<int>(static_cast<long long>(g + 1) * m_tiles / nseg), g, nseg,
+                         parts, arrivals});
   }
   // Largest units first, so that the last units pulled are short ones.
   std::stable_sort(units.begin(), units.end(), [&](const BskUnit& a, const BskUnit& b) {
-    return size[a.prob] > size[b.prob];
+    return (a.t1 - a.t0) * tile_cost[a.prob] > (b.t1 - b.t0) * tile_cost[b.prob];
   });
   BatchSkPlan* plan = new BatchSkPlan();
   plan->n_units = static_cast<int>(units.size());
@@ -1184,6 +1265,11 @@ int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, 
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&plan->probs), sizeof(BskProblem) * probs.size());
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&plan->units), sizeof(BskUnit) * units.size());
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&plan->queue), 2 * sizeof(int));
+  if (e == cudaSuccess)
+    e = cudaMalloc(reinterpret_cast<void**>(&plan->partials),
+                   sizeof(float) * static_cast<size_t>(parts) * 2 * kWalkers);
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&plan->arrivals), sizeof(int) * arrivals);
+  if (e == cudaSuccess) e = cudaMemset(plan->arrivals, 0, sizeof(int) * arrivals);
   if (e == cudaSuccess)
     e = cudaMemcpy(plan->probs, probs.data(), sizeof(BskProblem) * probs.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
@@ -1206,6 +1292,8 @@ cudaError_t launch_recompute_batch_sk(const void* plan_v, int j, cudaStream_t st
   p.units = plan->units;
   p.n_units = plan->n_units;
   p.queue = plan->queue;
+  p.partials = plan->partials;
+  p.arrivals = plan->arrivals;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(plan->grid, 1, 1);
   cfg.blockDim = dim3(kThreadsSk, 1, 1);

@@ -1569,6 +1569,8 @@ struct mhar_batch {
   void* sk = nullptr;           // stream-K plan (C == 0)
   void* upd = nullptr;          // the walker update of every problem
   uint64_t** steps = nullptr;   // device array of every problem's step counter
+  mhar::BatchProblem* probs = nullptr;   // device array
+  int2* status = nullptr;       // device array: the problems' status words, gathered
   cudaGraphExec_t g_chunk = nullptr;
   cudaGraphExec_t g_one = nullptr;
   int graph_len = 16;
@@ -1836,18 +1838,24 @@ int mhar_batch_create(const mhar_problem* problems, int32_t count, int32_t z,
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&b->steps), sizeof(uint64_t*) * steps.size());
     if (e == cudaSuccess)
       e = cudaMemcpy(b->steps, steps.data(), sizeof(uint64_t*) * steps.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) rc = batch_cuda(b, e, "step table");
+    std::vector<mhar::BatchProblem> probs;
+    for (mhar_ctx* c : b->ctx)
+      probs.push_back({c->d.Xhi, c->d.Xlo, c->d.status, c->n, c->n_ld, emit_count(c)});
+    if (e == cudaSuccess)
+      e = cudaMalloc(reinterpret_cast<void**>(&b->probs), sizeof(mhar::BatchProblem) * probs.size());
+    if (e == cudaSuccess)
+      e = cudaMemcpy(b->probs, probs.data(), sizeof(mhar::BatchProblem) * probs.size(),
+                     cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaMalloc(reinterpret_cast<void**>(&b->status), sizeof(int2) * probs.size());
+    if (e != cudaSuccess) rc = batch_cuda(b, e, "problem tables");
   }
   if (rc == MHAR_OK) rc = batch_buckets_init(b);
   if (rc == MHAR_OK) {
-    // Default shape: one CTA per unit when the units alone fill the GPU.
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->ctx[0]->device);
-    int strips = 0;
-    for (mhar_ctx* c : b->ctx) strips += mhar::tc_plan_strips(c);
-    int C = 1;
-    while (C < 8 && strips * C * 2 <= sms) C *= 2;
-    rc = batch_set_shape(b, C);
+    // Default shape: the persistent launch, whose units are cut to balance the SMs
+    // (clusters of one size for every body: 2 to 4 times its time on uneven bodies,
+    // 0.9 of it at best, on 48 small bodies of four strips).
+    rc = batch_set_shape(b, 0);
   }
   if (rc != MHAR_OK) {
     remember_create_error(b->err);
@@ -1974,8 +1982,9 @@ int mhar_batch_run(mhar_batch* b, int64_t steps, int64_t thin, double* const* ou
     batch_err(b, "out is NULL but samples are due");
     return MHAR_E_ARG;
   }
-  for (mhar_ctx* c : b->ctx) {
-    cudaError_t e = cudaMemsetAsync(c->d.status, 0, 2 * sizeof(int), b->stream);
+  const int problems = static_cast<int>(b->ctx.size());
+  {
+    cudaError_t e = mhar::launch_batch_status(b->probs, problems, nullptr, b->stream);
     if (e != cudaSuccess) return batch_cuda(b, e, "status reset");
   }
   int64_t done = 0, emitted = 0;
@@ -1997,11 +2006,26 @@ int mhar_batch_run(mhar_batch* b, int64_t steps, int64_t thin, double* const* ou
       b->since_audit = 0;
     }
     if (thin > 0 && done % thin == 0 && emitted < nsamp) {
-      for (size_t q = 0; q < b->ctx.size(); ++q) {
+      for (int q0 = 0; b->opts.out_on_device && q0 < problems; q0 += mhar::kBatchEmit) {
+        mhar::BatchOuts outs;
+        long long most = 0;
+        const int now = std::min(mhar::kBatchEmit, problems - q0);
+        for (int q = 0; q < now; ++q) {
+          const mhar_ctx* c = b->ctx[q0 + q];
+          const long long size = static_cast<long long>(emit_count(c)) * c->n;
+          outs.out[q] = out[q0 + q] ? out[q0 + q] + emitted * size : nullptr;
+          if (out[q0 + q]) most = std::max(most, size);
+        }
+        if (most == 0) continue;
+        cudaError_t e = mhar::launch_batch_emit(b->probs + q0, now, most, outs, b->stream);
+        if (e != cudaSuccess) return batch_cuda(b, e, "emit kernel");
+        ++b->launches;
+      }
+      for (size_t q = 0; !b->opts.out_on_device && q < b->ctx.size(); ++q) {
         mhar_ctx* c = b->ctx[q];
         if (!out[q]) continue;
         rc = emit_to(c, out[q] + static_cast<size_t>(emitted) * emit_count(c) * c->n,
-                     c->opts.out_on_device != 0, emit_count(c));
+                     false, emit_count(c));
         if (rc) {
           batch_err(b, "problem %zu: %s", q, c->err);
           return rc;
@@ -2011,12 +2035,18 @@ int mhar_batch_run(mhar_batch* b, int64_t steps, int64_t thin, double* const* ou
     }
   }
   int worst = MHAR_OK;
-  for (size_t q = 0; q < b->ctx.size(); ++q) {
-    mhar_ctx* c = b->ctx[q];
-    int st[2] = {0, 0};
-    cudaError_t e = cudaMemcpyAsync(st, c->d.status, sizeof(st), cudaMemcpyDeviceToHost, b->stream);
+  std::vector<int2> words(b->ctx.size());
+  {
+    cudaError_t e = mhar::launch_batch_status(b->probs, problems, b->status, b->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(words.data(), b->status, sizeof(int2) * words.size(),
+                          cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return batch_cuda(b, e, "status copy");
+  }
+  for (size_t q = 0; q < b->ctx.size(); ++q) {
+    mhar_ctx* c = b->ctx[q];
+    const int st[2] = {words[q].x, words[q].y};
     c->status_bits |= st[0];
     if (st[1]) {
       batch_err(b, "problem %zu: a tensor-core pipeline wait expired", q);
@@ -2081,6 +2111,8 @@ void mhar_batch_destroy(mhar_batch* b) {
   mhar::update_plan_destroy(b->upd);
   if (b->fork) cudaEventDestroy(b->fork);
   if (b->steps) cudaFree(b->steps);
+  if (b->probs) cudaFree(b->probs);
+  if (b->status) cudaFree(b->status);
   for (mhar_ctx* c : b->ctx) mhar_destroy(c);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
   delete b;

@@ -228,6 +228,22 @@ struct SmallRun {
 };
 cudaError_t launch_small(mhar_ctx* ctx, const SmallRun& r);
 
+// ---- a batch's samples and status words (kernels_simt.cu) -----------------------
+struct BatchProblem {
+  const float* Xhi;
+  const float* Xlo;
+  int* status;
+  int n, n_ld, walkers;      // walkers of a sample
+};
+constexpr int kBatchEmit = 128;
+struct BatchOuts {
+  double* out[kBatchEmit];   // null: no sample of this problem
+};
+cudaError_t launch_batch_emit(const BatchProblem* probs, int count, long long most,
+                              const BatchOuts& outs, cudaStream_t stream);
+cudaError_t launch_batch_status(const BatchProblem* probs, int count, int2* gather,
+                                cudaStream_t stream);   // gather null: clear
+
 // ---- preconditioner fit (kernels_fit.cu) --------------------------------------
 struct FitScratch {
   void* arena = nullptr;     // holds all of the below
