@@ -20,13 +20,14 @@
 //  (3) evaluates the row of the least bound in the mode's own arithmetic -- the
 //      products added in index order by one thread, the bits of
 //      chord_simt_kernel -- and every other row whose bound does not exceed
-//      the ratio found (screen_finish_kernel), then draws theta and moves the
-//      walker as update_kernel does.
-// On a 2000 x 100 body with 4096 walkers an iteration's chord and move take 60 us
-// in FP64 (4131 us with chord_simt_kernel<double>, 63 % of the FP64 pipe) and 43 us
-// in FP32 (234 us): split 8, screen 18 (the MMAs of 12 m n z flops and their
-// epilogue, as in the recompute kernels), finish 15 .. 25 (latency of the serial
-// sums).
+//      the ratio found (screen_finish_kernel; when a stream's second bound does
+//      not, the bounds of its rows are formed again in FP32 by the block), then
+//      draws theta and moves the walker as update_kernel does.
+// On a 2000 x 100 body with 4096 walkers an iteration's chord and move take 55 to 65
+// us in FP64 (4131 us with chord_simt_kernel<double>, 63 % of the FP64 pipe) and 50
+// in FP32 (234 us): split 7 .. 9, screen 18 (the MMAs of 12 m n z flops and their
+// epilogue, as in the recompute kernels), finish 21 .. 39 (latency of the serial
+// sums; 27 .. 87 before the second look at a stream's bounds).
 // So the chord ends, theta and the points have the bits of the direct
 // kernels.  Rows that tie within the bounds (duplicate rows, walkers on a
 // facet) cost more evaluations, never a different result.  Values the bounds
@@ -444,11 +445,19 @@ struct FinParams {
   const uint4* res;
   const unsigned int* tiles;
   const int2* flags;
+  const float* rows;        // the screen's row blocks, operands and walker factors
+  const __half* Ah;
+  const __half* Al;
+  const __half* Xh;
+  const __half* Xl;
+  const __half* Dh;
+  const __half* Dl;
+  const ScreenWalker* sw;
   uint64_t seed;
   const uint64_t* step_ptr;
   int j;
   uint32_t walker0;
-  int m, n, n_ld, z, z_ld, streams, tiles_per_cta, m_tiles, mE;
+  int m, n, n_ld, k_pad, z, z_ld, streams, tiles_per_cta, m_tiles, mE;
   double* lmin;
   double* lmax;
   double* theta;
@@ -524,12 +533,86 @@ __device__ __forceinline__ unsigned int key_limit(double lam, int ed) {
 
 constexpr int kFinThreads = 128;
 constexpr int kFinWalkers = kFinThreads / 4;
+constexpr int kFinList = 256;     // streams that a block looks at again in one round
+
+// Eight consecutive values hi + lo of an FP16 pair.
+__device__ __forceinline__ void pair8(const __half* hi, const __half* lo, float (&v)[8]) {
+  const uint4 h = __ldg(reinterpret_cast<const uint4*>(hi)), l = __ldg(reinterpret_cast<const uint4*>(lo));
+  const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
+    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&lw[e]));
+    v[2 * e] = a.x + b.x;
+    v[2 * e + 1] = a.y + b.y;
+  }
+}
+
+// Whether one row of walker k may hold a chord end on a side below the limit
+// `lim` (key_limit): the screen's bound, formed again in FP32 from the same
+// operands.  Four sums of a quarter of the products each stay inside the K's share for
+// the accumulation, (T + 1) 2^-22 with T = 3 MMAs a step of 16 columns.
+template <typename T>
+__device__ __forceinline__ bool may_hold(const FinParams<T>& p, int k, int row, bool side,
+                                         unsigned int lim) {
+  const size_t ar = static_cast<size_t>(row) * p.k_pad, wr = static_cast<size_t>(k) * p.k_pad;
+  float ps[4] = {}, gs[4] = {};
+#pragma unroll 2
+  for (int i = 0; i < p.n; i += 8) {
+    float a[8], x[8], d[8];
+    pair8(p.Ah + ar + i, p.Al + ar + i, a);
+    pair8(p.Xh + wr + i, p.Xl + wr + i, x);
+    pair8(p.Dh + wr + i, p.Dl + wr + i, d);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      ps[e & 3] = fmaf(a[e], x[e], ps[e & 3]);
+      gs[e & 3] = fmaf(a[e], d[e], gs[e & 3]);
+    }
+  }
+  const float P = (ps[0] + ps[1]) + (ps[2] + ps[3]), g = (gs[0] + gs[1]) + (gs[2] + gs[3]);
+  const float* blk = row_block(p.rows, row & ~31);
+  const int r = row & 31;
+  const ScreenWalker w = p.sw[k];
+  const bool inf = blk[96] != 0.0f;
+  const float kk = blk[32 + r] * (1.0f + 0x1p-20f);
+  const float sl = fmaf(-kk, inf ? w.ws : w.nxw2, fmaf(-P, w.ws, blk[r]));
+  const float den = fmaf(kk, inf ? w.ndinf : w.nd2, side ? -g : g);
+  if (!(den > 0.0f)) return false;
+  const float q = fmaxf(sl, 0.0f) / den * (1.0f - 0x1p-18f);
+  return __float_as_uint(q) <= lim;
+}
+
+// a . x and a . d of one row by one thread, each in index order.
+template <typename T>
+__device__ __forceinline__ void dots_in_order(const T* __restrict__ a, const T* x, const T* d,
+                                              int n_ld, T& ax, T& ad) {
+  constexpr int V = 16 / sizeof(T);
+  ax = ad = T(0);
+#pragma unroll 4
+  for (int i = 0; i < n_ld; i += V) {
+    alignas(16) T av[V];
+    alignas(16) T xv[V];
+    alignas(16) T dv[V];
+    *reinterpret_cast<float4*>(av) = __ldg(reinterpret_cast<const float4*>(a + i));
+    *reinterpret_cast<float4*>(xv) = *reinterpret_cast<const float4*>(x + i);
+    *reinterpret_cast<float4*>(dv) = *reinterpret_cast<const float4*>(d + i);
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      ax += av[u] * xv[u];
+      ad += av[u] * dv[u];
+    }
+  }
+}
 
 // Four threads per walker: (lambda_max, lambda_min) x (a . x, a . d).
 template <typename T>
 __global__ void __launch_bounds__(kFinThreads)
 screen_finish_kernel(const FinParams<T> p) {
   __shared__ double theta_s[kFinWalkers];
+  __shared__ unsigned long long again_s[2 * kFinWalkers];   // least ratio found in a list's rows
+  __shared__ unsigned int limit_s[2 * kFinWalkers];
+  __shared__ int list[kFinList];
+  __shared__ int listed;
   const int lane = threadIdx.x & 31;
   const int wl = threadIdx.x >> 2, t4 = threadIdx.x & 3;
   const int side = t4 >> 1, which = t4 & 1;
@@ -583,49 +666,50 @@ screen_finish_kernel(const FinParams<T> p) {
         lam = fmin(lam, fabs(static_cast<double>(s / g)));
     }
   }
-  // A stream whose second bound may lower it too: all its rows, by the warp.
-  bool need = false;
-  if (go) {
-    const unsigned int lim = key_limit(lam, fl.y);
-    for (int st = which; st < p.streams; st += 2) {
-      const uint4 v = p.res[static_cast<size_t>(st) * p.z_ld + kc];
-      need |= lim != 0u && (side ? v.w : v.y) <= lim;
-    }
+  // A stream whose second bound may lower it too: the bounds of all its rows
+  // again, by the block, and the mode's arithmetic for those that may.  (All its
+  // rows in that arithmetic by one warp held half of the FP64 iterations of a
+  // 2000 x 100 body with 4096 walkers 60 us, every FP32 one 20.)
+  int next = which;                          // this thread's next stream
+  if (which == 0) {
+    again_s[threadIdx.x >> 1] = 0x7ff0000000000000ull;
+    limit_s[threadIdx.x >> 1] = key_limit(lam, fl.y);
   }
-  unsigned int todo = __ballot_sync(0xffffffffu, need);
-  todo = (todo | (todo >> 1)) & 0x55555555u;     // one bit per (walker, side)
-  while (todo) {
-    const int src = __ffs(todo) - 1;
-    todo &= todo - 1;
-    const int wk = __shfl_sync(0xffffffffu, kc, src);
-    const int wside = (src >> 1) & 1;
-    const int ed = __shfl_sync(0xffffffffu, fl.y, src);
-    double best = __shfl_sync(0xffffffffu, lam, src);
-    const T* xk = p.X + static_cast<size_t>(wk) * p.n_ld;
-    const T* dk = p.D + static_cast<size_t>(wk) * p.n_ld;
-    for (int st = 0; st < p.streams; ++st) {
-      const uint4 v = p.res[static_cast<size_t>(st) * p.z_ld + wk];
-      const unsigned int lim = key_limit(best, ed);
-      if (lim == 0u || (wside ? v.w : v.y) > lim) continue;
-      double r = pos_inf();
-      const int ta = (st >> 2) * p.tiles_per_cta;
-      const int tb = min(p.m_tiles, ta + p.tiles_per_cta);
-      for (int nt = ta; nt < tb; ++nt) {
+  for (;;) {
+    if (threadIdx.x == 0) listed = 0;
+    __syncthreads();
+    const unsigned int lim = go ? limit_s[threadIdx.x >> 1] : 0u;
+    if (lim == 0u) next = p.streams;
+    for (; next < p.streams; next += 2) {
+      const uint4 v = p.res[static_cast<size_t>(next) * p.z_ld + kc];
+      if ((side ? v.w : v.y) > lim) continue;
+      const int at = atomicAdd(&listed, 1);
+      if (at >= kFinList) break;             // the next round's first
+      list[at] = (next << 6) | (wl << 1) | side;
+    }
+    __syncthreads();
+    const int count = min(listed, kFinList);
+    for (int e = 0; e < count; ++e) {
+      const int st = list[e] >> 6, ws = list[e] & 63;
+      const int wk = k0 + (ws >> 1);
+      const bool wside = ws & 1;
+      const int ta = (st >> 2) * p.tiles_per_cta, tb = min(p.m_tiles, ta + p.tiles_per_cta);
+      for (int nt = ta + (threadIdx.x >> 5); nt < tb; nt += kFinThreads / 32) {
         const int row = nt * kRowsTile + (st & 3) * 32 + lane;
-        if (row >= p.m) continue;
-        const T* a = p.A + static_cast<size_t>(row) * p.n_ld;
-        T s, g;
-        if (!row_terms(p, wk, row, dot_in_order(a, xk, p.n_ld), dot_in_order(a, dk, p.n_ld), s, g))
+        if (row >= p.m || !may_hold(p, wk, row, wside, limit_s[ws])) continue;
+        T ax, ad, s, g;
+        dots_in_order(p.A + static_cast<size_t>(row) * p.n_ld, p.X + static_cast<size_t>(wk) * p.n_ld,
+                      p.D + static_cast<size_t>(wk) * p.n_ld, p.n_ld, ax, ad);
+        if (!row_terms(p, wk, row, ax, ad, s, g))
           bad = true;
         else if (wside ? g < T(0) : g > T(0))
-          r = fmin(r, fabs(static_cast<double>(s / g)));
+          atomicMin(&again_s[ws], static_cast<unsigned long long>(
+                                      __double_as_longlong(fabs(static_cast<double>(s / g)))));
       }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) r = fmin(r, __shfl_xor_sync(0xffffffffu, r, off));
-      best = fmin(best, r);
     }
-    if ((lane & ~1) == (src & ~1)) lam = best;
+    if (!__syncthreads_or(next < p.streams)) break;
   }
+  lam = fmin(lam, __longlong_as_double(static_cast<long long>(again_s[threadIdx.x >> 1])));
   // Walkers outside the screen's range: every row.
   unsigned int forced = __ballot_sync(0xffffffffu, force && t4 == 0);
   while (forced) {
@@ -777,6 +861,8 @@ cudaError_t launch_screen_t(mhar_ctx* c, int j, const T* A, const T* b, const T*
   FinParams<T> f;
   f.A = A; f.b = b; f.kr = kr; f.X = X; f.D = D;
   f.corrn = sizeof(T) == 4 ? d.corrn : nullptr;
+  f.rows = d.rows; f.Ah = d.Ah; f.Al = d.Al; f.Xh = d.Xh; f.Xl = d.Xl; f.Dh = d.Dh; f.Dl = d.Dl;
+  f.sw = sw; f.k_pad = c->k_pad;
   f.nrm32 = nrm; f.res = res; f.tiles = d.scr_tiles; f.flags = flags;
   f.seed = c->opts.seed; f.step_ptr = d.step; f.j = j; f.walker0 = c->opts.walker0;
   f.m = c->m; f.n = c->n; f.n_ld = c->n_ld; f.z = c->z; f.z_ld = z_ld;
