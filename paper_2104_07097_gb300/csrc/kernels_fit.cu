@@ -25,6 +25,7 @@
 
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
+#include "normals_f64.cuh"
 #include "tc_common.cuh"
 
 namespace mhar {
@@ -149,8 +150,8 @@ __global__ void omega_kernel(uint64_t seed, int n, int rank, double* Q) {
   if (c < rank) {
     const U4 w = philox_block(seed, 0ull, static_cast<uint32_t>(c), static_cast<uint32_t>(q),
                               kStreamFit);
-    box_muller_f64(open_unit_f64(w.x), open_unit_f64(w.y), v[0], v[1]);
-    box_muller_f64(open_unit_f64(w.z), open_unit_f64(w.w), v[2], v[3]);
+    box_muller_f64(w.x, w.y, v[0], v[1]);
+    box_muller_f64(w.z, w.w, v[2], v[3]);
   }
 #pragma unroll
   for (int e = 0; e < 4; ++e)

@@ -20,6 +20,7 @@
 
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
+#include "normals_f64.cuh"
 
 namespace mhar {
 namespace {
@@ -52,11 +53,9 @@ __global__ void directions_kernel(int mode, int split, uint64_t seed, const uint
                             static_cast<uint32_t>(q), kStreamDirection);
   const int i0 = 4 * q;
   if (mode == 0) {
+    // One call: a branch for each half ran both for every warp.
     double v[2];
-    if (half == 0)
-      box_muller_f64(open_unit_f64(w.x), open_unit_f64(w.y), v[0], v[1]);
-    else
-      box_muller_f64(open_unit_f64(w.z), open_unit_f64(w.w), v[0], v[1]);
+    box_muller_f64(half ? w.z : w.x, half ? w.w : w.y, v[0], v[1]);
     double* dst = D64 + static_cast<size_t>(k) * n_ld + i0 + 2 * half;
 #pragma unroll
     for (int e = 0; e < 2; ++e)
@@ -424,8 +423,8 @@ precondition_kernel(uint64_t seed, const uint64_t* step_ptr, int j, uint32_t wal
     const U4 r = philox_block(seed, step, walker0 + static_cast<uint32_t>(k0 + w),
                               static_cast<uint32_t>(q), kStreamLowRank);
     double v[4];
-    box_muller_f64(open_unit_f64(r.x), open_unit_f64(r.y), v[0], v[1]);
-    box_muller_f64(open_unit_f64(r.z), open_unit_f64(r.w), v[2], v[3]);
+    box_muller_f64(r.x, r.y, v[0], v[1]);
+    box_muller_f64(r.z, r.w, v[2], v[3]);
 #pragma unroll
     for (int e = 0; e < 4; ++e)
       if (4 * q + e < rank) g[w][4 * q + e] = v[e];

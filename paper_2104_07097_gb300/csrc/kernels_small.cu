@@ -33,6 +33,7 @@
 
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
+#include "normals_f64.cuh"
 
 namespace mhar {
 namespace {
@@ -73,7 +74,7 @@ struct SmallParams {
 };
 
 __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, double& z0, double& z1) {
-  box_muller_f64(open_unit_f64(a), open_unit_f64(b), z0, z1);
+  box_muller_f64(a, b, z0, z1);
 }
 __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float& z0, float& z1) {
   box_muller_f32(a, b, z0, z1);

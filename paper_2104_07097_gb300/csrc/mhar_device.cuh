@@ -51,15 +51,6 @@ __device__ __forceinline__ double open_unit_f64(uint32_t w) {
   return (static_cast<double>(w) + 0.5) * 2.3283064365386963e-10;
 }
 
-// Box-Muller pair from two open uniforms.
-__device__ __forceinline__ void box_muller_f64(double ua, double ub, double& z0, double& z1) {
-  const double r = sqrt(-2.0 * log(ua));
-  double s, c;
-  sincospi(2.0 * ub, &s, &c);
-  z0 = r * c;
-  z1 = r * s;
-}
-
 // (w + 1/2) 2^-32 rounded once to FP32, without FP64 arithmetic: the high 24
 // bits times 256 are exact in FP32 and the low byte plus 1/2 is exact, so
 // their FP32 sum is the correctly rounded w + 1/2 (and scaling by 2^-32 is
