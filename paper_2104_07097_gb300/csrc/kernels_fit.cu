@@ -284,11 +284,11 @@ __device__ __forceinline__ void st_cluster_u32(int* local, uint32_t cta, uint32_
 // the earlier columns is of the order of the unit roundoff already.
 // Bound by the latency of the chain (products, exchange, update) and by the FP64
 // rate of the SMs, which one CTA alone used on one SM: n = 500, rank 32 took 1064
-// us in orth_kernel, 98 here.
-constexpr int kOrthCtas = 8;
+// us in orth_kernel, 89 here.
+constexpr int kOrthCtas = 16;             // 8 (a portable size): 98 us
 constexpr int kOrthThreads = 9 * 32;      // eight warps of products, one that sums
 constexpr int kOrthPasses = 3;
-constexpr int kOrthMaxLd = 872;           // 32 columns of 872 rows: 223232 bytes
+constexpr int kOrthMaxLd = 856;           // 32 columns of 856 rows: 219136 bytes
 
 __host__ __device__ constexpr int orth_ld(int n) {   // 8 mod 16: spreads the banks
   return ((n + kOrthCtas - 1) / kOrthCtas + 7) / 16 * 16 + 8;
@@ -318,7 +318,7 @@ orth_cluster_kernel(int n, int rank, const double* __restrict__ Y, double* __res
       auto& got = recv[turn];
       turn ^= 1;
       // Products of columns 0 .. c with v: 8 lanes a column, which then send
-      // the sum to one CTA each.
+      // the sum to two CTAs each.
       const int p = tid >> 3, g = tid & 7;
       if ((tid & ~31) >> 3 <= c && warp < 8) {
         double acc = 0.0;
@@ -326,7 +326,8 @@ orth_cluster_kernel(int n, int rank, const double* __restrict__ Y, double* __res
           for (int i = g; i < rows; i += 8) acc = fma(col[p * ld + i], v[i], acc);
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        st_cluster_f64(&got[cta][p], static_cast<uint32_t>(g), acc);
+        for (int to = g; to < kOrthCtas; to += 8)
+          st_cluster_f64(&got[cta][p], static_cast<uint32_t>(to), acc);
       }
       tc::cluster_sync_all();
       double nrm2 = 0.0, vv = 0.0;
@@ -335,7 +336,11 @@ orth_cluster_kernel(int n, int rank, const double* __restrict__ Y, double* __res
 #pragma unroll
         for (int r = 0; r < kOrthCtas; ++r) s[r] = lane <= c ? got[r][lane] : 0.0;
         // The same order in every CTA: every CTA decides alike.
-        const double dot = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+#pragma unroll
+        for (int w = kOrthCtas / 2; w > 0; w >>= 1)
+#pragma unroll
+          for (int r = 0; r < w; ++r) s[r] += s[r + w];
+        const double dot = s[0];
         const double cf = lane < c ? dot * inv2[lane] : 0.0;
         coef[lane] = cf;
         nrm2 = lane < c ? -dot * cf : dot;     // dot = 0 past c
@@ -397,17 +402,23 @@ ritz_matrix_kernel(int n, int rank, const double* __restrict__ Q, const double* 
   }
 }
 
+__device__ __forceinline__ float sqrt_approx(float v) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
 // T = V Lambda V^T by Jacobi rotations in cyclic row order, all rotations of
 // one antidiagonal p + q at once: (p, q) shares an index only with rotations
 // of smaller p + q before it in that order and of larger p + q after it, so
 // the result is the row-cyclic one with 2 rank - 3 steps a sweep instead of
 // rank (rank - 1) / 2.  Two CTAs: the first rotates T (a warp per pair), the
 // second V, one step behind, so V's half of the FP64 work is off the chain.
-// The angle comes from FP32 (a relative error of 1e-7 in tan leaves that share
-// of the entry to the next sweep); cos and sin are normalised in FP64, so the
+// The angle comes from FP32's approximate functions (a relative error of 1e-6 in
+// tan leaves that share of the entry to the next sweep); cos and sin are normalised in FP64, so the
 // rotations are orthogonal to the FP64 roundoff.
 // Bound by the chain of steps and one SM's FP64 rate; rank 32 with one warp and
-// one rotation at a time took most of 8018 us, 697 here.
+// one rotation at a time took most of 8018 us, 669 here.
 constexpr int kJacobiThreads = 512;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kJacobiThreads)
@@ -467,9 +478,9 @@ jacobi_kernel(int rank, const double* __restrict__ Tin, double* __restrict__ lam
           const float apq = static_cast<float>(M[pp][qq]);
           double2 r = make_double2(1.0, 0.0);
           if (apq != 0.0f) {
-            const float tau = static_cast<float>(M[qq][qq] - M[pp][pp]) / (2.0f * apq);
-            const double tn = static_cast<double>((tau >= 0.0f ? 1.0f : -1.0f) /
-                                                  (fabsf(tau) + sqrtf(1.0f + tau * tau)));
+            const float tau = __fdividef(static_cast<float>(M[qq][qq] - M[pp][pp]), 2.0f * apq);
+            const float root = fabsf(tau) + sqrt_approx(fmaf(tau, tau, 1.0f));
+            const double tn = static_cast<double>(__fdividef(tau >= 0.0f ? 1.0f : -1.0f, root));
             // 1 / sqrt(1 + tn^2), 1 <= 1 + tn^2 <= 2: one step of third order from
             // the FP32 value (error below 1e-20 of it before rounding).
             const double w = fma(tn, tn, 1.0);
@@ -609,6 +620,9 @@ cudaError_t launch_fit_factor(mhar_ctx* c, FitScratch* f, long long samples, int
       // The largest any call needs: the attribute belongs to the function.
       e = cudaFuncSetAttribute(orth_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                static_cast<int>(sizeof(double) * kMaxPcRank * kOrthMaxLd));
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(orth_cluster_kernel,
+                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
     }
     for (int it = 0; it <= power_iters; ++it) {

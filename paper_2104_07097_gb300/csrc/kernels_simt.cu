@@ -1501,10 +1501,15 @@ __global__ void prepare_tc_kernel(int m, int n, int n_ld, int m_pad, int k_pad, 
   int e = 0;
   if (mx > 0.0) frexp(mx, &e);  // mx = f 2^e, f in [0.5, 1)
   const double scale = ldexp(1.0, e);
+  const bool near_one = e >= -1000 && e <= 1000;
+  const double inv = near_one ? ldexp(1.0, -e) : 0.0;
   double q[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // |a|_2^2 |a|_1 |rep|_2^2 |rep|_1 |lo|_2^2 |lo|_1 nnz
   for (int i = threadIdx.x; i < k_pad; i += blockDim.x) {
     double a = 0.0;
-    if (r < m && i < n) a = A[static_cast<size_t>(r) * n_ld + i] * static_cast<double>(sigma[i]) / scale;
+    if (r < m && i < n) {
+      a = A[static_cast<size_t>(r) * n_ld + i] * static_cast<double>(sigma[i]);
+      a = near_one ? a * inv : a / scale;      // the same bits
+    }
     const float v = static_cast<float>(a);
     const __half h = __float2half_rn(v);
     const __half l = __float2half_rn(v - __half2float(h));

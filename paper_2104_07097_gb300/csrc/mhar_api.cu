@@ -77,9 +77,16 @@ int dmalloc(mhar_ctx* c, T** p, size_t count) {
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 bool all_finite(const double* p, size_t n) {
-  for (size_t i = 0; i < n; ++i)
-    if (!std::isfinite(p[i])) return false;
-  return true;
+  // All exponent bits set in none: integer operations without a branch, which the
+  // compiler makes vectors of.
+  constexpr uint64_t kExp = 0x7ff0000000000000ull;
+  uint64_t bad = 0;
+  for (size_t i = 0; i < n; ++i) {
+    uint64_t b;
+    std::memcpy(&b, p + i, sizeof(b));
+    bad |= (b & kExp) == kExp ? 1u : 0u;
+  }
+  return bad == 0;
 }
 
 // Tensor-core modes (FP16-pair operands).
@@ -110,10 +117,11 @@ void free_all(mhar_ctx* c) {
                   d.refresh_step, d.X64, d.Xhi, d.Xlo, d.D64, d.D32, d.Dh, d.Dl, d.S, d.corr, d.corrn, d.Xh, d.Xl, d.wscale, d.Dh2, d.Dl2,
                   d.key_lo, d.key_hi, d.lmin, d.lmax, d.theta, d.status, d.counters, d.step,
                   d.emit, d.check, d.pc_delta64, d.pc_U64, d.pc_delta32, d.pc_U32, d.sigma,
-                  d.small_at};
+                  d.small_at, c->fit_arena};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   d = mhar::DeviceBuffers();
+  c->fit_arena = nullptr;
 }
 
 // Projector set-up on the device (Section 3.2).  With L the Cholesky factor
@@ -669,7 +677,8 @@ bool factor_args_ok(mhar_ctx* c, int32_t rank, int32_t power_iters) {
 
 void fit_release(mhar_ctx* c, mhar::FitScratch* f) {
   cudaStreamSynchronize(c->stream);
-  if (f->arena) cudaFree(f->arena);
+  // A fit's workspace stays with the context up to kFitKeep bytes.
+  if (f->arena && f->arena != c->fit_arena) cudaFree(f->arena);
   *f = mhar::FitScratch();
 }
 
@@ -680,14 +689,21 @@ int fit_alloc(mhar_ctx* c, mhar::FitScratch* f) {
   const size_t counts[] = {n, n, n * n, n * n, n * R, n * R, R * R, R * R, R};
   size_t total = 32;                       // the flag
   for (size_t k : counts) total += (k + 31) / 32 * 32;
-  double* base = nullptr;
-  int rc;
-  if ((rc = dmalloc(c, &base, total)) || (rc = alloc_preconditioner(c))) {
-    f->arena = base;
+  constexpr size_t kFitKeep = 64u << 20;
+  double* base = static_cast<double*>(c->fit_arena);
+  int rc = MHAR_OK;
+  if (base) {
+    cudaError_t e = cudaMemsetAsync(base, 0, total * sizeof(double), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
+  } else {
+    rc = dmalloc(c, &base, total);
+    if (rc == MHAR_OK && total * sizeof(double) <= kFitKeep) c->fit_arena = base;
+  }
+  f->arena = base;
+  if (rc || (rc = alloc_preconditioner(c))) {
     fit_release(c, f);
     return rc;
   }
-  f->arena = base;
   f->flag = reinterpret_cast<int*>(base);
   base += 32;
   for (size_t i = 0; i < sizeof(counts) / sizeof(counts[0]); ++i) {
