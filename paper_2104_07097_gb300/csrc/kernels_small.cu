@@ -73,8 +73,16 @@ struct SmallParams {
   float* Xlo;
 };
 
+// Not inlined: its constants would take registers of the whole loop over the iterations.
+__device__ __noinline__ double2 normals_f64(uint32_t a, uint32_t b) {
+  double2 z;
+  box_muller_f64(a, b, z.x, z.y);
+  return z;
+}
 __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, double& z0, double& z1) {
-  box_muller_f64(a, b, z0, z1);
+  const double2 z = normals_f64(a, b);
+  z0 = z.x;
+  z1 = z.y;
 }
 __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float& z0, float& z1) {
   box_muller_f32(a, b, z0, z1);
@@ -177,6 +185,7 @@ small_kernel(const SmallParams<T> p, int G, int R) {
   const uint64_t step0 = p.step0;
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
 
+  if constexpr (sizeof(T) == 8) prefetch_normals_f64(tid);
   {
     const float4* src = reinterpret_cast<const float4*>(p.At);
     float4* dst = reinterpret_cast<float4*>(at);

@@ -183,6 +183,13 @@ __device__ __forceinline__ void unit_circle_f64(uint32_t w, double& sn, double& 
   if (quarter == 1u || quarter == 2u) cs = -cs;
 }
 
+// The tables into L1 ahead of the first draw (threads tid = 0 .. 16 or more).
+__device__ __forceinline__ void prefetch_normals_f64(int tid) {
+  const char* t = tid < 12 ? reinterpret_cast<const char*>(kLogTable) + 128 * tid
+                           : reinterpret_cast<const char*>(kSinTable) + 128 * (tid - 12);
+  if (tid < 17) asm volatile("prefetch.global.L1 [%0];" ::"l"(t));
+}
+
 // Box-Muller pair from two words.
 __device__ __forceinline__ void box_muller_f64(uint32_t wa, uint32_t wb, double& z0, double& z1) {
   const double r = radius_f64(wa);

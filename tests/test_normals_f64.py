@@ -66,7 +66,10 @@ int main() {
 
 @pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
 def test_normals_within_one_ulp(tmp_path):
-    text = open(os.path.join(CSRC, "normals_f64.cuh")).read().replace("#include <cuda_runtime.h>", "")
+    text = open(os.path.join(CSRC, "normals_f64.cuh")).read()
+    text = text.replace("#include <cuda_runtime.h>", "")
+    at = text.index("// The tables into L1")            # the one function that is PTX
+    text = text[:at] + text[text.index("// Box-Muller pair"):]
     (tmp_path / "normals.h").write_text(text)
     (tmp_path / "main.cpp").write_text(MAIN)
     exe = str(tmp_path / "normals")
