@@ -233,7 +233,8 @@ int mhar_set_audit(mhar_ctx* ctx, int32_t every, int32_t walkers);
  *         small bodies in the FP64 / FP32 modes, whose iterations share a launch
  *   ms[1] the rest of one iteration: the fused tensor-core kernel in the
  *         tensor-core modes, the chord and update kernels otherwise
- *         (Sections 4.4-4.5)
+ *         (Sections 4.4-4.5); all of it where the stored-slack kernel draws the
+ *         next directions beside the chord (no equalities or preconditioner)
  *   ms[2] one slack refresh (mixed mode; 0 otherwise)
  * The timed iterations are real: the chain and its counters advance. */
 int mhar_time_kernels(mhar_ctx* ctx, int iters, double* ms);

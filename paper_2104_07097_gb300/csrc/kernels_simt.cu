@@ -39,7 +39,7 @@ __device__ __forceinline__ double pos_inf() { return __longlong_as_double(0x7ff0
 __global__ void directions_kernel(int mode, int split, uint64_t seed, const uint64_t* step_ptr,
                                   int j, uint32_t walker0, int z, int n, int n_ld, int k_pad,
                                   const float* sigma, double* D64, float* D32, __half* Dh,
-                                  __half* Dl) {
+                                  __half* Dl, __half* Dh1, __half* Dl1) {
   const int quads = (n + 3) >> 2;
   const int per_quad = mode == 0 ? 2 : 1;
   const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -49,6 +49,10 @@ __global__ void directions_kernel(int mode, int split, uint64_t seed, const uint
   const int k = static_cast<int>(qi / quads);
   const int q = static_cast<int>(qi - static_cast<long long>(k) * quads);
   const uint64_t step = *step_ptr + static_cast<uint64_t>(j);
+  if (Dh1 != nullptr && (step & 1ull)) {
+    Dh = Dh1;  // iteration s's pair is s % 2
+    Dl = Dl1;
+  }
   const U4 w = philox_block(seed, step, walker0 + static_cast<uint32_t>(k),
                             static_cast<uint32_t>(q), kStreamDirection);
   const int i0 = 4 * q;
@@ -1615,7 +1619,7 @@ cudaError_t launch_directions(mhar_ctx* c, int j) {
   directions_kernel<<<blocks_for(threads, block), block, 0, c->stream>>>(
       mode, (c->mE == 0 && c->pc_rank < 0) ? 1 : 0, c->opts.seed, c->d.step, j, c->opts.walker0,
       c->z, c->n, c->n_ld,
-      c->k_pad, c->d.sigma, c->d.D64, c->d.D32, c->d.Dh, c->d.Dl);
+      c->k_pad, c->d.sigma, c->d.D64, c->d.D32, c->d.Dh, c->d.Dl, c->d.Dh2, c->d.Dl2);
   return cudaGetLastError();
 }
 

@@ -276,6 +276,8 @@ int tc_plan_strips(const mhar_ctx* ctx);      // walker strips of 128
 int tc_plan_m_tiles(const mhar_ctx* ctx);     // row tiles of 128
 void tc_plan_destroy(mhar_ctx* ctx);
 cudaError_t launch_chord_tc(mhar_ctx* ctx, int j);
+// r.iters iterations in one launch (no equalities, no preconditioner).
+cudaError_t launch_chord_tc_run(mhar_ctx* ctx, const SmallRun& r);
 // X split + S = b - A X (2 launches); check_drift: flag MHAR_ST_DRIFT where the
 // tracked slack differs from the recomputed one by more than its error bound.
 cudaError_t launch_refresh_tc(mhar_ctx* ctx, bool check_drift);

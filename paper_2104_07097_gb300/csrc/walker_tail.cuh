@@ -278,18 +278,16 @@ __device__ __forceinline__ void walker_tail_unstage(const WalkerTail& t, int str
   r.valid = 1;
 }
 
-// (0): run by kThreads threads (tid = 0..kThreads-1); `next_step` = s + 1.  (The
+// (0): the items first, first + stride, ... < last; `next_step` = s + 1.  (The
 // tensor-memory-operand kernel has its own, with the preconditioner.)
-template <int kThreads>
-__device__ void walker_draw_next(const WalkerTail& t, int cur, uint64_t seed, uint64_t next_step,
-                                 uint32_t walker0, int strip, int z, int w_begin, int w_count,
-                                 int tid) {
+__device__ __forceinline__ void walker_draw_items(const WalkerTail& t, int cur, uint64_t seed,
+                                                  uint64_t next_step, uint32_t walker0, int strip,
+                                                  int z, int w_begin, int w_count, int first,
+                                                  int last, int stride) {
   using namespace tail_detail;
-  const int chunks = (t.n + 7) >> 3;
-  const int items = w_count * chunks;
   __half* Dh = t.Dh[cur ^ 1];
   __half* Dl = t.Dl[cur ^ 1];
-  for (int it = tid; it < items; it += kThreads) {
+  for (int it = first; it < last; it += stride) {
     const int c = it / w_count, wo = it - c * w_count;
     const int k = strip * tc::kWalkers + w_begin + wo;
     if (k >= z) continue;
@@ -317,6 +315,15 @@ __device__ void walker_draw_next(const WalkerTail& t, int cur, uint64_t seed, ui
     }
     if (split_store8(v, Dh + o, Dl + o)) atomicOr(t.status, MHAR_ST_NONFINITE);
   }
+}
+
+// All of them, by kThreads threads (tid = 0..kThreads-1).
+template <int kThreads>
+__device__ void walker_draw_next(const WalkerTail& t, int cur, uint64_t seed, uint64_t next_step,
+                                 uint32_t walker0, int strip, int z, int w_begin, int w_count,
+                                 int tid) {
+  walker_draw_items(t, cur, seed, next_step, walker0, strip, z, w_begin, w_count, tid,
+                    w_count * ((t.n + 7) >> 3), kThreads);
 }
 
 // Shared scratch that walker_tail can route the moved points through, so
