@@ -985,14 +985,16 @@ __device__ __forceinline__ double load_point(int mode, const double* X64, const 
 //      s - b_i into the result.  A value FP32 cannot bound (overflow, NaN)
 //      counts as reaching it.
 // The screen is the standard FP32 bound (Higham, Accuracy and Stability,
-// Section 3.1; u = 2^-24): e = gamma_{n+8} ||a_i||_2 ||x||_2 + 4 u |b_i|,
-// gamma_k = k u / (1 - k u), the roundings of A, x, the products, the sums
-// and the comparison among its k; it takes nothing from the walk's own error
-// margins, which the check is there to verify.  Squares of entries below
+// Section 3.1; u = 2^-24): e = gamma_{n+10} ||a_i||_2 ||x||_2 + 4 u |b_i|,
+// gamma_k = k u / (1 - k u), the truncations of A and x (2 u each), the roundings
+// of the products, the sums and the comparison among its k; it takes nothing
+// from the walk's own error margins, which the check is there to verify.  Squares of entries below
 // 2^-75 leave the FP32 norms: kNormFloor per entry covers them.
 // A thread per (row, walker) in FP64, with an atomic each, took 5.35 ms for
 // 4096 walkers of a 2000 x 100 body and 1.39 ms for 1024 of them (ncu); the
-// two kernels take 0.15 and 0.07 ms.
+// two kernels took 109 + 45 us for the 4096 while the screen's conversions from
+// FP64 cost as much as its products and a warp evaluated a whole tile;
+// 80 + 16 us now.
 constexpr int kChkRows = 128;      // rows of a tile
 constexpr int kChkWalkers = 64;    // walkers of a tile
 constexpr int kChkK = 16;
@@ -1004,6 +1006,17 @@ __device__ __forceinline__ unsigned int f32_key(float f) {
 }
 __device__ __forceinline__ float f32_unkey(unsigned int k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// v truncated to FP32 in integer arithmetic (a conversion takes the FP64 pipe 16
+// clocks a warp); below the normal range 0, above it as converted.
+__device__ __forceinline__ float f32_truncated(double v) {
+  const unsigned int hi = static_cast<unsigned int>(__double2hiint(v));
+  const unsigned int lo = static_cast<unsigned int>(__double2loint(v));
+  const unsigned int e = hi & 0x7ff00000u;
+  if (e > 0x47e00000u) return static_cast<float>(v);
+  const unsigned int f = (hi & 0x80000000u) | (((hi & 0x7fffffffu) - 0x38000000u) << 3) | (lo >> 29);
+  return e >= 0x38100000u ? __uint_as_float(f) : 0.0f;
 }
 
 // blockIdx.x: group of `group` consecutive row tiles, blockIdx.y: 64 walkers.
@@ -1018,8 +1031,8 @@ check_screen_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
   __shared__ float an[kChkRows], xn[kChkWalkers], red[16][kChkWalkers];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int w0 = blockIdx.y * kChkWalkers;
-  const float gam = static_cast<float>(n + 8) * 0x1p-24f /
-                    (1.0f - static_cast<float>(n + 8) * 0x1p-24f) * 1.0009765625f;
+  const float gam = static_cast<float>(n + 10) * 0x1p-24f /
+                    (1.0f - static_cast<float>(n + 10) * 0x1p-24f) * 1.0009765625f;
   const float floor_n = static_cast<float>(n) * kNormFloor;
   float up[4], low = -INFINITY;
 #pragma unroll
@@ -1035,35 +1048,54 @@ check_screen_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[r][c] = 0.0f;
     float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sx = 0.0f;
+    // The next K step's part of both tiles is on its way during the products.
+    double2 av[4];
+    double2 xd[2];
+    float4 xh, xl;
+    auto fetch = [&](int k0) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = (tid >> 3) + 32 * j, c = (tid & 7) * 2;
+        av[j] = make_double2(0.0, 0.0);
+        if (i0 + r < m)
+          av[j] = *reinterpret_cast<const double2*>(A + static_cast<size_t>(i0 + r) * n_ld + k0 + c);
+      }
+      xd[0] = xd[1] = make_double2(0.0, 0.0);
+      xh = xl = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (xin) {
+        const size_t o = static_cast<size_t>(w0 + xw) * n_ld + k0 + xk;
+        if (mode == 0) {
+          xd[0] = *reinterpret_cast<const double2*>(X64 + o);
+          xd[1] = *reinterpret_cast<const double2*>(X64 + o + 2);
+        } else {
+          xh = *reinterpret_cast<const float4*>(Xhi + o);
+          xl = *reinterpret_cast<const float4*>(Xlo + o);
+        }
+      }
+    };
+    fetch(0);
     for (int k0 = 0; k0 < n_ld; k0 += kChkK) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int r = (tid >> 3) + 32 * j, c = (tid & 7) * 2;
-        double2 v = make_double2(0.0, 0.0);
-        if (i0 + r < m)
-          v = *reinterpret_cast<const double2*>(A + static_cast<size_t>(i0 + r) * n_ld + k0 + c);
-        const float f0 = static_cast<float>(v.x), f1 = static_cast<float>(v.y);
+        const float f0 = f32_truncated(av[j].x), f1 = f32_truncated(av[j].y);
         As[c][r] = f0;
         As[c + 1][r] = f1;
         sa[j] = fmaf(f0, f0, fmaf(f1, f1, sa[j]));
       }
-      float xv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      if (xin) {
-        const size_t o = static_cast<size_t>(w0 + xw) * n_ld + k0 + xk;
-        if (mode == 0) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) xv[e] = static_cast<float>(X64[o + e]);
-        } else {
-          const float4 h = *reinterpret_cast<const float4*>(Xhi + o);
-          const float4 l = *reinterpret_cast<const float4*>(Xlo + o);
-          xv[0] = h.x + l.x; xv[1] = h.y + l.y; xv[2] = h.z + l.z; xv[3] = h.w + l.w;
-        }
+      float xv[4];
+      if (mode == 0) {
+        xv[0] = f32_truncated(xd[0].x); xv[1] = f32_truncated(xd[0].y);
+        xv[2] = f32_truncated(xd[1].x); xv[3] = f32_truncated(xd[1].y);
+      } else {
+        xv[0] = xh.x + xl.x; xv[1] = xh.y + xl.y; xv[2] = xh.z + xl.z; xv[3] = xh.w + xl.w;
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         Xs[xk + e][xw] = xv[e];
         sx = fmaf(xv[e], xv[e], sx);
       }
+      if (k0 + kChkK < n_ld) fetch(k0 + kChkK);
       __syncthreads();
 #pragma unroll
       for (int kk = 0; kk < kChkK; ++kk) {
@@ -1121,24 +1153,27 @@ check_screen_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
   if ((tid & 31) == 0) atomicMax(best, f32_key(low));
 }
 
-// The FP64 values of the tiles the screen left: a warp looks at kChkEntries
+// The FP64 values of the tiles the screen left: a block looks at kChkEntries
 // entries of ub and takes those at or above the certain value one at a time, a
-// lane per row.  (Few entries a warp: sparse bodies with many slacks near the
-// least leave most of them, and 32 in turn took 35 us.)
-constexpr int kChkEntries = 4;
+// thread per row, the point staged once as FP64.  (A warp an entry with four rows a
+// lane, the point converted by every lane: 22 us each.  Few entries a block: sparse
+// bodies with many slacks near the least leave most of them.)
+constexpr int kChkEntries = 16;
+constexpr int kChkStage = 512;     // columns of the point staged at once
 
-__global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
-                                   const double* __restrict__ A, const double* __restrict__ b,
-                                   const double* __restrict__ X64, const float* __restrict__ Xhi,
-                                   const float* __restrict__ Xlo, const float* __restrict__ ub,
-                                   const unsigned int* __restrict__ best, long long entries,
-                                   unsigned long long* out_key) {
-  const int lane = threadIdx.x & 31;
-  const long long e0 =
-      (static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kChkEntries;
+__global__ void __launch_bounds__(kChkRows)
+check_exact_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
+                   const double* __restrict__ A, const double* __restrict__ b,
+                   const double* __restrict__ X64, const float* __restrict__ Xhi,
+                   const float* __restrict__ Xlo, const float* __restrict__ ub,
+                   const unsigned int* __restrict__ best, long long entries,
+                   unsigned long long* out_key) {
+  __shared__ __align__(16) double xs[kChkStage];
+  const int lane = threadIdx.x & 31, tid = threadIdx.x;
+  const long long e0 = static_cast<long long>(blockIdx.x) * kChkEntries;
   const float floor_v = f32_unkey(*best);
   const bool take = lane < kChkEntries && e0 + lane < entries && !(ub[e0 + lane] < floor_v);
-  unsigned int todo = __ballot_sync(0xffffffffu, take);
+  unsigned int todo = __ballot_sync(0xffffffffu, take);      // every warp the same
   while (todo) {
     const int t = __ffs(todo) - 1;
     todo &= todo - 1;
@@ -1146,38 +1181,32 @@ __global__ void check_exact_kernel(int mode, int m, int n, int n_ld, int walkers
     const int tile = static_cast<int>(en / walkers), k = static_cast<int>(en - static_cast<long long>(tile) * walkers);
     const size_t row = static_cast<size_t>(k) * n_ld;
     const int r1 = min(m, (tile + 1) * group * kChkRows);
-    // Four rows a lane at once, four entries of each ahead: the sums are
-    // serial (index order), so the loads of one hide behind the others.
+    unsigned long long top = 0ull;
     for (int r0 = tile * group * kChkRows; r0 < r1; r0 += kChkRows) {
-      const double* a[4];
-      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      const int r = r0 + tid;
+      const double* a = A + static_cast<size_t>(min(r, m - 1)) * n_ld;
+      double s = 0.0;                                        // in index order
+      for (int c0 = 0; c0 < n; c0 += kChkStage) {
+        const int c1 = min(n_ld - c0, kChkStage);            // zero past n
+        __syncthreads();
+        for (int i = tid; i < c1; i += kChkRows) xs[i] = load_point(mode, X64, Xhi, Xlo, row + c0 + i);
+        __syncthreads();
+        for (int i = 0; i < c1; i += 8) {                    // n_ld is a multiple of 32
+          double2 av[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        a[q] = A + static_cast<size_t>(min(r0 + 32 * q + lane, m - 1)) * n_ld;
-      for (int i = 0; i < n; i += 4) {     // n_ld is a multiple of 32; zero past n
-        double2 av[4][2];
-        double xv[4];
+          for (int q = 0; q < 4; ++q) av[q] = *reinterpret_cast<const double2*>(a + c0 + i + 2 * q);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          av[q][0] = *reinterpret_cast<const double2*>(a[q] + i);
-          av[q][1] = *reinterpret_cast<const double2*>(a[q] + i + 2);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = load_point(mode, X64, Xhi, Xlo, row + i + u);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          s[q] += av[q][0].x * xv[0];
-          s[q] += av[q][0].y * xv[1];
-          s[q] += av[q][1].x * xv[2];
-          s[q] += av[q][1].y * xv[3];
+          for (int q = 0; q < 4; ++q) {
+            s += av[q].x * xs[i + 2 * q];
+            s += av[q].y * xs[i + 2 * q + 1];
+          }
         }
       }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int r = r0 + 32 * q + lane;
-        if (r < r1) atomicMax(out_key, f64_key(s[q] - b[r]));
-      }
+      if (r < r1) top = max(top, f64_key(s - b[r]));
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, off));
+    if (lane == 0) atomicMax(out_key, top);
   }
 }
 
@@ -1839,7 +1868,7 @@ cudaError_t launch_check(mhar_ctx* c, int walkers, unsigned long long* out_keys)
       mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
       c->d.Xlo, ub, best);
   const long long entries = static_cast<long long>(groups) * walkers;
-  check_exact_kernel<<<blocks_for(entries, 4 * kChkEntries), 128, 0, c->stream>>>(
+  check_exact_kernel<<<blocks_for(entries, kChkEntries), kChkRows, 0, c->stream>>>(
       mode, c->m, c->n, c->n_ld, walkers, group, c->d.A64, c->d.b64, c->d.X64, c->d.Xhi,
       c->d.Xlo, ub, best, entries, out_keys);
   if (c->mE > 0) direct(0);
