@@ -160,6 +160,7 @@ template <typename T, bool SCREEN>
 __global__ void __launch_bounds__(kThreadsSmall)
 small_kernel(const SmallParams<T> p, int G, int R) {
   extern __shared__ __align__(16) uint8_t smem_small[];
+  __shared__ double adx[SCREEN ? 1 : kThreadsSmall / 2];     // a . d of few rows
   using AT = std::conditional_t<SCREEN, float, T>;
   const SmallLayout l = small_layout<T, SCREEN>(p.m, p.m_ld, p.n, G, R);
   AT* at = reinterpret_cast<AT*>(smem_small + l.at);
@@ -298,7 +299,23 @@ small_kernel(const SmallParams<T> p, int G, int R) {
         }
         __syncthreads();
       }
-      if (g < live) {
+      const int half = tpw >> 1;
+      if (sizeof(T) == 8 && m <= half) {
+        // Few rows: one thread forms a row's a . x, another, half the walker's
+        // threads on, its a . d.  (FP64 takes a warp 64 clocks an operation
+        // whatever its lanes do; two rows a thread as below took four for each
+        // column.)
+        const int which = t >= half, r = which ? t - half : t;
+        T acc = T(0);
+        if (g < live && r < m) {
+          const T* v = (which ? ds : xs) + g * n;
+          for (int c = 0; c < n; ++c) acc += at[static_cast<size_t>(c) * p.m_ld + r] * v[c];
+          if (which) adx[g * half + r] = static_cast<double>(acc);
+        }
+        __syncthreads();
+        if (g < live && r < m && !which)
+          fold_row<T>(p.b[r] - acc, static_cast<T>(adx[g * half + r]), hi, lo, bad);
+      } else if (g < live) {
         for (int r0 = t; r0 < m; r0 += 2 * tpw) {
           // Two rows at a time: their serial sums overlap.
           const int r1 = r0 + tpw < m ? r0 + tpw : r0;

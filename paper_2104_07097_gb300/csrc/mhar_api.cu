@@ -992,12 +992,17 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
     MHAR_CUDA(cudaStreamSynchronize(c->stream), "sync");
   }
 
-  // Walker state and bookkeeping.
+  // Walker state and bookkeeping.  The staging buffer of host samples holds
+  // sixteen of them, up to 4 MB.
+  c->emit_cap = static_cast<int64_t>(z) * n;
+  if (!c->opts.out_on_device)
+    c->emit_cap = std::max(c->emit_cap,
+                           std::min<int64_t>(16ll * emit_count(c) * n, (4ll << 20) / 8));
   if ((rc = dmalloc(c, &d.key_lo, z)) || (rc = dmalloc(c, &d.key_hi, z)) ||
       (rc = dmalloc(c, &d.lmin, z)) || (rc = dmalloc(c, &d.lmax, z)) ||
       (rc = dmalloc(c, &d.theta, z)) || (rc = dmalloc(c, &d.status, 2)) ||
       (rc = dmalloc(c, &d.counters, 2)) || (rc = dmalloc(c, &d.step, 1)) ||
-      (rc = dmalloc(c, &d.emit, static_cast<size_t>(z) * n)) || (rc = dmalloc(c, &d.check, 6)))
+      (rc = dmalloc(c, &d.emit, static_cast<size_t>(c->emit_cap))) || (rc = dmalloc(c, &d.check, 6)))
     return rc;
   {
     // Audit keys: running max violation from -inf, running residual from 0.
@@ -1170,10 +1175,14 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
   while (done < steps) {
     int64_t adv = steps - done;
     // A kernel that runs many iterations writes samples itself: all of a call's
-    // when they stay on the device, else one to the staging buffer at a time.
+    // when they stay on the device, else as many as the staging buffer holds at a
+    // time (one at a time, a launch and a copy each, took 30 us a sample).
     const bool fused = loops(c) && nsamp > 0;
     const bool whole = fused && c->opts.out_on_device;
-    if (thin > 0 && !whole) adv = std::min<int64_t>(adv, thin - (done % thin));
+    const int64_t sample = static_cast<int64_t>(emit_count(c)) * c->n;
+    const int64_t held = fused ? std::max<int64_t>(1, std::min(nsamp, c->emit_cap / sample)) : 1;
+    if (thin > 0 && !whole) adv = std::min<int64_t>(adv, held * thin - done % thin);
+    const int64_t before = done;
     if (k > 0) adv = std::min<int64_t>(adv, k - c->since_refresh);
     if (au > 0) adv = std::min<int64_t>(adv, au - c->since_audit);
     if (loops(c)) {
@@ -1188,9 +1197,9 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
     done += adv;
     c->step += static_cast<uint64_t>(adv);
     // Out of the staging buffer before the audit takes it as its scratch.
-    if (fused && !whole && done % thin == 0)
-      MHAR_CUDA(cudaMemcpyAsync(out + static_cast<size_t>(done / thin - 1) * emit_count(c) * c->n,
-                                c->d.emit, sizeof(double) * emit_count(c) * c->n,
+    if (fused && !whole && done / thin > before / thin)
+      MHAR_CUDA(cudaMemcpyAsync(out + static_cast<size_t>(before / thin) * sample, c->d.emit,
+                                sizeof(double) * static_cast<size_t>(done / thin - before / thin) * sample,
                                 cudaMemcpyDeviceToHost, c->stream),
                 "sample copy");
     if (au > 0) {

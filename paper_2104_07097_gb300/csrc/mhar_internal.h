@@ -133,6 +133,7 @@ struct mhar_ctx {
   bool use_ts = false;         // recompute mode: TMEM-operand kernel (n <= 128)
   bool use_sk = false;         // recompute mode: stream-K schedule (kernels_sk.cu)
   void* sk = nullptr;          // its segment table
+  int64_t emit_cap = 0;        // doubles that d.emit holds
   void* fit_arena = nullptr;   // a preconditioner fit's workspace, kept between fits
   bool use_small = false;      // FP64 / FP32 modes: all iterations of a call in one launch
   bool use_screen = false;     // FP64 / FP32 modes: screened chord (kernels_screen.cu)
