@@ -60,7 +60,6 @@ METRIC = "walker-steps/s"
 # commands are in profiles/); cold-cache per launch, as ncu replays it.  An
 # entry must be dropped when its kernel changes.
 PROFILED_TRAFFIC = {
-    ("rand100x2000", "recompute_ts_kernel"): 9.575e6 + 0.0,
     ("illcond500x10000", "recompute_sk_kernel"): 127.926e6 + 30.817e6,
 }
 L2_FLUSH_BYTES = 256 << 20
