@@ -107,7 +107,8 @@ typedef struct {
                              to the unsharded run)                            */
   void*    stream;        /* cudaStream_t for all work (NULL: legacy stream)   */
   int32_t  graph_chunk;   /* iterations per captured CUDA graph (default 16;
-                             0 = launch kernels one by one)                   */
+                             0 = launch kernels one by one); kernels that run
+                             many iterations a launch use no graph            */
   int32_t  refresh_fp64;  /* mixed mode: 0 (default) recomputes S on the tensor
                              cores from the same FP16-pair operands the walk
                              uses (FP32 accumulation); 1 recomputes it in FP64

@@ -615,7 +615,7 @@ cudaError_t launch_fit_factor(mhar_ctx* c, FitScratch* f, long long samples, int
     omega_kernel<<<blocks_for(static_cast<long long>(kMaxPcRank) * ((n + 3) / 4), 256), 256, 0,
                    c->stream>>>(c->opts.seed, n, rank, f->Q);
     const size_t smem = sizeof(double) * kMaxPcRank * orth_ld(n);
-    const bool cluster = orth_ld(n) <= kOrthMaxLd;
+    bool cluster = orth_ld(n) <= kOrthMaxLd;
     if (cluster) {
       // The largest any call needs: the attribute belongs to the function.
       e = cudaFuncSetAttribute(orth_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -628,10 +628,13 @@ cudaError_t launch_fit_factor(mhar_ctx* c, FitScratch* f, long long samples, int
     for (int it = 0; it <= power_iters; ++it) {
       symm_block_kernel<<<blocks_for(n, kSymmRows), kSymmWarps * 32, 0, c->stream>>>(
           n, f->sigma, f->Q, f->Y);
-      if (cluster)
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if (cluster) {
         orth_cluster_kernel<<<kOrthCtas, kOrthThreads, smem, c->stream>>>(n, rank, f->Y, f->Q);
-      else
-        orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->Y, f->Q);
+        // A device part without room for sixteen CTAs side by side refuses the launch.
+        cluster = cudaGetLastError() == cudaSuccess;
+      }
+      if (!cluster) orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->Y, f->Q);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     symm_block_kernel<<<blocks_for(n, kSymmRows), kSymmWarps * 32, 0, c->stream>>>(

@@ -881,8 +881,19 @@ cudaError_t launch_screen_t(mhar_ctx* c, int j, const T* A, const T* b, const T*
 // (10 to 76 times the screen's over n = 3 .. 200, m = 700 .. 4000, z = 1000 ..
 // 4096), the direct FP32 kernel 18 us at m z = 10^6 and n <= 32 (the screen
 // 19.4 .. 20.2), 25 against 23 at n = 64, and 90 against 26 .. 35 at m z = 8 10^6.
+// Of the bodies with fewer 64 x 64 tiles than SMs, in FP64 those that the small-body
+// kernel does not take (equalities, A past its shared memory) where a warp's serial
+// sums (n terms for every 32 rows) or all the products are many.  An iteration with
+// one equality, a warp a walker against the screen: 19.5 us where the screen's
+// launches take 23 (20 x 80 with 400 walkers, 60 terms), 32 (screen 24) at 160 terms,
+// 49 (28.5) at 300, 157 (33) at 1170; 32 (25) for 1500 walkers of 60 terms; 575 (36)
+// for 20 to 300 walkers of a 100 x 1500 body.
 bool screen_eligible(const mhar_ctx* c) {
-  if (simt_warp_path(c) || c->k_pad > 2048 || c->m_pad / kRowsTile > 65535) return false;
+  if (c->k_pad > 2048 || c->m_pad / kRowsTile > 65535) return false;
+  if (simt_warp_path(c))
+    return c->opts.precision == MHAR_FP64 &&
+           (static_cast<long long>(c->n) * ((c->m + 31) / 32) >= 128 ||
+            static_cast<long long>(c->m) * c->n * c->z >= 1ll << 21);
   return c->opts.precision == MHAR_FP64 || c->n >= 64 ||
          static_cast<long long>(c->m) * c->z >= 1ll << 21;
 }
