@@ -470,37 +470,86 @@ struct FinParams {
   const float* corr;
 };
 
-// a . v in index order (the padding beyond n is zero).  One thread's serial
-// sum: its rows are brought into L1 a kilobyte ahead, or every 128-byte line
-// would cost the sum an L2 round trip.
-constexpr int kAheadBytes = 1024;
-
+// a . v in index order (the padding beyond n is zero), one thread's serial sum.
 template <typename T>
 __device__ __forceinline__ T dot_in_order(const T* __restrict__ a, const T* v, int n_ld) {
-  constexpr int V = 16 / sizeof(T), kLine = 128 / sizeof(T), kAhead = kAheadBytes / sizeof(T);
-  for (int i = 0; i < min(n_ld, kAhead); i += kLine) {
-    prefetch_l1(a + i);
-    prefetch_l1(v + i);
-  }
+  constexpr int V = 16 / sizeof(T);
   T acc = T(0);
-  for (int i0 = 0; i0 < n_ld; i0 += kLine) {
-    if (i0 + kAhead < n_ld) {
-      prefetch_l1(a + i0 + kAhead);
-      prefetch_l1(v + i0 + kAhead);
-    }
+#pragma unroll 4
+  for (int i = 0; i < n_ld; i += V) {
+    alignas(16) T av[V];
+    alignas(16) T xv[V];
+    *reinterpret_cast<float4*>(av) = __ldg(reinterpret_cast<const float4*>(a + i));
+    *reinterpret_cast<float4*>(xv) = *reinterpret_cast<const float4*>(v + i);
 #pragma unroll
-    for (int i = 0; i < kLine; i += 4 * V) {
-      alignas(16) T av[4 * V];
-      alignas(16) T xv[4 * V];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        *reinterpret_cast<float4*>(av + u * V) = __ldg(reinterpret_cast<const float4*>(a + i0 + i) + u);
-        *reinterpret_cast<float4*>(xv + u * V) = reinterpret_cast<const float4*>(v + i0 + i)[u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4 * V; ++u) acc += av[u] * xv[u];
-    }
+    for (int u = 0; u < V; ++u) acc += av[u] * xv[u];
   }
+  return acc;
+}
+
+// The same for a warp's 32 sums at once (eight walkers x two sides' rows x (a . x,
+// a . d)): the 16 rows, 8 points and 8 directions come into shared memory 128
+// bytes of each at a time, whole lines, kFinStages steps ahead.  Read by the threads
+// themselves each 16 bytes took a line of its own (136 clocks a term in FP64, 59 in
+// FP32); with this and the move's loads in batches an iteration of the 2000 x 100
+// body takes 41 us in FP32 (44.5 before) and 85.6 in FP64 (87.9, bound by the FP64
+// chain).
+constexpr int kFinStages = 4;
+constexpr int kFinRow = 144;                       // bytes between two staged pieces
+constexpr int kFinDir = 24 * kFinRow + 64;         // the directions, off the points' banks
+constexpr int kFinBuf = kFinDir + 8 * kFinRow;     // one step of a warp
+
+template <typename T>
+__device__ __forceinline__ T warp_dots(const T* __restrict__ A, const T* X, const T* D, int row,
+                                       int k, int n_ld, uint8_t* buf) {
+  constexpr int V = 16 / sizeof(T);
+  const int lane = threadIdx.x & 31, piece = lane & 7;
+  const int steps = n_ld * static_cast<int>(sizeof(T)) / 128;
+  // Eight copies a step: lanes 8 q .. 8 q + 7 take vector 4 j + q.
+  const uint8_t* src[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int v = 4 * j + (lane >> 3);
+    const int who = j < 4 ? __shfl_sync(0xffffffffu, row, (2 * v) & 31)
+                          : __shfl_sync(0xffffffffu, k, (4 * (v & 7)) & 31);
+    const T* from = j < 4 ? A : j < 6 ? X : D;
+    src[j] = reinterpret_cast<const uint8_t*>(from + static_cast<size_t>(who) * n_ld) + 16 * piece;
+  }
+  auto issue = [&](int st) {
+    if (st < steps) {
+      const uint32_t to = smem_u32(buf + (st % kFinStages) * kFinBuf) + 16 * piece;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int v = 4 * j + (lane >> 3);
+        const uint32_t dst = to + static_cast<uint32_t>(v * kFinRow + (j >= 6 ? 64 : 0));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src[j] + 128 * st)
+                     : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int st = 0; st < kFinStages - 1; ++st) issue(st);
+  const int mine = (lane >> 1) * kFinRow;
+  const int other = (lane & 1 ? kFinDir : 16 * kFinRow) + (lane >> 2) * kFinRow;
+  T acc = T(0);
+  for (int st = 0; st < steps; ++st) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kFinStages - 2) : "memory");
+    __syncwarp();
+    const uint8_t* at = buf + (st % kFinStages) * kFinBuf;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      alignas(16) T av[V];
+      alignas(16) T xv[V];
+      *reinterpret_cast<float4*>(av) = *reinterpret_cast<const float4*>(at + mine + 16 * u);
+      *reinterpret_cast<float4*>(xv) = *reinterpret_cast<const float4*>(at + other + 16 * u);
+#pragma unroll
+      for (int e = 0; e < V; ++e) acc += av[e] * xv[e];
+    }
+    __syncwarp();
+    issue(st + kFinStages - 1);      // over the step before, read by every lane
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
   return acc;
 }
 
@@ -533,6 +582,7 @@ __device__ __forceinline__ unsigned int key_limit(double lam, int ed) {
 
 constexpr int kFinThreads = 128;
 constexpr int kFinWalkers = kFinThreads / 4;
+constexpr size_t kFinSmem = static_cast<size_t>(kFinThreads / 32) * kFinStages * kFinBuf;
 constexpr int kFinList = 256;     // streams that a block looks at again in one round
 
 // Eight consecutive values hi + lo of an FP16 pair.
@@ -613,6 +663,7 @@ screen_finish_kernel(const FinParams<T> p) {
   __shared__ unsigned int limit_s[2 * kFinWalkers];
   __shared__ int list[kFinList];
   __shared__ int listed;
+  extern __shared__ __align__(16) uint8_t fin_smem[];       // kFinStages steps a warp
   const int lane = threadIdx.x & 31;
   const int wl = threadIdx.x >> 2, t4 = threadIdx.x & 3;
   const int side = t4 >> 1, which = t4 & 1;
@@ -646,17 +697,16 @@ screen_finish_kernel(const FinParams<T> p) {
     if (o1 < b1 || (o1 == b1 && ost < bst)) { b1 = o1; bst = ost; }
     const bool has = b1 <= lim && b1 < kNone;
     if (!__any_sync(0xffffffffu, has)) break;
-    T acc = T(0);
     int row = 0;
     if (has) {
       const unsigned int t = p.tiles[static_cast<size_t>(bst) * p.z_ld + kc];
       row = static_cast<int>(side ? t >> 16 : t & 0xffffu) * kRowsTile + (bst & 3) * 32 +
             static_cast<int>(b1 & 31u);
-      acc = dot_in_order(p.A + static_cast<size_t>(row) * p.n_ld,
-                         (which ? p.D : p.X) + static_cast<size_t>(kc) * p.n_ld, p.n_ld);
       last = b1;
       last_st = bst;
     }
+    const T acc = warp_dots(p.A, p.X, p.D, row, kc, p.n_ld,
+                            fin_smem + (threadIdx.x >> 5) * kFinStages * kFinBuf);
     const T oth = __shfl_xor_sync(0xffffffffu, acc, 1);
     if (has) {
       T s, g;
@@ -765,43 +815,59 @@ screen_finish_kernel(const FinParams<T> p) {
     theta_s[wl] = t;
   }
   __syncthreads();
-  // The rows of the block's walkers are one contiguous range.  Padding: x and
-  // d are 0 there, and stay so.
-  const int items = min(kFinWalkers, p.z - k0) * p.n_ld;
-  const size_t base = static_cast<size_t>(k0) * p.n_ld;
-  constexpr int V = 16 / sizeof(T);
-#pragma unroll 4
-  for (int i = threadIdx.x * V; i < items; i += kFinThreads * V) {
-    const int w = i / p.n_ld;
-    const double t = theta_s[w];
-    if constexpr (sizeof(T) == 8) {
-      double2 x = *reinterpret_cast<const double2*>(p.X64 + base + i);
-      const double2 d = *reinterpret_cast<const double2*>(p.D + base + i);
-      x.x += t * d.x;
-      x.y += t * d.y;
-      *reinterpret_cast<double2*>(p.X64 + base + i) = x;
-    } else {
-      const float tf = static_cast<float>(t);
-      const float4 d4 = *reinterpret_cast<const float4*>(p.D + base + i);
-      float4 h4 = *reinterpret_cast<const float4*>(p.Xhi + base + i);
-      float4 l4 = *reinterpret_cast<const float4*>(p.Xlo + base + i);
-      const float d[4] = {d4.x, d4.y, d4.z, d4.w};
-      float h[4] = {h4.x, h4.y, h4.z, h4.w}, l[4] = {l4.x, l4.y, l4.z, l4.w};
+  // A warp along the rows of every fourth walker of the block, the loads of four of
+  // them before the first store (one after the other: 4 us of an FP64 iteration).
+  // Padding: x and d are 0 there, and stay so.
+  constexpr int V = 16 / sizeof(T), kWarps = kFinThreads / 32, kBatch = 4;
+  for (int i = lane * V; i < p.n_ld; i += 32 * V) {
+#pragma unroll 1
+    for (int w0 = threadIdx.x >> 5; w0 < kFinWalkers; w0 += kBatch * kWarps) {
+      float4 x4[kBatch], l4[kBatch], d4[kBatch];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        df_axpy(h[u], l[u], tf, d[u]);
-        if (p.corr != nullptr && tf != 0.0f) {
-          const int c = i - w * p.n_ld + u;
-          float dlt = 0.0f;
-          if (c < p.n)
-            for (int e = 0; e < p.mE; ++e)
-              dlt = fmaf(p.Q32[static_cast<size_t>(e) * p.n_ld + c],
-                         p.corr[static_cast<size_t>(k0 + w) * p.mE + e], dlt);
-          l[u] = fmaf(-tf, dlt, l[u]);
+      for (int q = 0; q < kBatch; ++q) {
+        const int kk = min(k0 + w0 + q * kWarps, p.z - 1);
+        const size_t o = static_cast<size_t>(kk) * p.n_ld + i;
+        d4[q] = *reinterpret_cast<const float4*>(p.D + o);
+        if constexpr (sizeof(T) == 8) {
+          x4[q] = *reinterpret_cast<const float4*>(p.X64 + o);
+        } else {
+          x4[q] = *reinterpret_cast<const float4*>(p.Xhi + o);
+          l4[q] = *reinterpret_cast<const float4*>(p.Xlo + o);
         }
       }
-      *reinterpret_cast<float4*>(p.Xhi + base + i) = make_float4(h[0], h[1], h[2], h[3]);
-      *reinterpret_cast<float4*>(p.Xlo + base + i) = make_float4(l[0], l[1], l[2], l[3]);
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int w = w0 + q * kWarps, kk = k0 + w;
+        if (kk >= p.z) break;
+        const size_t o = static_cast<size_t>(kk) * p.n_ld + i;
+        const double t = theta_s[w];
+        if constexpr (sizeof(T) == 8) {
+          double2 x = *reinterpret_cast<const double2*>(&x4[q]);
+          const double2 d = *reinterpret_cast<const double2*>(&d4[q]);
+          x.x += t * d.x;
+          x.y += t * d.y;
+          *reinterpret_cast<double2*>(p.X64 + o) = x;
+        } else {
+          const float tf = static_cast<float>(t);
+          const float d[4] = {d4[q].x, d4[q].y, d4[q].z, d4[q].w};
+          float h[4] = {x4[q].x, x4[q].y, x4[q].z, x4[q].w}, l[4] = {l4[q].x, l4[q].y, l4[q].z, l4[q].w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            df_axpy(h[u], l[u], tf, d[u]);
+            if (p.corr != nullptr && tf != 0.0f) {
+              const int c = i + u;
+              float dlt = 0.0f;
+              if (c < p.n)
+                for (int e = 0; e < p.mE; ++e)
+                  dlt = fmaf(p.Q32[static_cast<size_t>(e) * p.n_ld + c],
+                             p.corr[static_cast<size_t>(kk) * p.mE + e], dlt);
+              l[u] = fmaf(-tf, dlt, l[u]);
+            }
+          }
+          *reinterpret_cast<float4*>(p.Xhi + o) = make_float4(h[0], h[1], h[2], h[3]);
+          *reinterpret_cast<float4*>(p.Xlo + o) = make_float4(l[0], l[1], l[2], l[3]);
+        }
+      }
     }
   }
 }
@@ -870,7 +936,8 @@ cudaError_t launch_screen_t(mhar_ctx* c, int j, const T* A, const T* b, const T*
   f.lmin = d.lmin; f.lmax = d.lmax; f.theta = d.theta; f.status = d.status; f.counters = d.counters;
   f.X64 = d.X64; f.Xhi = d.Xhi; f.Xlo = d.Xlo; f.Q32 = d.Q32;
   f.corr = sizeof(T) == 4 ? d.corr : nullptr;
-  screen_finish_kernel<T><<<(c->z + kFinWalkers - 1) / kFinWalkers, kFinThreads, 0, c->stream>>>(f);
+  screen_finish_kernel<T>
+      <<<(c->z + kFinWalkers - 1) / kFinWalkers, kFinThreads, kFinSmem, c->stream>>>(f);
   return cudaGetLastError();
 }
 
@@ -936,6 +1003,14 @@ cudaError_t screen_prepare(mhar_ctx* c, int* outside) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kSmemScr));
+  if (e == cudaSuccess)
+    e = c->opts.precision == MHAR_FP64
+            ? cudaFuncSetAttribute(screen_finish_kernel<double>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   static_cast<int>(kFinSmem))
+            : cudaFuncSetAttribute(screen_finish_kernel<float>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   static_cast<int>(kFinSmem));
   return e;
 }
 
