@@ -12,7 +12,6 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libmhar.so")
 SOURCES = ["mhar_api.cu", "kernels_simt.cu", "kernels_tc.cu", "kernels_rc.cu", "kernels_ts.cu", "noalloc.cu", "kernels_fit.cu", "kernels_sk.cu", "kernels_screen.cu", "kernels_small.cu"]
-HEADERS = ["mhar_device.cuh", "mhar_internal.h", "tc_common.cuh", "walker_tail.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include")]
@@ -24,7 +23,8 @@ def _nvcc() -> str:
 
 
 def _inputs_mtime() -> float:
-    files = [os.path.join(CSRC, f) for f in SOURCES + HEADERS]
+    # Every header beside the sources: a list of names missed a new one.
+    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".h"))]
     files.append(os.path.join(ROOT, "include", "mhar.h"))
     files.append(os.path.abspath(__file__))
     return max(os.path.getmtime(f) for f in files)
