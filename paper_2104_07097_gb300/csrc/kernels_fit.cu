@@ -547,11 +547,14 @@ ritz_finish_kernel(int n, int n_ld, int rank, const double* __restrict__ Q,
     for (int idx = threadIdx.x; idx < kMaxPcRank * kMaxPcRank; idx += blockDim.x)
       V[idx >> 5][idx & 31] = V_in[idx];
   if (warp == 0 && lane < rank) {
-    const double mine = lam_in[lane];
+    // NaN counts as -Inf, ties go by the index: perm is a permutation whatever the values.
+    auto key = [&](int q) { const double v = lam_in[q]; return isnan(v) ? -INFINITY : v; };
+    const double mine = key(lane);
     int at = 0;
-    for (int q = 0; q < rank; ++q) at += lam_in[q] > mine || (lam_in[q] == mine && q < lane);
+    for (int q = 0; q < rank; ++q) at += key(q) > mine || (key(q) == mine && q < lane);
     perm[at] = lane;
     lam[at] = fmax(mine, 0.0);
+    if (!isfinite(lam_in[lane])) atomicOr(flag, 1);
   }
   // Trace of Sigma for the absolute floor.
   double part = 0.0;
