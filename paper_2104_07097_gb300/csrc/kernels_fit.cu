@@ -23,6 +23,7 @@
 // preconditioner is frozen.
 #include <cmath>
 
+#include "jacobi_angle.cuh"
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
 #include "normals_f64.cuh"
@@ -402,21 +403,15 @@ ritz_matrix_kernel(int n, int rank, const double* __restrict__ Q, const double* 
   }
 }
 
-__device__ __forceinline__ float sqrt_approx(float v) {
-  float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-
 // T = V Lambda V^T by Jacobi rotations in cyclic row order, all rotations of
 // one antidiagonal p + q at once: (p, q) shares an index only with rotations
 // of smaller p + q before it in that order and of larger p + q after it, so
 // the result is the row-cyclic one with 2 rank - 3 steps a sweep instead of
 // rank (rank - 1) / 2.  Two CTAs: the first rotates T (a warp per pair), the
 // second V, one step behind, so V's half of the FP64 work is off the chain.
-// The angle comes from FP32's approximate functions (a relative error of 1e-6 in
-// tan leaves that share of the entry to the next sweep); cos and sin are normalised in FP64, so the
-// rotations are orthogonal to the FP64 roundoff.
+// The angle comes from FP32's approximate functions (jacobi_angle.cuh: a relative error
+// of 1e-6 in tan leaves that share of the entry to the next sweep); cos and sin are
+// normalised in FP64, so the rotations are orthogonal to the FP64 roundoff.
 // Bound by the chain of steps and one SM's FP64 rate; rank 32 with one warp and
 // one rotation at a time took most of 8018 us, 669 here.
 constexpr int kJacobiThreads = 512;
@@ -475,20 +470,8 @@ jacobi_kernel(int rank, const double* __restrict__ Tin, double* __restrict__ lam
       if (t_side) {
         if (warp == 0 && lane < pairs) {
           const int pp = p0 + lane, qq = t - pp;
-          const float apq = static_cast<float>(M[pp][qq]);
-          double2 r = make_double2(1.0, 0.0);
-          if (apq != 0.0f) {
-            const float tau = __fdividef(static_cast<float>(M[qq][qq] - M[pp][pp]), 2.0f * apq);
-            const float root = fabsf(tau) + sqrt_approx(fmaf(tau, tau, 1.0f));
-            const double tn = static_cast<double>(__fdividef(tau >= 0.0f ? 1.0f : -1.0f, root));
-            // 1 / sqrt(1 + tn^2), 1 <= 1 + tn^2 <= 2: one step of third order from
-            // the FP32 value (error below 1e-20 of it before rounding).
-            const double w = fma(tn, tn, 1.0);
-            const double y = static_cast<double>(rsqrtf(static_cast<float>(w)));
-            const double d = fma(-w * y, y, 1.0);
-            r.x = fma(y * d, fma(0.375, d, 0.5), y);
-            r.y = tn * r.x;
-          }
+          const double2 r = jacobi_rotation(static_cast<float>(M[pp][qq]),
+                                            static_cast<float>(M[qq][qq] - M[pp][pp]));
           cs[lane] = r;
           st_cluster_f64(&cs[lane].x, 1u, r.x);
           st_cluster_f64(&cs[lane].y, 1u, r.y);
