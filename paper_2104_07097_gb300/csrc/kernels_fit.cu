@@ -131,13 +131,14 @@ cov_accumulate_kernel(int mode, int z, int n, int n_ld, int tiles, const double*
 
 // Sigma (full, symmetric) from S1 and the upper tiles of S2.
 __global__ void cov_finalize_kernel(int n, double N, const double* s1, const double* s2,
-                                    double* sigma, int* flag) {
+                                    double* sigma, int* flag, int* expo) {
   const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= static_cast<long long>(n) * n) return;
   const int i = static_cast<int>(idx / n), jj = static_cast<int>(idx % n);
   const int lo = min(i, jj), hi = max(i, jj);
   const double v = (s2[static_cast<size_t>(lo) * n + hi] - s1[i] * s1[jj] / N) / (N - 1.0);
   if (!isfinite(v)) atomicOr(flag, 1);
+  else if (i == jj) atomicMax(expo, (__double2hiint(v) >> 20) & 0x7ff);
   sigma[idx] = v;
 }
 
@@ -215,17 +216,26 @@ __device__ double block_sum(double v, double* red) {
   return red[32];
 }
 
+// A power of two that brings Y = Sigma Q near 1, so that squares of covariances past
+// 2^+-511 stay in range (Q has the same bits); expo: the largest biased exponent of
+// Sigma's diagonal.
+__device__ __forceinline__ double orth_scale(const int* expo) {
+  return ldexp(1.0, -max(-1000, min(1000, *expo - 1022)));
+}
+
 // Q = orth(Y) for the first `rank` columns (zero beyond): classical
 // Gram-Schmidt, each column projected out twice, then normalised.  One block:
 // the general form, for n past what the cluster keeps in shared memory.
 __global__ void __launch_bounds__(kFitThreads)
-orth_kernel(int n, int rank, const double* __restrict__ Y, double* __restrict__ Q) {
+orth_kernel(int n, int rank, const int* expo, const double* __restrict__ Y,
+            double* __restrict__ Q) {
+  const double scale = orth_scale(expo);
   __shared__ double dots[kMaxPcRank];
   __shared__ double red[33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int c = 0; c < kMaxPcRank; ++c) {
     for (int i = threadIdx.x; i < n; i += blockDim.x)
-      Q[static_cast<size_t>(i) * kMaxPcRank + c] = c < rank ? Y[static_cast<size_t>(i) * kMaxPcRank + c] : 0.0;
+      Q[static_cast<size_t>(i) * kMaxPcRank + c] = c < rank ? Y[static_cast<size_t>(i) * kMaxPcRank + c] * scale : 0.0;
     if (c >= rank) continue;
     for (int pass = 0; pass < 2; ++pass) {
       __syncthreads();
@@ -296,7 +306,8 @@ __host__ __device__ constexpr int orth_ld(int n) {   // 8 mod 16: spreads the ba
 }
 
 __global__ void __cluster_dims__(kOrthCtas, 1, 1) __launch_bounds__(kOrthThreads)
-orth_cluster_kernel(int n, int rank, const double* __restrict__ Y, double* __restrict__ Q) {
+orth_cluster_kernel(int n, int rank, const int* expo, const double* __restrict__ Y,
+                    double* __restrict__ Q) {
   extern __shared__ double col[];                      // [32][ld]
   __shared__ double recv[2][kOrthCtas][kMaxPcRank];    // products of each CTA's rows
   __shared__ double coef[kMaxPcRank];                  // products / |q_p|^2
@@ -306,8 +317,9 @@ orth_cluster_kernel(int n, int rank, const double* __restrict__ Y, double* __res
   const int cta = static_cast<int>(blockIdx.x);
   const int ld = orth_ld(n), per = (n + kOrthCtas - 1) / kOrthCtas;
   const int r0 = cta * per, rows = max(0, min(per, n - r0));
+  const double scale = orth_scale(expo);
   for (int e = tid; e < rows * kMaxPcRank; e += kOrthThreads)
-    col[(e & 31) * ld + (e >> 5)] = Y[static_cast<size_t>(r0) * kMaxPcRank + e];
+    col[(e & 31) * ld + (e >> 5)] = Y[static_cast<size_t>(r0) * kMaxPcRank + e] * scale;
   // No CTA writes into another before that one runs.
   tc::cluster_sync_all();
 
@@ -594,7 +606,7 @@ cudaError_t launch_fit_factor(mhar_ctx* c, FitScratch* f, long long samples, int
                               int power_iters) {
   const int n = c->n;
   cov_finalize_kernel<<<blocks_for(static_cast<long long>(n) * n, 256), 256, 0, c->stream>>>(
-      n, static_cast<double>(samples), f->s1, f->s2, f->sigma, f->flag);
+      n, static_cast<double>(samples), f->s1, f->s2, f->sigma, f->flag, f->flag + 1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (rank > 0) {
@@ -616,11 +628,12 @@ cudaError_t launch_fit_factor(mhar_ctx* c, FitScratch* f, long long samples, int
           n, f->sigma, f->Q, f->Y);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if (cluster) {
-        orth_cluster_kernel<<<kOrthCtas, kOrthThreads, smem, c->stream>>>(n, rank, f->Y, f->Q);
+        orth_cluster_kernel<<<kOrthCtas, kOrthThreads, smem, c->stream>>>(n, rank, f->flag + 1,
+                                                                           f->Y, f->Q);
         // A device part without room for sixteen CTAs side by side refuses the launch.
         cluster = cudaGetLastError() == cudaSuccess;
       }
-      if (!cluster) orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->Y, f->Q);
+      if (!cluster) orth_kernel<<<1, kFitThreads, 0, c->stream>>>(n, rank, f->flag + 1, f->Y, f->Q);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     symm_block_kernel<<<blocks_for(n, kSymmRows), kSymmWarps * 32, 0, c->stream>>>(

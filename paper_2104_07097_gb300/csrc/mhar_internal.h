@@ -258,7 +258,8 @@ struct FitScratch {
   double* T = nullptr;       // 32 x 32: Q^T Sigma Q
   double* V = nullptr;       // 32 x 32: its eigenvectors
   double* lam = nullptr;     // 32: its eigenvalues
-  int* flag = nullptr;       // [0] set when a fit kernel met a non-finite value
+  int* flag = nullptr;       // [0] set when a fit kernel met a non-finite value,
+                             // [1] the largest biased exponent of Sigma's diagonal
 };
 cudaError_t launch_fit_shift(mhar_ctx* ctx, FitScratch* f);   // shift = walker 0's point
 cudaError_t launch_fit_accumulate(mhar_ctx* ctx, FitScratch* f);

@@ -34,3 +34,21 @@ def test_overflowing_covariance(n, rank):
         for a, b in zip(smp.preconditioner(), ref.preconditioner()):
             assert np.array_equal(a, b)
         assert np.array_equal(smp.run(3, thin=1), ref.run(3, thin=1))
+
+
+@pytest.mark.parametrize("half", [-300, 300])
+@pytest.mark.parametrize("n,rank", [(5, 1), (20, 7), (64, 32)])
+def test_covariance_of_any_scale(n, rank, half):
+    """Every step of the fit scales exactly with a power of two: moments of points times
+    2^half, whose squared covariances leave FP64's range, give (delta, U) times 2^half."""
+    p = wl.cube(n)
+    s1, s2, count = moments(n, n)
+    out = []
+    for k in (0, half):
+        with mhar.Sampler(p.A, p.b, p.x0, 16, precision="fp64", seed=5) as smp:
+            smp.fit_from_moments(s1 * 2.0 ** k, s2 * 2.0 ** (2 * k), count, rank, 2)
+            delta, U = smp.preconditioner()
+            out.append((delta * 2.0 ** -k, U * 2.0 ** -k))
+    (d0, U0), (d1, U1) = out
+    assert np.abs(U0).max() > 0.0
+    assert np.array_equal(d0, d1) and np.array_equal(U0, U1)
