@@ -939,8 +939,13 @@ __global__ void batch_emit_kernel(const BatchProblem* __restrict__ probs, const 
   }
 }
 
-__global__ void batch_status_kernel(const BatchProblem* __restrict__ probs, int count, int2* gather) {
+// Clearing also zeroes the arrival counters of cut strips: after an expired wait some
+// stand part of the way.
+__global__ void batch_status_kernel(const BatchProblem* __restrict__ probs, int count, int2* gather,
+                                    const BatchCounters counters) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = 0; gather == nullptr && i < counters.sets; ++i)
+    for (int t = q; t < counters.count[i]; t += gridDim.x * blockDim.x) counters.at[i][t] = 0;
   if (q >= count) return;
   int* st = probs[q].status;
   if (gather != nullptr) {
@@ -1817,8 +1822,9 @@ cudaError_t launch_batch_emit(const BatchProblem* probs, int count, long long mo
 }
 
 cudaError_t launch_batch_status(const BatchProblem* probs, int count, int2* gather,
-                                cudaStream_t stream) {
-  batch_status_kernel<<<blocks_for(count, kThreads), kThreads, 0, stream>>>(probs, count, gather);
+                                const BatchCounters& counters, cudaStream_t stream) {
+  batch_status_kernel<<<blocks_for(count, kThreads), kThreads, 0, stream>>>(probs, count, gather,
+                                                                            counters);
   return cudaGetLastError();
 }
 

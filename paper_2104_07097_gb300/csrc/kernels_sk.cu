@@ -1173,7 +1173,15 @@ struct BatchSkPlan {
   int* arrivals = nullptr;
   int n_units = 0;
   int grid = 0;
+  int strips = 0;
 };
+
+void batch_sk_counters(const void* plan_v, BatchCounters* counters) {
+  const BatchSkPlan* plan = static_cast<const BatchSkPlan*>(plan_v);
+  if (!plan) return;
+  counters->at[counters->sets] = plan->arrivals;
+  counters->count[counters->sets++] = plan->strips;
+}
 
 void batch_sk_destroy(void* plan_v) {
   BatchSkPlan* plan = static_cast<BatchSkPlan*>(plan_v);
@@ -1259,6 +1267,7 @@ int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, 
   BatchSkPlan* plan = new BatchSkPlan();
   plan->n_units = static_cast<int>(units.size());
   plan->grid = std::min(sms, plan->n_units);
+  plan->strips = arrivals;
   cudaError_t e = cudaFuncSetAttribute(recompute_batch_sk_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kSmemBsk));

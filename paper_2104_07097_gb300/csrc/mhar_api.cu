@@ -1576,6 +1576,7 @@ int mhar_check(mhar_ctx* c, mhar_stats* s) {
 // balance between a unit's set-up and walker-side work and its MMAs, and
 // with it the best launch shape, changes from bucket to bucket.
 constexpr int kBatchBuckets = 5;
+static_assert(kBatchBuckets <= mhar::kBatchCounters, "a set of arrival counters for each bucket");
 
 int batch_bucket_of(const mhar_ctx* c) {
   const int kc = c->k_pad / mhar::kTcKChunk;
@@ -1723,6 +1724,16 @@ int batch_set_shape(mhar_batch* b, int C) {
                                             &b->table, &b->units, b->err, sizeof(b->err));
   if (rc == MHAR_OK) b->C = C;
   return rc;
+}
+
+// The arrival counters of the persistent launches in use.
+mhar::BatchCounters batch_counters(const mhar_batch* b) {
+  mhar::BatchCounters a;
+  if (!b->per_bucket)
+    mhar::batch_sk_counters(b->sk, &a);
+  else
+    for (const BatchBucket& k : b->buckets) mhar::batch_sk_counters(k.sk, &a);
+  return a;
 }
 
 cudaError_t batch_enqueue(mhar_batch* b, int count) {
@@ -1906,6 +1917,20 @@ int mhar_batch_create(const mhar_problem* problems, int32_t count, int32_t z,
   return MHAR_OK;
 }
 
+// For tests: every arrival counter of the persistent launches at `value`, as an expired
+// wait may leave it.  Returns how many there are.
+int mhar_test_batch_arrivals(mhar_batch* b, int32_t value) {
+  int total = 0;
+  const mhar::BatchCounters a = batch_counters(b);
+  for (int i = 0; i < a.sets; ++i) {
+    const std::vector<int> v(a.count[i], value);
+    if (cudaMemcpy(a.at[i], v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+      return -1;
+    total += a.count[i];
+  }
+  return total;
+}
+
 int mhar_batch_tune(mhar_batch* b, int32_t iters, int32_t* cluster) {
   if (!b || iters < 1 || iters > 1024) return MHAR_E_ARG;
   int max_tiles = 1;
@@ -2024,7 +2049,8 @@ int mhar_batch_run(mhar_batch* b, int64_t steps, int64_t thin, double* const* ou
   }
   const int problems = static_cast<int>(b->ctx.size());
   {
-    cudaError_t e = mhar::launch_batch_status(b->probs, problems, nullptr, b->stream);
+    cudaError_t e = mhar::launch_batch_status(b->probs, problems, nullptr, batch_counters(b),
+                                              b->stream);
     if (e != cudaSuccess) return batch_cuda(b, e, "status reset");
   }
   int64_t done = 0, emitted = 0;
@@ -2077,7 +2103,7 @@ int mhar_batch_run(mhar_batch* b, int64_t steps, int64_t thin, double* const* ou
   int worst = MHAR_OK;
   std::vector<int2> words(b->ctx.size());
   {
-    cudaError_t e = mhar::launch_batch_status(b->probs, problems, b->status, b->stream);
+    cudaError_t e = mhar::launch_batch_status(b->probs, problems, b->status, {}, b->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(words.data(), b->status, sizeof(int2) * words.size(),
                           cudaMemcpyDeviceToHost, b->stream);

@@ -243,7 +243,16 @@ struct BatchOuts {
 };
 cudaError_t launch_batch_emit(const BatchProblem* probs, int count, long long most,
                               const BatchOuts& outs, cudaStream_t stream);
+// Arrival counters of the batch's persistent launches: one set for the whole batch or one
+// a bucket.
+constexpr int kBatchCounters = 8;
+struct BatchCounters {
+  int* at[kBatchCounters];
+  int count[kBatchCounters];
+  int sets = 0;
+};
 cudaError_t launch_batch_status(const BatchProblem* probs, int count, int2* gather,
+                                const BatchCounters& counters,
                                 cudaStream_t stream);   // gather null: clear
 
 // ---- preconditioner fit (kernels_fit.cu) --------------------------------------
@@ -300,6 +309,7 @@ cudaError_t launch_recompute_batch(const void* table, int units, int C, int j,
 // batch's (problem, strip, row tile) work cut into cost-balanced ranges.
 int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan, char* err, size_t err_len);
 void batch_sk_destroy(void* plan);
+void batch_sk_counters(const void* plan, BatchCounters* counters);   // adds the plan's set
 cudaError_t launch_recompute_batch_sk(const void* plan, int j, cudaStream_t stream);
 // The batch kernels leave the walker-side work (the moves and the FP16 pairs
 // of the moved points, walker_tail.cuh) to one update launch per iteration
