@@ -27,6 +27,7 @@
 // 64 x 500, 100 walkers 8.8 (137); 100 x 390, 20 walkers 11.6 (164); FP32 2.3,
 // 9.1, 4.2, 4.5 and 5.9 us.  What is left is latency: the serial FP64 sums and
 // division, and five barriers.
+#include <cfloat>
 #include <cmath>
 #include <cuda_fp16.h>
 #include <type_traits>
@@ -385,8 +386,9 @@ small_kernel(const SmallParams<T> p, int G, int R) {
             const float s = fmaxf(bf - ax[q] - fmaf(ga, nx, 0x1p-22f * fabsf(bf)), 0.0f) *
                             (1.0f - 0x1p-20f);
             const float dh = fmaf(ga, nd, ad[q]), dl = fmaf(ga, nd, -ad[q]);
-            const float bh = dh > 0.0f ? s * rcp_approx(dh) : INFINITY;
-            const float bl = dl > 0.0f ? s * rcp_approx(dl) : INFINITY;
+            // A quotient past FP32's range (short directions) is still a row's.
+            const float bh = dh > 0.0f ? fminf(s * rcp_approx(dh), FLT_MAX) : INFINITY;
+            const float bl = dl > 0.0f ? fminf(s * rcp_approx(dl), FLT_MAX) : INFINITY;
             lbs[(2 * g) * m + r] = bh;
             lbs[(2 * g + 1) * m + r] = bl;
             if (bh < INFINITY)
