@@ -42,6 +42,7 @@
 
 #include "mhar_device.cuh"
 #include "mhar_internal.h"
+#include "screen_row.cuh"
 #include "tc_common.cuh"
 
 namespace mhar {
@@ -55,6 +56,7 @@ constexpr int kWBytes = 4 * kOperandBytes;           // Dh, Dl, Xh, Xl
 constexpr int kABytes = 2 * kOperandBytes;           // A hi, A lo
 constexpr int kEpiWarps = 16;
 constexpr int kPWarp = 2 + kEpiWarps;
+static_assert(kRowsTile == 128 && kEpiWarps == 16, "screen_row's tiles and streams");
 constexpr int kThreadsScr = (3 + kEpiWarps) * 32;
 constexpr unsigned int kNone = 0x7f800000u;          // a bound at or above +Inf: no row
 
@@ -699,9 +701,7 @@ screen_finish_kernel(const FinParams<T> p) {
     if (!__any_sync(0xffffffffu, has)) break;
     int row = 0;
     if (has) {
-      const unsigned int t = p.tiles[static_cast<size_t>(bst) * p.z_ld + kc];
-      row = static_cast<int>(side ? t >> 16 : t & 0xffffu) * kRowsTile + (bst & 3) * 32 +
-            static_cast<int>(b1 & 31u);
+      row = screen_row(p.tiles[static_cast<size_t>(bst) * p.z_ld + kc], side != 0, bst, b1, p.m);
       last = b1;
       last_st = bst;
     }
