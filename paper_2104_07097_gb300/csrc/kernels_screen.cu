@@ -37,6 +37,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -872,14 +873,26 @@ screen_finish_kernel(const FinParams<T> p) {
   }
 }
 
-// CTAs along the rows: as many as the SMs leave for each walker strip.
+// CTAs along the rows: up to what the SMs leave for each walker strip, the number with
+// the least time estimated from a CTA's tiles (2700 clocks for the epilogue, no less than
+// six MMAs of 85 a K step) and 850 clocks for each four streams more that the finish goes
+// through.  As many as there are SMs, with few walkers, was slower than the direct FP32
+// kernel: an iteration of 65 walkers of an 8000 x 64 body 72 us with 63 CTAs along the
+// rows, 35 with 16 (21: 35, 8: 39; direct 26); of 300 of a 4000 x 64 body 39 and 31 (39).
 int screen_tiles_per_cta(const mhar_ctx* c) {
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   const int strips = (c->z + kWalkers - 1) / kWalkers, tiles = c->m_pad / kRowsTile;
-  int C = sms / strips;
-  C = C < 1 ? 1 : (C > tiles ? tiles : C);
-  return (tiles + C - 1) / C;
+  const int most = std::max(1, std::min(sms / strips, tiles));
+  const long long tile = std::max(2700, 6 * 85 * (c->kdim / kTcK));
+  int per = tiles;
+  long long best = 0;
+  for (int C = 1; C <= most; ++C) {
+    const int t = (tiles + C - 1) / C;
+    const long long est = t * tile + 850ll * C;
+    if (best == 0 || est < best) { best = est; per = t; }
+  }
+  return per;
 }
 
 template <typename T>
@@ -943,11 +956,14 @@ cudaError_t launch_screen_t(mhar_ctx* c, int j, const T* A, const T* b, const T*
 
 }  // namespace
 
-// Bodies past the warp-per-walker path.  The screen's three launches take about
-// 19 us whatever the body; the direct FP64 kernel 200 us and more from there on
-// (10 to 76 times the screen's over n = 3 .. 200, m = 700 .. 4000, z = 1000 ..
-// 4096), the direct FP32 kernel 18 us at m z = 10^6 and n <= 32 (the screen
-// 19.4 .. 20.2), 25 against 23 at n = 64, and 90 against 26 .. 35 at m z = 8 10^6.
+// Bodies past the warp-per-walker path; times of whole iterations, draw included.  FP64:
+// 203 us and more with the direct kernel, 25 .. 88 with the screen (n = 4 .. 100, m = 700
+// .. 4000, z = 300 .. 4096).  FP32, the screen against the direct kernel, by the products
+// m n z from n = 64 on: 35 / 26 us at 33 10^6 (65 walkers, 8000 x 64), 27 / 27 at 38 10^6
+// (300, 2000 x 64), 24 / 27 at 41 10^6 (640, 1000 x 64), 34 / 50 at 115 10^6 (300, 4000 x
+// 96); a single strip of walkers 37 / 32 at 50 10^6 (65, 8000 x 96), 39 / 40 at 67 10^6.
+// Fewer columns take the direct kernel longer than their products say: 25 / 21 at m z =
+// 1.5 10^6, 26 / 45 at 3 10^6 (n = 16, 32).
 // Of the bodies with fewer 64 x 64 tiles than SMs, in FP64 those that the small-body
 // kernel does not take (equalities, A past its shared memory) where a warp's serial
 // sums (n terms for every 32 rows) or all the products are many.  An iteration with
@@ -961,8 +977,9 @@ bool screen_eligible(const mhar_ctx* c) {
     return c->opts.precision == MHAR_FP64 &&
            (static_cast<long long>(c->n) * ((c->m + 31) / 32) >= 128 ||
             static_cast<long long>(c->m) * c->n * c->z >= 1ll << 21);
-  return c->opts.precision == MHAR_FP64 || c->n >= 64 ||
-         static_cast<long long>(c->m) * c->z >= 1ll << 21;
+  if (c->opts.precision == MHAR_FP64) return true;
+  const long long mz = static_cast<long long>(c->m) * c->z;
+  return c->n >= 64 ? mz * c->n >= (c->z <= kWalkers ? 1ll << 26 : 1ll << 25) : mz >= 1ll << 21;
 }
 
 size_t screen_arena(mhar_ctx* c, uint8_t* base) {
