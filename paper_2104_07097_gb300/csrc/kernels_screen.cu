@@ -465,6 +465,8 @@ struct FinParams {
   double* lmax;
   double* theta;
   int* status;
+  unsigned long long* slow;  // screen_slow
+  int slow_at;               // walkers of a warp outside the range
   unsigned long long* counters;
   double* X64;
   float* Xhi;
@@ -761,8 +763,10 @@ screen_finish_kernel(const FinParams<T> p) {
     if (!__syncthreads_or(next < p.streams)) break;
   }
   lam = fmin(lam, __longlong_as_double(static_cast<long long>(again_s[threadIdx.x >> 1])));
-  // Walkers outside the screen's range: every row.
+  // Walkers outside the screen's range: every row, one walker after the other.
   unsigned int forced = __ballot_sync(0xffffffffu, force && t4 == 0);
+  if (lane == 0 && __popc(forced) >= p.slow_at)
+    atomicMax(p.slow, static_cast<unsigned long long>(*p.step_ptr + static_cast<uint64_t>(p.j) + 1ull));
   while (forced) {
     const int src = __ffs(forced) - 1;
     forced &= forced - 1;
@@ -949,6 +953,13 @@ cudaError_t launch_screen_t(mhar_ctx* c, int j, const T* A, const T* b, const T*
   f.lmin = d.lmin; f.lmax = d.lmax; f.theta = d.theta; f.status = d.status; f.counters = d.counters;
   f.X64 = d.X64; f.Xhi = d.Xhi; f.Xlo = d.Xlo; f.Q32 = d.Q32;
   f.corr = sizeof(T) == 4 ? d.corr : nullptr;
+  // From so many walkers of the eight of a warp on, the direct kernels take less time: an
+  // iteration with 1, 2, 3, 4 of them 1180, 2290, 3400, 4510 us for 4096 walkers of a 2000 x
+  // 100 body in FP64 (direct 4160), 162, 294, 427, 561 for 3001 of a 700 x 20 body (410);
+  // FP32 with one 535 (239) and 82 (35); with a warp a walker, 20 of a 1500 x 100 body, one
+  // 808 (570).
+  f.slow = screen_slow(d);
+  f.slow_at = sizeof(T) == 8 && !simt_warp_path(c) ? 3 : 1;
   screen_finish_kernel<T>
       <<<(c->z + kFinWalkers - 1) / kFinWalkers, kFinThreads, kFinSmem, c->stream>>>(f);
   return cudaGetLastError();

@@ -241,6 +241,9 @@ bool tail_draws(const mhar_ctx* c) {
   return recompute(c) && c->mE == 0 && (c->pc_rank < 0 || c->use_ts);
 }
 
+// FP64 / FP32 modes: whether the next iteration's chord is screened.
+bool screened(const mhar_ctx* c) { return c->use_screen && c->direct_left == 0; }
+
 // The stored-slack kernel does so in a launch of many iterations.
 bool stored_loop(const mhar_ctx* c) { return stored(c) && c->mE == 0 && c->pc_rank < 0; }
 
@@ -255,7 +258,7 @@ bool projection_draws(const mhar_ctx* c) {
 // the update kernel unless one warp per walker does both.
 int chord_launches(const mhar_ctx* c) {
   if (recompute(c)) return (!c->use_ts && c->use_sk) ? 2 : 1;
-  if (c->use_screen) return 3;
+  if (screened(c)) return 3;
   return (mixed(c) || mhar::simt_warp_path(c)) ? 1 : 2;
 }
 
@@ -294,7 +297,7 @@ cudaError_t enqueue_chord(mhar_ctx* c, int j) {
     if (c->use_ts) return mhar::launch_recompute_ts(c, j);
     return c->use_sk ? mhar::launch_recompute_sk(c, j) : mhar::launch_recompute_tc(c, j);
   }
-  if (c->use_screen) return mhar::launch_screen(c, j);
+  if (screened(c)) return mhar::launch_screen(c, j);
   if (mhar::simt_warp_path(c)) return mhar::launch_chord_update_warp(c, j);
   cudaError_t e = mhar::launch_chord_simt(c);
   return e == cudaSuccess ? mhar::launch_update_simt(c, j) : e;
@@ -383,10 +386,63 @@ int advance_loop(mhar_ctx* c, int64_t count, double* out, int64_t thin, int64_t 
   return MHAR_OK;
 }
 
+void drop_graphs(mhar_ctx* c) {
+  if (c->g_chunk) cudaGraphExecDestroy(c->g_chunk);
+  if (c->g_one) cudaGraphExecDestroy(c->g_one);
+  c->g_chunk = nullptr;
+  c->g_one = nullptr;
+  c->graph_len = 0;
+}
+
+// Screened contexts.  Walkers whose coordinates or directions lie outside the screen's
+// range have all their rows evaluated one walker after the other, up to 16 times the time
+// of the direct kernels when it is all of them (bodies of size 1e-17, say).  The finish
+// notes the last iteration in which that was slower (screen_slow).  The host looks after
+// the first kScreenFirst iterations from a new state, then every kScreenLook and at the
+// end of each call, and goes over to the direct kernels -- the same bits -- for 4, 16, 64
+// .. 1024 iterations, with a screened one as a trial between the stretches.  A look takes
+// a synchronisation, 10 us.
+constexpr int64_t kScreenLook = 256;
+
+void screen_restart(mhar_ctx* c) {
+  c->direct_left = c->direct_len = 0;
+  c->screen_left = mhar::kScreenFirst;
+}
+
+void screen_decide(mhar_ctx* c, unsigned long long slow) {
+  if (slow == c->step) {
+    c->direct_len = c->direct_len == 0 ? 4 : std::min<int64_t>(4 * c->direct_len, 1024);
+    c->direct_left = c->direct_len;
+  } else {
+    c->direct_len = 0;
+    c->screen_left = kScreenLook;
+  }
+}
+
+// After `done` iterations of one kind (c->step counts them).
+int screen_look(mhar_ctx* c, int64_t done) {
+  if (c->direct_left > 0) {
+    c->direct_left -= done;
+    if (c->direct_left == 0) c->screen_left = 1;
+    return MHAR_OK;
+  }
+  c->screen_left -= done;
+  if (c->screen_left > 0) return MHAR_OK;
+  unsigned long long slow = 0;
+  MHAR_CUDA(cudaMemcpyAsync(&slow, mhar::screen_slow(c->d), sizeof(slow), cudaMemcpyDeviceToHost,
+                            c->stream), "status copy");
+  MHAR_CUDA(cudaStreamSynchronize(c->stream), "status sync");
+  screen_decide(c, slow);
+  return MHAR_OK;
+}
+
 int advance(mhar_ctx* c, int64_t count) {
   int frc = ensure_operands(c);
   if (frc) return frc;
-  if (c->opts.graph_chunk <= 0) {
+  // A single screened iteration between stretches of direct ones has no graph of its own.
+  const bool trial = screened(c) && c->direct_len > 0;
+  if (c->g_one && !trial && c->graphs_direct != (c->direct_left > 0)) drop_graphs(c);
+  if (c->opts.graph_chunk <= 0 || trial) {
     while (count > 0) {
       const int now = count > (1 << 20) ? (1 << 20) : static_cast<int>(count);
       int rc = enqueue_iterations(c, now);
@@ -402,6 +458,7 @@ int advance(mhar_ctx* c, int64_t count) {
     rc = capture(c, c->opts.graph_chunk, &c->g_chunk);
     if (rc != MHAR_OK) return rc;
     c->graph_len = c->opts.graph_chunk;
+    c->graphs_direct = c->direct_left > 0;
     c->launches_one = kernels_per_iteration(c) + 1;
     c->launches_chunk = static_cast<int64_t>(c->graph_len) * kernels_per_iteration(c) + 1;
   }
@@ -452,14 +509,6 @@ int emit_to(mhar_ctx* c, double* out, bool out_device, int walkers) {
   return MHAR_OK;
 }
 
-void drop_graphs(mhar_ctx* c) {
-  if (c->g_chunk) cudaGraphExecDestroy(c->g_chunk);
-  if (c->g_one) cudaGraphExecDestroy(c->g_one);
-  c->g_chunk = nullptr;
-  c->g_one = nullptr;
-  c->graph_len = 0;
-}
-
 // Makes (delta, U, sigma) current: padded copies are on the device already;
 // re-splits A with the new coordinate scales and, in the stored-slack mode,
 // recomputes the slack from the points.
@@ -467,6 +516,7 @@ int adopt_preconditioner(mhar_ctx* c, int rank) {
   c->pc_rank = rank;
   c->operands_fresh = false;
   drop_graphs(c);
+  screen_restart(c);
   if (mixed(c)) {
     MHAR_CUDA(mhar::launch_prepare_tc_operands(c), "operand preparation kernel");
     ++c->launches;
@@ -824,7 +874,7 @@ const char* mhar_kernel_name(const mhar_ctx* c) {
   if (recompute(c)) return c->use_ts ? "recompute_ts_kernel" : (c->use_sk ? "recompute_sk_kernel" : "recompute_tc_kernel");
   if (stored(c)) return "walker_tc_kernel";
   if (c->use_small) return "small_kernel";
-  if (c->use_screen) return "screen_kernel";
+  if (screened(c)) return "screen_kernel";
   return mhar::simt_warp_path(c) ? "chord_warp_kernel" : "chord_simt_kernel";
 }
 
@@ -1000,7 +1050,7 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
                            std::min<int64_t>(16ll * emit_count(c) * n, (4ll << 20) / 8));
   if ((rc = dmalloc(c, &d.key_lo, z)) || (rc = dmalloc(c, &d.key_hi, z)) ||
       (rc = dmalloc(c, &d.lmin, z)) || (rc = dmalloc(c, &d.lmax, z)) ||
-      (rc = dmalloc(c, &d.theta, z)) || (rc = dmalloc(c, &d.status, 2)) ||
+      (rc = dmalloc(c, &d.theta, z)) || (rc = dmalloc(c, &d.status, 4)) ||
       (rc = dmalloc(c, &d.counters, 2)) || (rc = dmalloc(c, &d.step, 1)) ||
       (rc = dmalloc(c, &d.emit, static_cast<size_t>(c->emit_cap))) || (rc = dmalloc(c, &d.check, 6)))
     return rc;
@@ -1166,14 +1216,17 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
     return MHAR_E_ARG;
   }
   if (steps == 0) return MHAR_OK;
-  MHAR_CUDA(cudaMemsetAsync(c->d.status, 0, 2 * sizeof(int), c->stream), "status reset");
+  MHAR_CUDA(cudaMemsetAsync(c->d.status, 0, 4 * sizeof(int), c->stream), "status reset");
   int rc;
   if (stored(c) && (rc = reset_drift(c))) return rc;
   int64_t done = 0, emitted = 0;
   const int64_t k = stored(c) ? c->opts.refresh_k : 0;
   const int64_t au = c->opts.audit_every;
+  bool last_screened = false;
   while (done < steps) {
     int64_t adv = steps - done;
+    if (c->use_screen)
+      adv = std::min(adv, c->direct_left > 0 ? c->direct_left : c->screen_left);
     // A kernel that runs many iterations writes samples itself: all of a call's
     // when they stay on the device, else as many as the staging buffer holds at a
     // time (one at a time, a launch and a copy each, took 30 us a sample).
@@ -1196,6 +1249,8 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
     if (rc) return rc;
     done += adv;
     c->step += static_cast<uint64_t>(adv);
+    last_screened = screened(c);
+    if (c->use_screen && (rc = screen_look(c, adv))) return rc;
     // Out of the staging buffer before the audit takes it as its scratch.
     if (fused && !whole && done / thin > before / thin)
       MHAR_CUDA(cudaMemcpyAsync(out + static_cast<size_t>(before / thin) * sample, c->d.emit,
@@ -1217,10 +1272,15 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
       ++emitted;
     }
   }
-  int st[2] = {0, 0};
+  int st[4] = {0, 0, 0, 0};
   MHAR_CUDA(cudaMemcpyAsync(st, c->d.status, sizeof(st), cudaMemcpyDeviceToHost, c->stream),
             "status copy");
   MHAR_CUDA(cudaStreamSynchronize(c->stream), "run sync");
+  if (last_screened && screened(c)) {      // else the look after its last iteration decided
+    unsigned long long slow;
+    std::memcpy(&slow, st + 2, sizeof(slow));
+    screen_decide(c, slow);
+  }
   if (stored(c)) {
     unsigned long long kd = 0;
     MHAR_CUDA(cudaMemcpy(&kd, reinterpret_cast<unsigned long long*>(c->d.check) + 2, sizeof(kd),
@@ -1266,6 +1326,7 @@ int mhar_set_state(mhar_ctx* c, const double* X, uint64_t step) {
             "copy X");
   MHAR_CUDA(mhar::launch_set_points(c, c->d.emit), "set points kernel");
   c->operands_fresh = false;
+  screen_restart(c);
   MHAR_CUDA(cudaMemcpyAsync(c->d.step, &step, sizeof(step), cudaMemcpyHostToDevice, c->stream),
             "copy step");
   c->step = step;
