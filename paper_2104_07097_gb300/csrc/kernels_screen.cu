@@ -23,16 +23,17 @@
 //      the ratio found (screen_finish_kernel; when a stream's second bound does
 //      not, the bounds of its rows are formed again in FP32 by the block), then
 //      draws theta and moves the walker as update_kernel does.
-// On a 2000 x 100 body with 4096 walkers an iteration's chord and move take 55 to 65
-// us in FP64 (4131 us with chord_simt_kernel<double>, 63 % of the FP64 pipe) and 50
-// in FP32 (234 us): split 7 .. 9, screen 18 (the MMAs of 12 m n z flops and their
-// epilogue, as in the recompute kernels), finish 21 .. 39 (latency of the serial
-// sums; 27 .. 87 before the second look at a stream's bounds).
+// On a 2000 x 100 body with 4096 walkers an iteration's chord and move take 48 us in
+// FP64 (4131 us with chord_simt_kernel<double>, 63 % of the FP64 pipe) and 36 in FP32
+// (234 us), after a draw of 24 and 2.5 us: split 7.8 and 5.5, screen 15.8 (the MMAs of
+// 12 m n z flops and their epilogue, as in the recompute kernels), finish 24.3 and 14.8
+// (latency of the serial sums).
 // So the chord ends, theta and the points have the bits of the direct
 // kernels.  Rows that tie within the bounds (duplicate rows, walkers on a
 // facet) cost more evaluations, never a different result.  Values the bounds
 // do not cover (outside 2^-50 .. 2^50) take the direct formulas: a body at
-// creation, a walker by its flag (`force`).
+// creation, a walker by its flag (`force`), a context whose walkers are mostly such ones
+// by the host (screen_look, mhar_api.cu).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -496,9 +497,9 @@ __device__ __forceinline__ T dot_in_order(const T* __restrict__ a, const T* v, i
 // a . d)): the 16 rows, 8 points and 8 directions come into shared memory 128
 // bytes of each at a time, whole lines, kFinStages steps ahead.  Read by the threads
 // themselves each 16 bytes took a line of its own (136 clocks a term in FP64, 59 in
-// FP32); with this and the move's loads in batches an iteration of the 2000 x 100
-// body takes 41 us in FP32 (44.5 before) and 85.6 in FP64 (87.9, bound by the FP64
-// chain).
+// FP32); with this and the move's loads in batches an iteration of a call on the 2000 x
+// 100 body, draw and the call's own launches included, takes 41 us in FP32 (44.5 before)
+// and 85.6 in FP64 (87.9, bound by the FP64 chain).
 constexpr int kFinStages = 4;
 constexpr int kFinRow = 144;                       // bytes between two staged pieces
 constexpr int kFinDir = 24 * kFinRow + 64;         // the directions, off the points' banks

@@ -15,18 +15,18 @@
 //     thread per row, the sums in index order -- the arithmetic and the bits of
 //     chord_warp_kernel.
 //   Chord, screened (FP64): a lower bound of every row's ratio from FP32 dot
-//     products and the standard bound gamma_{n+6} ||a_i|| ||x|| on their errors
+//     products and the standard bound gamma_{n+8} ||a_i|| ||x|| on their errors
 //     (kernels_screen.cu does the same on the tensor cores), then FP64 in index
 //     order for the least one and for every row whose bound does not exceed the
 //     ratio found: FP64 runs at 1/64 of the FP32 rate, and the 300 rows of a
 //     37-dimensional body need two.  Walkers whose coordinates leave the range
 //     the bound covers evaluate every row in FP64.
-// Measured per iteration, launches of 256 iterations (before: a draw and
-// chord_warp_kernel each, in a graph): FP64 10 x 20, 100 walkers 3.7 us (16.5);
-// 8000 walkers 24 (209, chord_simt_kernel); 37 x 300, 301 walkers 6.9 (62);
-// 64 x 500, 100 walkers 8.8 (137); 100 x 390, 20 walkers 11.6 (164); FP32 2.3,
-// 9.1, 4.2, 4.5 and 5.9 us.  What is left is latency: the serial FP64 sums and
-// division, and five barriers.
+// Measured per iteration, launches of 1024 iterations (before: a draw and
+// chord_warp_kernel each, in a graph): FP64 10 x 20, 100 walkers 2.6 us (16.5);
+// 8000 walkers 22 (209, chord_simt_kernel); 37 x 300, 301 walkers 7.3 (62);
+// 64 x 500, 100 walkers 9.8 (137); 100 x 390, 20 walkers 13.3 (164); FP32 2.3,
+// 9.1, 4.1, 4.5 and 5.9 us.  What is left is latency: the serial FP64 sums and
+// division, and four barriers of the block (six screened).
 #include <cfloat>
 #include <cmath>
 #include <cuda_fp16.h>

@@ -586,8 +586,6 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
                  min(p.draw_chunks * w_count, quads / 2), kDrawThreads, tail, state);
     } else {
       // ---- epilogue: s = b - p, ratios, per-walker partial chord ------------------
-      // First, while the first row tiles are on their way: iteration s+1's
-      // directions into the other pair (walker_tail.cuh, step 0).
       const int e = warp - 2;
       const int q = warp & 3;
       const int cg = e >> 2;              // 32-column group of each 128-column tile
@@ -611,7 +609,7 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
       const int k = strip * kWalkers + wl;
       const float ws = __ldcg(p.wscale + k);
       // The operand norms of this thread's walker (written by the warps that
-      // loaded the operands into tensor memory, before the draw above).
+      // loaded the operands into tensor memory).
       named_bar<kEpiWarps * 32>();
       WalkerNorms wn;
       wn.nd2 = tail->nrm[0][wl];

@@ -1965,8 +1965,9 @@ int mhar_batch_create(const mhar_problem* problems, int32_t count, int32_t z,
   if (rc == MHAR_OK) rc = batch_buckets_init(b);
   if (rc == MHAR_OK) {
     // Default shape: the persistent launch, whose units are cut to balance the SMs
-    // (clusters of one size for every body: 2 to 4 times its time on uneven bodies,
-    // 0.9 of it at best, on 48 small bodies of four strips).
+    // (clusters of one size for every body: 2 to 4 times its time on uneven bodies; one
+    // CTA a unit 0.94 .. 1.02 of a call of 16 iterations on 40 .. 300 small bodies of
+    // nearly one size, 609 against 647 us at the best, 100 bodies of 20 to 40 dimensions).
     rc = batch_set_shape(b, 0);
   }
   if (rc != MHAR_OK) {
