@@ -443,8 +443,10 @@ const char* mhar_batch_last_error(const mhar_batch* batch);
 /* Frees the batch and every problem's device memory; NULL is ignored. */
 void mhar_batch_destroy(mhar_batch* batch);
 
-/* Name of the kernel that runs the chord of one iteration on this context
- * (e.g. "recompute_ts_kernel"); never NULL. */
+/* Name of the kernel that runs the chord of the next iteration on this context
+ * (e.g. "recompute_ts_kernel"); never NULL.  In the FP64 / FP32 modes it follows
+ * the walkers: while many lie outside the range of the screened chord, the direct
+ * kernels run, with the same results. */
 const char* mhar_kernel_name(const mhar_ctx* ctx);
 
 /* Human-readable description of the last error on ctx (never NULL); with
