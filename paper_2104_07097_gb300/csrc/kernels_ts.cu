@@ -37,7 +37,7 @@
 //     barrier an iteration remains, behind which the moved points' FP16 pairs and
 //     the next directions are read back from L2.
 // An iteration of n = 100, m = 2000, z = 4096 takes 13.7 us (17.3 with one launch an
-// iteration), n = 40, m = 400 with a rank-32 preconditioner 7.8 (25.7).  Of the 13.7
+// iteration), n = 40, m = 400 with a rank-32 preconditioner 7.6 (25.7).  Of the 13.7
 // (clock64): operands into tensor memory 1.1, four tiles 8.0 (100 cycles an MMA), the
 // exchange and theta 1.0, the move 1.7, the barrier 1.0.  Drawing the directions
 // before the tiles cost 2.4 us, 8 with the preconditioner; a barrier of the
@@ -51,6 +51,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <array>
 #include <cstdio>
 #include <type_traits>
 
@@ -75,6 +76,7 @@ constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kDrawWarp = 2 + kEpiWarps;
 constexpr int kDrawThreads = 64;
 constexpr int kThreadsTs = kDrawWarp * 32 + kDrawThreads;
+constexpr int kThreadsOne = kDrawWarp * 32;          // a single iteration draws nothing
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kOpCol = 256;                     // first TMEM column of the walker operands
 
@@ -393,8 +395,13 @@ __device__ __forceinline__ void ts_move(const WalkerTail& wt, int cur, int strip
 // FP16 each) in the last chunk, 1..4, the other chunk having 4.  A
 // compile-time K structure makes each pass one straight run of MMAs (the
 // issuing thread's stream between MMAs is the limiter).
-template <int KCH, int LAST>
-__global__ void __launch_bounds__(kThreadsTs, 1)
+// RUN: many iterations, and the draws; else one iteration whose directions a kernel
+// before it drew and projected (equalities), without what only the loop needs and without
+// its two cluster barriers.  One kernel for both took an iteration with an equality 22.5 us
+// on 294 walkers of a 2229 x 51 body, 18.1 now, 30.5 and 27.3 on 4096 of a 2000 x 100 body;
+// the loop gains too (illcond40x400 with rank 32, 100 iterations: 785 -> 764 us).
+template <int KCH, int LAST, bool RUN>
+__global__ void __launch_bounds__(RUN ? kThreadsTs : kThreadsOne, 1)
 recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
                     const __grid_constant__ TsParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -437,7 +444,12 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
   }
   tc_fence_before();
   __syncwarp();
-  cluster_sync_all();   // every CTA's barriers are ready
+  if constexpr (RUN) {
+    cluster_sync_all();   // every CTA's barriers are ready
+  } else {
+    cluster_arrive();     // waited for before the first message to one of them
+    __syncthreads();
+  }
   tc_fence_after();
   const uint32_t tmem = tail->tmem_base;
   volatile int* timed_out = &tail->timed_out;
@@ -449,22 +461,25 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
   const int tid = static_cast<int>(threadIdx.x) - 64;   // of the epilogue, then the draw threads
   const int my_c = tid / w_count, my_w = tid - my_c * w_count;   // a resident thread's item
   const int theta_threads = (w_count + 31) & ~31;
-  const int quads = p.wt.draw ? ((p.wt.n + 7) >> 3) * 2 * w_count : 0;
+  const int quads = RUN && p.wt.draw ? ((p.wt.n + 7) >> 3) * 2 * w_count : 0;
   const int epi_draws = kEpiThreads - theta_threads;             // threads that draw after the tiles
-  uint4* state = p.resident ? reinterpret_cast<uint4*>(stage) : nullptr;
-  if (tid >= 0 && tid < kWalkers) {
-    const bool in = tid < p.wt.n_ld;
-    tail->sigma[tid] = in ? p.wt.sigma[tid] : 1.0f;
-    tail->delta[tid] = in && p.wt.pc_rank >= 0 ? p.wt.pc_delta[tid] : 0.0f;
+  uint4* state = RUN && p.resident ? reinterpret_cast<uint4*>(stage) : nullptr;
+  const int iters = RUN ? p.iters : 1;
+  if constexpr (RUN) {
+    if (tid >= 0 && tid < kWalkers) {
+      const bool in = tid < p.wt.n_ld;
+      tail->sigma[tid] = in ? p.wt.sigma[tid] : 1.0f;
+      tail->delta[tid] = in && p.wt.pc_rank >= 0 ? p.wt.pc_delta[tid] : 0.0f;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   if (state != nullptr && warp >= 2 && warp < kDrawWarp)
     ts_load_state(p.wt, static_cast<int>(step0 & 1ull), strip, p.z, w_begin, w_count, tid, state);
   int pu = 0;                // producer: pair uses issued
   int p0 = 0;                // MMA thread: first pair use of the tile
   int g = 0;                 // tiles of the iterations before
 #pragma unroll 1
-  for (int it = 0; it < p.iters; ++it, g += ntiles) {
+  for (int it = 0; it < iters; ++it, g += ntiles) {
     const uint64_t step = step0 + static_cast<uint64_t>(it);
     const int cur = static_cast<int>(step & 1ull);  // this iteration's direction pair
 
@@ -532,7 +547,7 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
         // This iteration's tiles and the first of the next one's, which then
         // arrive while the walkers move.
         const int per = ntiles * KCH;
-        const int end = min(p.iters * per, (it + 1) * per + kPairs);
+        const int end = min(iters * per, (it + 1) * per + kPairs);
         for (; pu < end; ++pu) {
           const int s = pu % kPairs, nt = (pu / KCH) % ntiles, kc = pu % KCH;
           const int yr = row_base + nt * kTile;
@@ -647,6 +662,10 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
       }
       // The partial chord to the CTA that holds the walker: the data and its
       // arrival in one message (a cluster barrier took 1500 cycles here).
+      if constexpr (!RUN) {
+        __syncwarp();
+        cluster_wait();
+      }
       {
         const int owner = wl / share;
         push2(&tail->recv[(4 * static_cast<int>(rank) + cg) * share + wl - owner * share],
@@ -673,7 +692,7 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
             t = static_cast<float>(static_cast<double>(L) +
                                    u * (static_cast<double>(H) - static_cast<double>(L)));
           }
-          if (it + 1 == p.iters) {
+          if (it + 1 == iters) {
             p.lmin[kk] = L;
             p.lmax[kk] = H;
             p.theta[kk] = t;
@@ -695,12 +714,12 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
       named_bar<kEpiThreads>();
       // Algorithm 2's thinning: a sample after this iteration?
       const int done = p.phase + it + 1;
-      double* out = p.out != nullptr && done % p.thin == 0
+      double* out = RUN && p.out != nullptr && done % p.thin == 0
                         ? p.out + static_cast<size_t>(done / p.thin - 1) * p.emit * p.n
                         : nullptr;
       if (state != nullptr) {
         ts_move_resident(p.wt, cur, strip, p.z, w_begin, my_c, my_w, tid, tail, state, out, p.emit,
-                         it + 1 == p.iters);
+                         it + 1 == iters);
       } else {
         ts_move(p.wt, cur, strip, p.z, w_begin, w_count, tid, tail, stage);
         if (out != nullptr) {   // this CTA's walkers, a warp per row
@@ -721,7 +740,22 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
     // ready for the next iteration (at the end: no message is still under way).
     tc_fence_before();
     __syncwarp();
-    cluster_sync_all();
+    if constexpr (RUN) {
+      cluster_sync_all();
+    } else {
+      // Every message to this CTA has arrived (c_full), and no other reads of it: nothing
+      // to wait for but its own warps.
+      if (warp < 2) cluster_wait();
+      __syncthreads();
+      if (*timed_out) {
+        // An expired wait: messages may still be on their way.  Until the other CTAs are
+        // here or have ended, and a bounded while for the messages.
+        cluster_sync_all();
+        if (threadIdx.x == 0)
+          for (int i = 0; i < (1 << 14) && !mbar_try_wait(smem_u32(&tail->c_full), 0u); ++i) {}
+        __syncthreads();
+      }
+    }
     tc_fence_after();
   }
 
@@ -731,7 +765,7 @@ recompute_ts_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_cons
                  : "memory");
   }
   if (p.step_out != nullptr && threadIdx.x == 0 && rank == 0 && strip == 0)
-    *p.step_out = step0 + static_cast<uint64_t>(p.iters);
+    *p.step_out = step0 + static_cast<uint64_t>(iters);
 }
 
 struct TsShape {
@@ -753,12 +787,17 @@ TsShape ts_shape(const mhar_ctx* c, const TcPlan* plan) {
   return s;
 }
 
-// Instantiations by (chunks, last-chunk K steps): index 4 (KCH - 1) + LAST - 1.
+// Instantiations by (one iteration, many), then by (chunks, last-chunk K steps): index
+// 4 (KCH - 1) + LAST - 1.
 using TsKernel = void (*)(CUtensorMap, CUtensorMap, TsParams);
-constexpr TsKernel kTsKernels[8] = {
-    recompute_ts_kernel<1, 1>, recompute_ts_kernel<1, 2>, recompute_ts_kernel<1, 3>,
-    recompute_ts_kernel<1, 4>, recompute_ts_kernel<2, 1>, recompute_ts_kernel<2, 2>,
-    recompute_ts_kernel<2, 3>, recompute_ts_kernel<2, 4>};
+template <bool RUN>
+constexpr std::array<TsKernel, 8> ts_kernels() {
+  return {recompute_ts_kernel<1, 1, RUN>, recompute_ts_kernel<1, 2, RUN>,
+          recompute_ts_kernel<1, 3, RUN>, recompute_ts_kernel<1, 4, RUN>,
+          recompute_ts_kernel<2, 1, RUN>, recompute_ts_kernel<2, 2, RUN>,
+          recompute_ts_kernel<2, 3, RUN>, recompute_ts_kernel<2, 4, RUN>};
+}
+constexpr std::array<TsKernel, 8> kTsKernels[2] = {ts_kernels<false>(), ts_kernels<true>()};
 
 }  // namespace
 
@@ -772,9 +811,10 @@ int ts_prepare(mhar_ctx* c) {
     return MHAR_E_CUDA;
   }
   cudaError_t e = cudaSuccess;
-  for (TsKernel k : kTsKernels)
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  for (const auto& form : kTsKernels)
+    for (TsKernel k : form)
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                static_cast<int>(kSmemTs));
   if (e != cudaSuccess) {
     snprintf(c->err, sizeof(c->err), "recompute (TMEM operand) kernel attributes: %s",
@@ -835,7 +875,7 @@ cudaError_t launch_ts(mhar_ctx* c, int j, const SmallRun* r) {
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.C, plan->strips, 1);
-  cfg.blockDim = dim3(kThreadsTs, 1, 1);
+  cfg.blockDim = dim3(r ? kThreadsTs : kThreadsOne, 1, 1);
   cfg.dynamicSmemBytes = kSmemTs;
   cfg.stream = c->stream;
   cudaLaunchAttribute attr[2];
@@ -849,7 +889,7 @@ cudaError_t launch_ts(mhar_ctx* c, int j, const SmallRun* r) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const TsKernel k = kTsKernels[4 * (p.k_chunks - 1) + last_chunk_steps(p.kdim, p.k_chunks) - 1];
+  const TsKernel k = kTsKernels[r ? 1 : 0][4 * (p.k_chunks - 1) + last_chunk_steps(p.kdim, p.k_chunks) - 1];
   return cudaLaunchKernelEx(&cfg, k, plan->ah64, plan->al64, p);
 }
 
