@@ -62,6 +62,7 @@ constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kDrawWarp = 2 + kEpiWarps;
 constexpr int kDrawThreads = 64;
 constexpr int kThreadsTc = kDrawWarp * 32 + kDrawThreads;
+constexpr int kThreadsOne = kDrawWarp * 32;           // a single iteration draws nothing
 constexpr int kMaxClusterTc = 16;
 static_assert(kStagesRes * 2 * kOperandBytes + 4 * kOperandBytes <= kStages * kStageBytes,
               "the resident layout fits the streamed one's space");
@@ -205,7 +206,13 @@ __device__ __forceinline__ void four_products(uint32_t d, uint64_t wh, uint64_t 
   }
 }
 
-__global__ void __launch_bounds__(kThreadsTc, 1)
+// RUN: many iterations, and the draws; else a refresh, or one iteration whose directions a
+// kernel before it drew (equalities, a preconditioner), without what only the loop needs and
+// without its two cluster barriers: with an equality 16.6 -> 14.9 us on 2 walkers of a
+// 60 x 5 body, 36.8 -> 35.6 on 4096 of a 2000 x 100 body.  (The loop's form keeps the
+// refresh's branch: compiled out, 64 iterations of rand100x2000 took 0.6 % longer.)
+template <bool RUN>
+__global__ void __launch_bounds__(RUN ? kThreadsTc : kThreadsOne, 1)
 walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
                  const __grid_constant__ CUtensorMap tm_wh, const __grid_constant__ CUtensorMap tm_wl,
                  const __grid_constant__ CUtensorMap tm_wh2, const __grid_constant__ CUtensorMap tm_wl2,
@@ -260,7 +267,12 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
   }
   tc_fence_before();
   __syncwarp();
-  cluster_sync_all();        // every CTA's barriers are ready
+  if constexpr (RUN) {
+    cluster_sync_all();      // every CTA's barriers are ready
+  } else {
+    cluster_arrive();        // waited for before the first message to one of them
+    __syncthreads();
+  }
   tc_fence_after();
   const uint32_t tmem = tail->tmem_base;
   volatile int* timed_out = &tail->timed_out;
@@ -272,10 +284,11 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
   const int w_begin = static_cast<int>(rank) * share;
   const int w_count = max(0, min(share, kWalkers - w_begin));
   const int chunks = (p.n + 7) >> 3;
-  const int draw_all = p.wt.draw && !refresh ? w_count * chunks : 0;
+  const int draw_all = RUN && p.wt.draw && !refresh ? w_count * chunks : 0;
+  const int iters = RUN ? p.iters : 1;
   int a_it = 0, m_it = 0;
 #pragma unroll 1
-  for (int it = 0; it < p.iters; ++it) {
+  for (int it = 0; it < iters; ++it) {
     const uint64_t step = step0 + static_cast<uint64_t>(it);
     const int cur = static_cast<int>(step & 1ull);
     // Updates of the tracked slack since the last refresh.
@@ -298,7 +311,7 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
           }
         }
         // This iteration's stages; those of A alone also the first of the next.
-        const int end = min(p.iters * per, (it + 1) * per + (resident ? stages : 0));
+        const int end = min(iters * per, (it + 1) * per + (resident ? stages : 0));
         for (; a_it < end; ++a_it) {
           const int s = a_it % stages, nt = (a_it / p.k_chunks) % ntiles, kc = a_it % p.k_chunks;
           if (a_it >= stages) mbar_wait(&tail->empty[s], ((a_it / stages) - 1) & 1, timed_out, p.err);
@@ -448,6 +461,7 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
       tail->part_lo[cg][wl] = lo;
       tail->part_hi[cg][wl] = hi;
       named_bar<kEpiThreads>();
+      if constexpr (!RUN) cluster_wait();
       if (cg == 0) {
         // This CTA's partial chord to every CTA of the cluster, data and arrival in
         // one message.
@@ -476,7 +490,7 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
                                    u * (static_cast<double>(H) - static_cast<double>(L)));
           }
           if (rank == 0) {
-            if (it + 1 == p.iters) {
+            if (it + 1 == iters) {
               p.lmin[k] = L;
               p.lmax[k] = H;
               p.theta[k] = t;
@@ -521,7 +535,7 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
       const int c0 = static_cast<int>(rank) * slice;
       const int pieces = 2 * max(0, min(chunks, c0 + slice) - c0);
       const int done = p.phase + it + 1;
-      double* const out = p.out != nullptr && done % p.thin == 0
+      double* const out = RUN && p.out != nullptr && done % p.thin == 0
                               ? p.out + static_cast<size_t>(done / p.thin - 1) * p.emit * p.n
                               : nullptr;
 #pragma unroll 2
@@ -576,7 +590,22 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
     // message is under way.
     tc_fence_before();
     __syncwarp();
-    cluster_sync_all();
+    if constexpr (RUN) {
+      cluster_sync_all();
+    } else {
+      // Every message to this CTA has arrived (c_full), and no other reads of it: nothing
+      // to wait for but its own warps.
+      if (warp < 2 || refresh) cluster_wait();
+      __syncthreads();
+      if (*timed_out && !refresh) {
+        // An expired wait: messages may still be on their way.  Until the other CTAs are
+        // here or have ended, and a bounded while for the messages.
+        cluster_sync_all();
+        if (threadIdx.x == 0)
+          for (int i = 0; i < (1 << 14) && !mbar_try_wait(smem_u32(&tail->c_full), 0u); ++i) {}
+        __syncthreads();
+      }
+    }
     tc_fence_after();
   }
   if (warp == 1) {
@@ -585,7 +614,7 @@ walker_tc_kernel(const __grid_constant__ CUtensorMap tm_ah, const __grid_constan
                  : "memory");
   }
   if (p.step_out != nullptr && threadIdx.x == 0 && rank == 0 && strip == 0)
-    *p.step_out = step0 + static_cast<uint64_t>(p.iters);
+    *p.step_out = step0 + static_cast<uint64_t>(iters);
 }
 
 // Refresh operands: each walker's point x = hi + lo scaled by a power of two
@@ -680,7 +709,7 @@ cudaError_t launch_walker_tc(mhar_ctx* c, int mode, int j, bool check_drift, con
   p.draw_items = cycles / 3400 * kDrawThreads;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(plan->C, plan->strips, 1);
-  cfg.blockDim = dim3(kThreadsTc, 1, 1);
+  cfg.blockDim = dim3(r ? kThreadsTc : kThreadsOne, 1, 1);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = c->stream;
   cudaLaunchAttribute attr[1];
@@ -691,10 +720,10 @@ cudaError_t launch_walker_tc(mhar_ctx* c, int mode, int j, bool check_drift, con
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (mode == kModeRefresh)
-    return cudaLaunchKernelEx(&cfg, walker_tc_kernel, plan->ah, plan->al, plan->xh, plan->xl,
+    return cudaLaunchKernelEx(&cfg, walker_tc_kernel<false>, plan->ah, plan->al, plan->xh, plan->xl,
                               plan->xh, plan->xl, p);
   const bool two = c->d.Dh2 != nullptr;      // pairs of even and odd iterations
-  return cudaLaunchKernelEx(&cfg, walker_tc_kernel, plan->ah, plan->al, plan->dh, plan->dl,
+  return cudaLaunchKernelEx(&cfg, r ? walker_tc_kernel<true> : walker_tc_kernel<false>, plan->ah, plan->al, plan->dh, plan->dl,
                             two ? plan->dh2 : plan->dh, two ? plan->dl2 : plan->dl, p);
 }
 
@@ -723,10 +752,14 @@ int tc_plan_create(mhar_ctx* c) {
     snprintf(c->err, sizeof(c->err), "cuTensorMapEncodeTiled failed");
     return MHAR_E_CUDA;
   }
-  cudaError_t e = cudaFuncSetAttribute(walker_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kSmemBytes));
-  if (e == cudaSuccess && plan->C > 8)
-    e = cudaFuncSetAttribute(walker_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaSuccess;
+  for (auto k : {walker_tc_kernel<false>, walker_tc_kernel<true>}) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(kSmemBytes));
+    if (e == cudaSuccess && plan->C > 8)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
   if (e != cudaSuccess) {
     delete plan;
     snprintf(c->err, sizeof(c->err), "tensor-core kernel attributes: %s", cudaGetErrorString(e));
