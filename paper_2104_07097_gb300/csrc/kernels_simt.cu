@@ -517,7 +517,7 @@ draw_precondition_kernel(uint64_t seed, const uint64_t* step_ptr, int j, uint32_
       for (int e = 0; e < 4; ++e) acc[w][e] *= dl[e];
     }
 #pragma unroll 2
-    for (int c = 0; c < kMaxPcRank; c += 4) {
+    for (int c = 0; c < rank; c += 4) {        // g and U are 0 past the rank
       float4 gv[4];
 #pragma unroll
       for (int w = 0; w < 4; ++w) gv[w] = *reinterpret_cast<const float4*>(&g[wg + w][c]);
