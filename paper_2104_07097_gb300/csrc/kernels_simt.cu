@@ -1216,10 +1216,14 @@ check_exact_kernel(int mode, int m, int n, int n_ld, int walkers, int group,
 }
 
 // Both parts in one launch, every (row, walker) in FP64: a block per (128 rows,
-// walker).  Small checks (kCheckScreen products and below; the equalities of
-// the larger ones, with m = 0): about 5 us and 7 us per 2^20 products where the
-// screen's launches take 25 us and hardly grow.
+// walker).  Small checks (kCheckScreen products and below, or kCheckPairs rows times
+// walkers; the equalities of the larger ones, with m = 0).  A call on 50 and more columns
+// goes by the pairs: at 32000 of them 68 us against the screen's 68 (8000 x 50, 4 walkers),
+// 71 / 73 (8000 x 100, 4), 105 / 108 (8000 x 300, 4), 192 / 210 (8000 x 1000, 4), at 64000
+// 104 / 73 (8000 x 100, 8); all values equal, as before a chain's first step, 78 / 355
+// (4000 x 300, 4).  On fewer columns equal values make the screen slow for longer.
 constexpr long long kCheckScreen = 1ll << 22;
+constexpr long long kCheckPairs = 1ll << 15;
 
 __global__ void check_kernel(int mode, int m, int n, int n_ld, int mE, const double* A,
                              const double* b, const double* AE, const double* bE,
@@ -1840,7 +1844,8 @@ cudaError_t launch_set_points(mhar_ctx* c, const double* X_dev) {
 }
 
 bool check_direct(const mhar_ctx* c, int walkers) {
-  return static_cast<long long>(c->m) * c->n * walkers <= kCheckScreen;
+  const long long pairs = static_cast<long long>(c->m) * walkers;
+  return pairs <= kCheckPairs || pairs * c->n <= kCheckScreen;
 }
 
 int check_launches(const mhar_ctx* c, int walkers) {
