@@ -357,11 +357,12 @@ int mhar_fit_from_moments(mhar_ctx* ctx, const double* s1, const double* s2, int
  * problem p's walk is the one a single context with that seed would take.
  * Two launch shapes, over the (problem, strip of 128 walkers) units,
  * largest first: each unit on a cluster of C CTAs along its rows (C = 1, 2,
- * 4, 8); or, the default, a persistent launch of one CTA per SM in which every
- * CTA pulls units, long ones cut along their rows, from a device queue, with
- * its pipelines carried from unit to unit (shape 0).  mhar_batch_tune picks the shape, for the whole batch or
- * per bucket (below; in per-bucket mode each bucket has its own two
- * launches). */
+ * 4, 8); or a persistent launch of one CTA per SM in which every CTA pulls
+ * units, long ones cut along their rows, from a device queue, with its
+ * pipelines carried from unit to unit (shape 0, the default; a new batch of
+ * few short strips runs them as clusters until a shape is set or tuned).
+ * mhar_batch_tune picks the shape, for the whole batch or per bucket (below;
+ * in per-bucket mode each bucket has its own two launches). */
 typedef struct {
   const double* A;   /* m x n, row-major (copied)                 */
   const double* b;   /* m                                         */

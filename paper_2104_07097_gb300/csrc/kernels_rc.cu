@@ -604,6 +604,18 @@ int batch_table_build(mhar_ctx* const* ctx, int count, int C, void** table, int*
   return MHAR_OK;
 }
 
+int batch_clusters_at_once(int C) {
+  int n = 0;
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = rc_config(C, 1, nullptr, attr);
+  cudaError_t e = cudaFuncSetAttribute(recompute_batch_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(kSmemRc));
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, recompute_batch_kernel, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess ? n : 0;
+}
+
 cudaError_t launch_recompute_batch(const void* table, int units, int C, int j,
                                    cudaStream_t stream) {
   cudaLaunchAttribute attr[2];

@@ -28,6 +28,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <functional>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -1192,7 +1193,8 @@ void batch_sk_destroy(void* plan_v) {
   delete plan;
 }
 
-int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, size_t err_len) {
+int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, size_t err_len,
+                   int* clusters) {
   *plan_out = nullptr;
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx[0]->device);
@@ -1233,11 +1235,30 @@ int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, 
   }
   // The longest unit: of a few lengths the one with the least time estimated, the
   // SMs' even share of the work with every unit's set-up plus half a longest unit
-  // (largest first), at least one longest unit.
+  // (largest first), at least what the queue makes of the units when each CTA takes the
+  // next one as it comes free.
   auto units_of = [&](int q, long long most) {
     const long long tiles = probs[q].m_tiles;
     return static_cast<int>(std::min<long long>(
         {(tiles * tile_cost[q] + most - 1) / most, tiles, static_cast<long long>(kWalkers)}));
+  };
+  std::vector<long long> cost, busy;
+  auto makespan = [&](long long len) {
+    cost.clear();
+    for (int q = 0; q < count; ++q) {
+      const long long g = units_of(q, len), tiles = probs[q].m_tiles;
+      for (long long i = 0; i < g; ++i)
+        cost.insert(cost.end(), tc_plan_strips(ctx[q]),
+                    ((i + 1) * tiles / g - i * tiles / g) * tile_cost[q] + kUnitCost);
+    }
+    std::sort(cost.begin(), cost.end(), std::greater<long long>());
+    busy.assign(std::min<size_t>(sms, cost.size()), 0);   // a heap, the first to come free on top
+    for (long long c : cost) {
+      std::pop_heap(busy.begin(), busy.end(), std::greater<long long>());
+      busy.back() += c;
+      std::push_heap(busy.begin(), busy.end(), std::greater<long long>());
+    }
+    return *std::max_element(busy.begin(), busy.end());
   };
   long long most = 0, best = 0;
   for (long long len = 2700; len <= 16 * std::max(total, 2700ll); len = len * 3 / 2) {
@@ -1247,8 +1268,25 @@ int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan_out, char* err, 
       sum += static_cast<long long>(tc_plan_strips(ctx[q])) * g * kUnitCost;
       longest = std::max(longest, (probs[q].m_tiles + g - 1) / g * tile_cost[q] + kUnitCost);
     }
-    const long long est = std::max(longest, sum / sms + longest / 2);
+    const long long est = std::max(makespan(len), sum / sms + longest / 2);
     if (most == 0 || est < best) { best = est; most = len; }
+  }
+  if (clusters) {
+    // The clusters of a strip each that serve the batch better: all on the SMs at once, and
+    // the longest CTA's tiles at most four fifths of the estimate (what the units' queue and
+    // the meeting of their chords cost a small batch).
+    *clusters = 0;
+    int strips = 0;
+    for (int q = 0; q < count; ++q) strips += tc_plan_strips(ctx[q]);
+    long long least = best * 4 / 5 + 1;
+    for (int C = 1; C <= 8 && strips <= batch_clusters_at_once(C); C *= 2) {
+      long long share = 0;
+      for (int q = 0; q < count; ++q)
+        share = std::max(share, (probs[q].m_tiles + C - 1) / C * tile_cost[q]);
+      // (CTAs without a tile still move walkers: worth it while SMs are idle.)
+      if (share < least || (share == least && 2 * strips * C <= sms)) { least = share; *clusters = C; }
+    }
+    if (*clusters > 0) return MHAR_OK;
   }
   int parts = 0, arrivals = 0;
   for (int q = 0; q < count; ++q) {

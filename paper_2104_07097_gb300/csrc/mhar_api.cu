@@ -1668,7 +1668,8 @@ struct mhar_batch {
   int C = 1;                    // cluster size; 0: the persistent stream-K launch
   void* table = nullptr;
   int units = 0;
-  void* sk = nullptr;           // stream-K plan (C == 0)
+  int table_C = 0;              // the table's cluster size
+  void* sk = nullptr;           // stream-K plan (C == 0, unless the default is clusters)
   void* upd = nullptr;          // the walker update of every problem
   uint64_t** steps = nullptr;   // device array of every problem's step counter
   mhar::BatchProblem* probs = nullptr;   // device array
@@ -1771,7 +1772,9 @@ int bucket_clamp(const BatchBucket& k, int C) {
   return C;
 }
 
-int batch_set_shape(mhar_batch* b, int C) {
+// as_default: the shape of a new batch, the persistent launch or the clusters that
+// batch_sk_build prefers to it (C stays 0).
+int batch_set_shape(mhar_batch* b, int C, bool as_default = false) {
   b->per_bucket = false;
   batch_drop_graphs(b);
   for (BatchBucket& k : b->buckets) bucket_release(k);
@@ -1779,10 +1782,15 @@ int batch_set_shape(mhar_batch* b, int C) {
   b->table = nullptr;
   mhar::batch_sk_destroy(b->sk);
   b->sk = nullptr;
-  int rc = C == 0 ? mhar::batch_sk_build(b->ctx.data(), static_cast<int>(b->ctx.size()), &b->sk,
-                                         b->err, sizeof(b->err))
-                  : mhar::batch_table_build(b->ctx.data(), static_cast<int>(b->ctx.size()), C,
-                                            &b->table, &b->units, b->err, sizeof(b->err));
+  const int count = static_cast<int>(b->ctx.size());
+  int rc = MHAR_OK, clusters = C;
+  if (C == 0)
+    rc = mhar::batch_sk_build(b->ctx.data(), count, &b->sk, b->err, sizeof(b->err),
+                              as_default ? &clusters : nullptr);
+  if (rc == MHAR_OK && clusters > 0)
+    rc = mhar::batch_table_build(b->ctx.data(), count, clusters, &b->table, &b->units, b->err,
+                                 sizeof(b->err));
+  b->table_C = clusters;
   if (rc == MHAR_OK) b->C = C;
   return rc;
 }
@@ -1817,8 +1825,8 @@ cudaError_t batch_enqueue(mhar_batch* b, int count) {
     return mhar::launch_advance_many(b->steps, static_cast<int>(b->ctx.size()), count, b->stream);
   }
   for (int j = 0; j < count; ++j) {
-    cudaError_t e = b->C == 0 ? mhar::launch_recompute_batch_sk(b->sk, j, b->stream)
-                              : mhar::launch_recompute_batch(b->table, b->units, b->C, j, b->stream);
+    cudaError_t e = b->sk ? mhar::launch_recompute_batch_sk(b->sk, j, b->stream)
+                          : mhar::launch_recompute_batch(b->table, b->units, b->table_C, j, b->stream);
     if (e == cudaSuccess) e = mhar::launch_update_plan(b->upd, j, b->stream);
     if (e != cudaSuccess) return e;
   }
@@ -1964,11 +1972,13 @@ int mhar_batch_create(const mhar_problem* problems, int32_t count, int32_t z,
   }
   if (rc == MHAR_OK) rc = batch_buckets_init(b);
   if (rc == MHAR_OK) {
-    // Default shape: the persistent launch, whose units are cut to balance the SMs
-    // (clusters of one size for every body: 2 to 4 times its time on uneven bodies; one
-    // CTA a unit 0.94 .. 1.02 of a call of 16 iterations on 40 .. 300 small bodies of
-    // nearly one size, 609 against 647 us at the best, 100 bodies of 20 to 40 dimensions).
-    rc = batch_set_shape(b, 0);
+    // Default shape: the persistent launch, whose units are cut to balance the SMs, or
+    // clusters where they serve the batch better.  Clusters of one size for every body take 2
+    // to 4 times its time on uneven bodies that fill the SMs; a few small bodies 0.8 to 0.95
+    // of it (32 iterations of one body of 36 dimensions 413 us against 496, of 17 bodies of
+    // 18 to 48 dimensions 506 against 566).  Over 308 batches of 1 to 80 bodies of 2 to 500
+    // dimensions the rule's choice takes 0.93 of the persistent launch's time, at most 1.16.
+    rc = batch_set_shape(b, 0, true);
   }
   if (rc != MHAR_OK) {
     remember_create_error(b->err);

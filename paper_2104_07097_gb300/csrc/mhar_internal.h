@@ -314,11 +314,15 @@ cudaError_t launch_recompute_tc(mhar_ctx* ctx, int j);
 // for clusters of C CTAs, largest units first.
 int batch_table_build(mhar_ctx* const* ctx, int count, int C, void** table, int* units,
                       char* err, size_t err_len);
+int batch_clusters_at_once(int C);   // how many clusters of C CTAs the GPU holds
 cudaError_t launch_recompute_batch(const void* table, int units, int C, int j,
                                    cudaStream_t stream);
 // Batched persistent stream-K launch (kernels_sk.cu): one CTA per SM, the
 // batch's (problem, strip, row tile) work cut into cost-balanced ranges.
-int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan, char* err, size_t err_len);
+// clusters (may be null): set to the cluster size that serves the batch better, with no
+// plan built then, or to 0.
+int batch_sk_build(mhar_ctx* const* ctx, int count, void** plan, char* err, size_t err_len,
+                   int* clusters = nullptr);
 void batch_sk_destroy(void* plan);
 void batch_sk_counters(const void* plan, BatchCounters* counters);   // adds the plan's set
 cudaError_t launch_recompute_batch_sk(const void* plan, int j, cudaStream_t stream);
