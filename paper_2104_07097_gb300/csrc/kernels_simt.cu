@@ -1909,7 +1909,10 @@ cudaError_t launch_reproject(mhar_ctx* c) {
 }
 
 cudaError_t launch_prepare_tc_operands(mhar_ctx* c, bool blocks) {
-  prepare_tc_kernel<<<c->m_pad, kThreads, 0, c->stream>>>(
+  // No more threads than columns: the sums' tree over a block is FP64 work, most of it on
+  // zeros for short rows (the same bits without them; 3072 rows of 31 columns 89 -> 39 us).
+  const int block = c->k_pad <= 64 ? 64 : c->k_pad <= 128 ? 128 : kThreads;
+  prepare_tc_kernel<<<c->m_pad, block, 0, c->stream>>>(
       c->m, c->n, c->n_ld, c->m_pad, c->k_pad, mma_per_step(c), c->d.A64, c->d.b64, c->d.Ah,
       c->d.Al, c->d.row_scale, c->d.bS, c->d.rowk, c->d.sigma);
   if (!blocks) return cudaGetLastError();

@@ -97,11 +97,10 @@ bool mixed(const mhar_ctx* c) {
 bool stored(const mhar_ctx* c) { return c->opts.precision == MHAR_MIXED_F16X3; }
 bool recompute(const mhar_ctx* c) { return c->opts.precision == MHAR_MIXED_RECOMPUTE; }
 
-// Gives up the screened chord's operands (pointers into one allocation).
+// Gives up the screened chord's operands (pointers into d.emit's allocation).
 void drop_screen(mhar_ctx* c) {
   mhar::DeviceBuffers& d = c->d;
   if (!d.scr_mem) return;
-  cudaFree(d.scr_mem);
   d.scr_mem = nullptr;
   d.Ah = d.Al = d.Dh = d.Dl = d.Xh = d.Xl = nullptr;
   d.row_scale = d.bS = d.rows = d.rowk = d.scr_walker = d.scr_nrm = nullptr;
@@ -117,7 +116,7 @@ void free_all(mhar_ctx* c) {
                   d.refresh_step, d.X64, d.Xhi, d.Xlo, d.D64, d.D32, d.Dh, d.Dl, d.S, d.corr, d.corrn, d.Xh, d.Xl, d.wscale, d.Dh2, d.Dl2,
                   d.key_lo, d.key_hi, d.lmin, d.lmax, d.theta, d.status, d.counters, d.step,
                   d.emit, d.check, d.pc_delta64, d.pc_U64, d.pc_delta32, d.pc_U32, d.sigma,
-                  d.small_at, c->fit_arena};
+                  c->fit_arena};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   d = mhar::DeviceBuffers();
@@ -896,26 +895,26 @@ void mhar_destroy(mhar_ctx* c) {
   delete c;
 }
 
-// FP64 / FP32 modes: the operands of the screened chord (kernels_screen.cu) or of
-// the small-body kernel (kernels_small.cu).  A body outside their range, or
-// memory that does not hold them, leaves the direct kernels in place.
-static int try_fast_chord(mhar_ctx* c) {
+// FP64 / FP32 modes: bytes of the operands of the screened chord (kernels_screen.cu) or
+// of the small-body kernel (kernels_small.cu), 0 for neither.
+static size_t fast_chord_bytes(mhar_ctx* c) {
+  if (mixed(c)) return 0;
+  if (mhar::small_eligible(c)) return mhar::small_arena(c, nullptr);
+  return mhar::screen_eligible(c) ? mhar::screen_arena(c, nullptr) : 0;
+}
+
+// Their set-up, in `mem` (cleared; null: memory did not hold them).  A body outside
+// their range leaves the direct kernels in place.
+static int try_fast_chord(mhar_ctx* c, uint8_t* mem) {
+  if (!mem) return MHAR_OK;
   const bool small = mhar::small_eligible(c);
-  if (!small && !mhar::screen_eligible(c)) return MHAR_OK;
   mhar::DeviceBuffers& d = c->d;
-  const size_t bytes = small ? mhar::small_arena(c, nullptr) : mhar::screen_arena(c, nullptr);
-  uint8_t* mem = nullptr;
-  if (cudaMalloc(reinterpret_cast<void**>(&mem), bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return MHAR_OK;
-  }
   if (small) {
     mhar::small_arena(c, mem);
   } else {
     d.scr_mem = mem;
     mhar::screen_arena(c, mem);
   }
-  MHAR_CUDA(cudaMemsetAsync(mem, 0, bytes, c->stream), "operand memset");
   int outside = 0;
   MHAR_CUDA(small ? mhar::small_prepare(c, d.status + 1) : mhar::screen_prepare(c, d.status + 1),
             "operand preparation kernels");
@@ -925,7 +924,6 @@ static int try_fast_chord(mhar_ctx* c) {
   MHAR_CUDA(cudaStreamSynchronize(c->stream), "sync");
   if (outside) {
     if (small) {
-      cudaFree(d.small_at);
       d.small_at = nullptr;
       d.small_an = nullptr;
     } else {
@@ -1052,8 +1050,18 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
       (rc = dmalloc(c, &d.lmin, z)) || (rc = dmalloc(c, &d.lmax, z)) ||
       (rc = dmalloc(c, &d.theta, z)) || (rc = dmalloc(c, &d.status, 4)) ||
       (rc = dmalloc(c, &d.counters, 2)) || (rc = dmalloc(c, &d.step, 1)) ||
-      (rc = dmalloc(c, &d.emit, static_cast<size_t>(c->emit_cap))) || (rc = dmalloc(c, &d.check, 6)))
+      (rc = dmalloc(c, &d.check, 6)))
     return rc;
+  // The fast chord's operands behind the samples' staging buffer: an allocation of their
+  // own took 50 to 65 us, and as much to free.
+  const size_t staged = (static_cast<size_t>(c->emit_cap) + 31) / 32 * 32;
+  const size_t fast = fast_chord_bytes(c);
+  uint8_t* fast_mem = nullptr;
+  if (fast > 0 && dmalloc(c, &d.emit, staged + (fast + sizeof(double) - 1) / sizeof(double)) == MHAR_OK)
+    fast_mem = reinterpret_cast<uint8_t*>(d.emit + staged);
+  else if ((rc = dmalloc(c, &d.emit, staged)))
+    return rc;
+  c->err[0] = '\0';   // memory that holds the samples alone is no error
   {
     // Audit keys: running max violation from -inf, running residual from 0.
     const unsigned long long init[2] = {host_key(-INFINITY), host_key(0.0)};
@@ -1155,7 +1163,7 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
       if (rc) return rc;
     }
     if (stored(c) && ((rc = reset_drift(c)) || (rc = refresh(c)))) return rc;
-  } else if ((rc = try_fast_chord(c))) {
+  } else if ((rc = try_fast_chord(c, fast_mem))) {
     return rc;
   }
   MHAR_CUDA(cudaStreamSynchronize(c->stream), "create sync");

@@ -70,7 +70,7 @@ struct DeviceBuffers {
   // FP64 / FP32 modes, screened chord (kernels_screen.cu): the walkers' bound
   // factors, the FP32 mode's margin norms, range flags and scale exponents, and
   // the bounds each epilogue thread kept.
-  // One allocation, scr_mem, holds these and the FP16 operands above.
+  // scr_mem, behind the samples in emit's allocation, holds these and the FP16 operands above.
   uint8_t* scr_mem = nullptr;
   float* scr_walker = nullptr;   // 4 z
   float* scr_nrm = nullptr;      // 4 z (FP32 mode)
@@ -79,7 +79,7 @@ struct DeviceBuffers {
   unsigned int* scr_tiles = nullptr;  // streams x z_ld
 
   // Small bodies in one launch (kernels_small.cu): A by columns, gamma ||a_i||_2.
-  uint8_t* small_at = nullptr;   // one allocation
+  uint8_t* small_at = nullptr;   // behind the samples in emit's allocation
   float* small_an = nullptr;     // inside it
 
   // Chord bookkeeping.
