@@ -116,12 +116,11 @@ void free_all(mhar_ctx* c) {
                   d.refresh_step, d.X64, d.Xhi, d.Xlo, d.D64, d.D32, d.Dh, d.Dl, d.S, d.corr, d.corrn, d.Xh, d.Xl, d.wscale, d.Dh2, d.Dl2,
                   d.key_lo, d.key_hi, d.lmin, d.lmax, d.theta, d.status, d.counters, d.step,
                   d.emit, d.check, d.pc_delta64, d.pc_U64, d.pc_delta32, d.pc_U32, d.sigma,
-                  c->fit_arena, c->stage};
+                  c->fit_arena};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   d = mhar::DeviceBuffers();
   c->fit_arena = nullptr;
-  c->stage = nullptr;
 }
 
 // Projector set-up on the device (Section 3.2).  With L the Cholesky factor
@@ -1041,12 +1040,12 @@ static int create_impl(mhar_ctx* c, const double* A, const double* b, const doub
     MHAR_CUDA(cudaStreamSynchronize(c->stream), "sync");
   }
 
-  // Walker state and bookkeeping.  The buffer of samples holds up to sixteen for the host,
-  // 512 KB (sample_stage has more: with 4 MB here creation took 100 us and more longer).
+  // Walker state and bookkeeping.  The staging buffer of host samples holds
+  // sixteen of them, up to 4 MB.
   c->emit_cap = static_cast<int64_t>(z) * n;
   if (!c->opts.out_on_device)
     c->emit_cap = std::max(c->emit_cap,
-                           std::min<int64_t>(16ll * emit_count(c) * n, (512ll << 10) / 8));
+                           std::min<int64_t>(16ll * emit_count(c) * n, (4ll << 20) / 8));
   if ((rc = dmalloc(c, &d.key_lo, z)) || (rc = dmalloc(c, &d.key_hi, z)) ||
       (rc = dmalloc(c, &d.lmin, z)) || (rc = dmalloc(c, &d.lmax, z)) ||
       (rc = dmalloc(c, &d.theta, z)) || (rc = dmalloc(c, &d.status, 4)) ||
@@ -1213,29 +1212,6 @@ int mhar_create(const double* A, const double* b, int m, int n, const double* AE
   return MHAR_OK;
 }
 
-// Where a kernel that runs many iterations leaves samples for the host, and how many at a
-// time: as many as d.emit holds, or up to sixteen, 4 MB, in a buffer that the first call
-// with more than that allocates (100 us).
-static double* sample_stage(mhar_ctx* c, int64_t samples, int64_t sample, int64_t* held) {
-  int64_t cap = c->emit_cap;
-  double* at = c->d.emit;
-  const int64_t want = std::min<int64_t>(16 * sample, (4ll << 20) / 8);
-  if (!c->stage && samples * sample > cap && want > cap) {
-    if (cudaMalloc(reinterpret_cast<void**>(&c->stage), sizeof(double) * want) == cudaSuccess) {
-      c->stage_cap = want;
-    } else {
-      cudaGetLastError();
-      c->stage = nullptr;
-    }
-  }
-  if (c->stage && samples * sample > cap) {
-    at = c->stage;
-    cap = c->stage_cap;
-  }
-  *held = std::max<int64_t>(1, std::min(samples, cap / sample));
-  return at;
-}
-
 int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
   if (!c) return MHAR_E_ARG;
   if (steps < 0 || thin < 0) {
@@ -1265,8 +1241,7 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
     const bool fused = loops(c) && nsamp > 0;
     const bool whole = fused && c->opts.out_on_device;
     const int64_t sample = static_cast<int64_t>(emit_count(c)) * c->n;
-    int64_t held = 1;
-    double* const stage = fused && !whole ? sample_stage(c, nsamp, sample, &held) : nullptr;
+    const int64_t held = fused ? std::max<int64_t>(1, std::min(nsamp, c->emit_cap / sample)) : 1;
     if (thin > 0 && !whole) adv = std::min<int64_t>(adv, held * thin - done % thin);
     const int64_t before = done;
     if (k > 0) adv = std::min<int64_t>(adv, k - c->since_refresh);
@@ -1274,7 +1249,7 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
     if (loops(c)) {
       double* to = !fused ? nullptr : whole
                        ? out + static_cast<size_t>(done / thin) * emit_count(c) * c->n
-                       : stage;
+                       : c->d.emit;
       rc = advance_loop(c, adv, to, thin, fused ? done % thin : 0);
     } else {
       rc = advance(c, adv);
@@ -1286,7 +1261,7 @@ int mhar_run(mhar_ctx* c, int64_t steps, int64_t thin, double* out) {
     if (c->use_screen && (rc = screen_look(c, adv))) return rc;
     // Out of the staging buffer before the audit takes it as its scratch.
     if (fused && !whole && done / thin > before / thin)
-      MHAR_CUDA(cudaMemcpyAsync(out + static_cast<size_t>(before / thin) * sample, stage,
+      MHAR_CUDA(cudaMemcpyAsync(out + static_cast<size_t>(before / thin) * sample, c->d.emit,
                                 sizeof(double) * static_cast<size_t>(done / thin - before / thin) * sample,
                                 cudaMemcpyDeviceToHost, c->stream),
                 "sample copy");

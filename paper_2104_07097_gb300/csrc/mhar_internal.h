@@ -136,8 +136,6 @@ struct mhar_ctx {
   bool use_sk = false;         // recompute mode: stream-K schedule (kernels_sk.cu)
   void* sk = nullptr;          // its segment table
   int64_t emit_cap = 0;        // doubles that d.emit holds
-  double* stage = nullptr;     // more room for samples on their way to the host
-  int64_t stage_cap = 0;       // doubles that it holds
   void* fit_arena = nullptr;   // a preconditioner fit's workspace, kept between fits
   bool use_small = false;      // FP64 / FP32 modes: all iterations of a call in one launch
   bool use_screen = false;     // FP64 / FP32 modes: screened chord (kernels_screen.cu)
