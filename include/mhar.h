@@ -446,8 +446,8 @@ void mhar_batch_destroy(mhar_batch* batch);
 
 /* Name of the kernel that runs the chord of the next iteration on this context
  * (e.g. "recompute_ts_kernel"); never NULL.  In the FP64 / FP32 modes it follows
- * the walkers: while many lie outside the range of the screened chord, the direct
- * kernels run, with the same results. */
+ * the walkers: while the screened chord would be the slower (walkers outside its
+ * range, very many rows that tie) the direct kernels run, with the same results. */
 const char* mhar_kernel_name(const mhar_ctx* ctx);
 
 /* Human-readable description of the last error on ctx (never NULL); with

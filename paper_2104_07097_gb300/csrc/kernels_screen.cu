@@ -467,7 +467,7 @@ struct FinParams {
   double* theta;
   int* status;
   unsigned long long* slow;  // screen_slow
-  int slow_at;               // walkers of a warp outside the range
+  unsigned int slow_clocks;  // of a block: more, and the direct kernels take less time
   unsigned long long* counters;
   double* X64;
   float* Xhi;
@@ -670,6 +670,8 @@ screen_finish_kernel(const FinParams<T> p) {
   __shared__ int list[kFinList];
   __shared__ int listed;
   extern __shared__ __align__(16) uint8_t fin_smem[];       // kFinStages steps a warp
+  __shared__ unsigned int started;
+  if (threadIdx.x == 0) started = static_cast<unsigned int>(clock());
   const int lane = threadIdx.x & 31;
   const int wl = threadIdx.x >> 2, t4 = threadIdx.x & 3;
   const int side = t4 >> 1, which = t4 & 1;
@@ -766,8 +768,6 @@ screen_finish_kernel(const FinParams<T> p) {
   lam = fmin(lam, __longlong_as_double(static_cast<long long>(again_s[threadIdx.x >> 1])));
   // Walkers outside the screen's range: every row, one walker after the other.
   unsigned int forced = __ballot_sync(0xffffffffu, force && t4 == 0);
-  if (lane == 0 && __popc(forced) >= p.slow_at)
-    atomicMax(p.slow, static_cast<unsigned long long>(*p.step_ptr + static_cast<uint64_t>(p.j) + 1ull));
   while (forced) {
     const int src = __ffs(forced) - 1;
     forced &= forced - 1;
@@ -876,6 +876,8 @@ screen_finish_kernel(const FinParams<T> p) {
       }
     }
   }
+  if (threadIdx.x == 0 && static_cast<unsigned int>(clock()) - started > p.slow_clocks)
+    atomicMax(p.slow, static_cast<unsigned long long>(*p.step_ptr + static_cast<uint64_t>(p.j) + 1ull));
 }
 
 // CTAs along the rows: up to what the SMs leave for each walker strip, the number with
@@ -898,6 +900,33 @@ int screen_tiles_per_cta(const mhar_ctx* c) {
     if (best == 0 || est < best) { best = est; per = t; }
   }
   return per;
+}
+
+// The direct kernels' time, in clocks of a block of the finish: one that takes longer makes
+// the iteration slower than they are.  Walkers outside the screen's range do, one after
+// the other (an FP64 iteration of 4096 walkers of a 2000 x 100 body with 1, 2, 3, 4 of a
+// warp's eight outside 1180, 2290, 3400, 4510 us, direct 4160; FP32 with one 535, 239), and
+// bodies of very many rows that tie within the bounds: 4000 rows in one dimension, 3000
+// walkers, FP32 4495 us (direct 129), 8800 rows about a circle, 300 walkers, 267 (40).
+// Tiles of 64 rows x 64 walkers: in FP64 31 + 2.16 n_ld us a tile and SM, two tiles at
+// least (203 us at 160 tiles, n_ld = 32, 2673 at 4032; 601 and 7984 at n_ld = 128), in
+// FP32 2.6 + 0.116 n_ld and 6 (20, 173; 42, 446).  A warp a walker: 0.125 us for a column
+// of 32 rows (570 us for 100 x 1500, 50 for 64 x 128).
+unsigned int screen_slow_clocks(const mhar_ctx* c) {
+  int sms = 148;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  double us;
+  if (simt_warp_path(c)) {
+    us = 8.0 + 0.125 * c->n * ((c->m + 31) / 32) * std::max(1.0, c->z / 600.0);
+  } else {
+    const double tiles = static_cast<double>((c->m + 63) / 64) * ((c->z + 63) / 64) / sms;
+    us = c->opts.precision == MHAR_FP64
+             ? (31.0 + 2.16 * c->n_ld) * std::max(2.0, tiles)
+             : (2.6 + 0.116 * c->n_ld) * std::max(2.0, tiles) + 6.0;
+  }
+  const int blocks = (c->z + kFinWalkers - 1) / kFinWalkers;
+  const int waves = (blocks + 3 * sms - 1) / (3 * sms);      // three blocks on an SM
+  return static_cast<unsigned int>(std::min(us * 1900.0 / waves, 4.0e9));
 }
 
 template <typename T>
@@ -954,13 +983,8 @@ cudaError_t launch_screen_t(mhar_ctx* c, int j, const T* A, const T* b, const T*
   f.lmin = d.lmin; f.lmax = d.lmax; f.theta = d.theta; f.status = d.status; f.counters = d.counters;
   f.X64 = d.X64; f.Xhi = d.Xhi; f.Xlo = d.Xlo; f.Q32 = d.Q32;
   f.corr = sizeof(T) == 4 ? d.corr : nullptr;
-  // From so many walkers of the eight of a warp on, the direct kernels take less time: an
-  // iteration with 1, 2, 3, 4 of them 1180, 2290, 3400, 4510 us for 4096 walkers of a 2000 x
-  // 100 body in FP64 (direct 4160), 162, 294, 427, 561 for 3001 of a 700 x 20 body (410);
-  // FP32 with one 535 (239) and 82 (35); with a warp a walker, 20 of a 1500 x 100 body, one
-  // 808 (570).
   f.slow = screen_slow(d);
-  f.slow_at = sizeof(T) == 8 && !simt_warp_path(c) ? 3 : 1;
+  f.slow_clocks = screen_slow_clocks(c);
   screen_finish_kernel<T>
       <<<(c->z + kFinWalkers - 1) / kFinWalkers, kFinThreads, kFinSmem, c->stream>>>(f);
   return cudaGetLastError();

@@ -394,9 +394,10 @@ void drop_graphs(mhar_ctx* c) {
 }
 
 // Screened contexts.  Walkers whose coordinates or directions lie outside the screen's
-// range have all their rows evaluated one walker after the other, up to 16 times the time
-// of the direct kernels when it is all of them (bodies of size 1e-17, say).  The finish
-// notes the last iteration in which that was slower (screen_slow).  The host looks after
+// range (bodies of size 1e-17, say) have all their rows evaluated one walker after the
+// other, and bodies of very many rows that tie have most: up to 35 times the time of the
+// direct kernels.  The finish notes the last iteration slower than they are
+// (screen_slow_clocks, kernels_screen.cu).  The host looks after
 // the first kScreenFirst iterations from a new state, then every kScreenLook and at the
 // end of each call, and goes over to the direct kernels -- the same bits -- for 4, 16, 64
 // .. 1024 iterations, with a screened one as a trial between the stretches.  A look takes

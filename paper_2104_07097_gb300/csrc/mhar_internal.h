@@ -15,7 +15,7 @@ constexpr int kTcM = 128;        // rows of A per MMA tile (TMEM lanes)
 constexpr int kTcKChunk = 64;    // FP16 elements per 128-byte swizzled row chunk
 constexpr int kTcK = 16;         // K of one kind::f16 MMA
 // Screened iterations from a new state before the host first looks how they went.
-constexpr int kScreenFirst = 32;
+constexpr int kScreenFirst = 16;
 
 struct DeviceBuffers {
   // Problem (row-major, zero padded to the leading dimensions below).
@@ -139,8 +139,8 @@ struct mhar_ctx {
   void* fit_arena = nullptr;   // a preconditioner fit's workspace, kept between fits
   bool use_small = false;      // FP64 / FP32 modes: all iterations of a call in one launch
   bool use_screen = false;     // FP64 / FP32 modes: screened chord (kernels_screen.cu)
-  // While many walkers lie outside the screen's range: iterations left to take with the
-  // direct kernels, the length of that stretch; else iterations until the host looks.
+  // While the screen is slower than the direct kernels: iterations left to take with them,
+  // the length of that stretch; else iterations until the host looks.
   int64_t direct_left = 0, direct_len = 0, screen_left = mhar::kScreenFirst;
   bool graphs_direct = false;  // the captured graphs launch the direct kernels
   int pc_rank = -1;            // -1: isotropic directions; else rank of U (0..32)
@@ -213,8 +213,8 @@ cudaError_t launch_draw_precondition(mhar_ctx* ctx, int j, int split);
 
 // ---- FP64 / FP32 modes, screened on the tensor cores (kernels_screen.cu) -------
 bool screen_eligible(const mhar_ctx* ctx);    // by its sizes
-// The device word that holds the last iteration (its number + 1) in which walkers outside
-// the screen's range made it slower than the direct kernels; behind the status words.
+// The device word that holds the last iteration (its number + 1) that took longer than the
+// direct kernels take (screen_slow_clocks); behind the status words.
 inline unsigned long long* screen_slow(const DeviceBuffers& d) {
   return reinterpret_cast<unsigned long long*>(d.status + 2);
 }

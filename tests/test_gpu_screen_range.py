@@ -1,6 +1,6 @@
-"""Screened contexts whose walkers leave the range that the screen covers go over to the
-direct kernels, and back when they return: always the bits of the direct kernels (which an
-all-zero row 0 . x <= 2^60 keeps a context on)."""
+"""Screened contexts that would be slower than the direct kernels (walkers outside the range
+that the screen covers, very many rows that tie) go over to those, and back: always the bits
+of the direct kernels (which an all-zero row 0 . x <= 2^60 keeps a context on)."""
 import numpy as np
 import pytest
 
@@ -90,3 +90,16 @@ def test_returns(precision, direct, eq):
     q.run(4)
     assert q.run(1) == "screen_kernel"   # the trial after four
     assert q.run(30, 6) == "screen_kernel"
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,m,z", [(1, 4000, 3000), (2, 8800, 300)])
+def test_rows_that_tie(precision, n, m, z):
+    """An interval's ends 2000 times over, 8800 tangents of a circle."""
+    p = wl.random_polytope(n, m, seed=5, check_bounded=False)
+    q = Pair(p, z, precision, "chord_simt_kernel")
+    q.run(3, 1)
+    for steps, thin in ((1, 1), (2, 1), (30, 10)):
+        q.run(steps, thin)
+    if n == 1:                # twice the direct kernels' time and more in FP64 too
+        assert q.s.kernel_name() == "chord_simt_kernel"
