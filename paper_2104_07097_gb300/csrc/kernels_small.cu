@@ -27,7 +27,6 @@
 // 64 x 500, 100 walkers 9.8 (137); 100 x 390, 20 walkers 13.3 (164); FP32 2.3,
 // 9.1, 4.1, 4.5 and 5.9 us.  What is left is latency: the serial FP64 sums and
 // division, and four barriers of the block (six screened).
-#include <cfloat>
 #include <cmath>
 #include <cuda_fp16.h>
 #include <type_traits>
@@ -186,6 +185,7 @@ small_kernel(const SmallParams<T> p, int G, int R) {
   const int n = p.n, m = p.m;
   const uint64_t step0 = p.step0;
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
+  const float kNoBound = __int_as_float(0x7fffffff);
 
   if constexpr (sizeof(T) == 8) prefetch_normals_f64(tid);
   {
@@ -386,14 +386,15 @@ small_kernel(const SmallParams<T> p, int G, int R) {
             const float s = fmaxf(bf - ax[q] - fmaf(ga, nx, 0x1p-22f * fabsf(bf)), 0.0f) *
                             (1.0f - 0x1p-20f);
             const float dh = fmaf(ga, nd, ad[q]), dl = fmaf(ga, nd, -ad[q]);
-            // A quotient past FP32's range (short directions) is still a row's.
-            const float bh = dh > 0.0f ? fminf(s * rcp_approx(dh), FLT_MAX) : INFINITY;
-            const float bl = dl > 0.0f ? fminf(s * rcp_approx(dl), FLT_MAX) : INFINITY;
+            // NaN: not on that side.  (+Inf is a quotient past FP32's range, from short
+            // directions, and a row's like any other.)
+            const float bh = dh > 0.0f ? s * rcp_approx(dh) : kNoBound;
+            const float bl = dl > 0.0f ? s * rcp_approx(dl) : kNoBound;
             lbs[(2 * g) * m + r] = bh;
             lbs[(2 * g + 1) * m + r] = bl;
-            if (bh < INFINITY)
+            if (dh > 0.0f)
               kh = min(kh, (static_cast<unsigned long long>(__float_as_uint(bh)) << 32) | r);
-            if (bl < INFINITY)
+            if (dl > 0.0f)
               kl = min(kl, (static_cast<unsigned long long>(__float_as_uint(bl)) << 32) | r);
           }
         }
@@ -446,7 +447,7 @@ small_kernel(const SmallParams<T> p, int G, int R) {
           bool take = force;
           if (!force) {
             const float qh = lbs[(2 * g) * m + r], ql = lbs[(2 * g + 1) * m + r];
-            take = (qh <= fh && qh < INFINITY && r != rh) || (ql <= fl && ql < INFINITY && r != rl);
+            take = (qh <= fh && r != rh) || (ql <= fl && r != rl);
           }
           if (take) {
             const T* a = p.A + static_cast<size_t>(r) * p.n_ld;
