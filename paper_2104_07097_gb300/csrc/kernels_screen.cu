@@ -32,8 +32,9 @@
 // kernels.  Rows that tie within the bounds (duplicate rows, walkers on a
 // facet) cost more evaluations, never a different result.  Values the bounds
 // do not cover (outside 2^-50 .. 2^50) take the direct formulas: a body at
-// creation, a walker by its flag (`force`), a context whose walkers are mostly such ones
-// by the host (screen_look, mhar_api.cu).
+// creation, a walker by its flag (`force`).  An iteration that takes longer than the direct
+// kernels take sends its context to them for a while (screen_slow_clocks here, screen_look
+// in mhar_api.cu).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
