@@ -220,7 +220,8 @@ __device__ double block_sum(double v, double* red) {
 // 2^+-511 stay in range (Q has the same bits); expo: the largest biased exponent of
 // Sigma's diagonal.
 __device__ __forceinline__ double orth_scale(const int* expo) {
-  return ldexp(1.0, -max(-1000, min(1000, *expo - 1022)));
+  const int k = max(-1000, min(1000, __ldg(expo) - 1022));
+  return __hiloint2double((1023 - k) << 20, 0);              // 2^-k
 }
 
 // Q = orth(Y) for the first `rank` columns (zero beyond): classical
